@@ -76,69 +76,62 @@ const Ops* pick_ops(int D, int store) {
     return nullptr;
 }
 
-// Compensated FP64 sum over nb partial vectors of `width` values (width <= kMaxWidth).
+// Compensated FP64 sum over nb partial vectors of `width` values (width <= kMaxWidth), each
+// followed by its corrections where stride = 2 width.
+// Warp k of a CTA sums value k: its lanes take the CTA's rows in turn (TwoSum), then a fixed
+// tree over the lanes.  With more than one CTA each writes its (sum, correction) pairs, and the
+// last one to finish (a counter in the auxiliary buffer, zero between launches) adds the pairs in
+// the same way.  The order of every operation is fixed, so the result does not depend on the
+// schedule.  One value per warp and no more CTAs than rows can feed: the FP64 pipe takes a warp
+// instruction every 16 cycles and SM whether or not its lanes are in use, and a thread that summed
+// all the values of its rows took 28 us for 304 partial vectors of five values and 45 us of eleven.
 constexpr int kMaxWidth = 12;   // widest partial vector: step totals 5, statistics kStatsSums
 static_assert(kStatsSums <= kMaxWidth, "finalize width");
-// The sum runs on kFinBlocks CTAs: CTA b takes a contiguous range of the partial vectors,
-// each thread a Neumaier sum of its share, the CTA a fixed pairwise tree of the threads'
-// (sum, compensation) pairs; the last CTA to finish (a counter in the auxiliary buffer,
-// zero between launches) adds the kFinBlocks pairs in order and writes the result.  The
-// order of every operation is fixed, so the result does not depend on the schedule.
-constexpr int kFinBlocks = 32;
-constexpr int kFinThreads = 128;
+constexpr int kFinBlocks = 128;
+constexpr int kFinRows = 256;   // rows per CTA that are worth another CTA
 
-__device__ __forceinline__ void neumaier_add(double& s, double& c, double v) {
-    const double t = s + v;
-    c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
-    s = t;
+__device__ __forceinline__ void warp_dd_sum(double& s, double& c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, s, o);
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+        dd_add(s, c, v);
+    }
 }
 
-__global__ void __launch_bounds__(kFinThreads)
-finalize_kernel(const double* __restrict__ partials, int nb, int width, double* __restrict__ scratch,
-                unsigned* __restrict__ count, double* __restrict__ out) {
-    const int tid = threadIdx.x;
-    double s[kMaxWidth] = {}, c[kMaxWidth] = {};
+__global__ void finalize_kernel(const double* __restrict__ partials, int nb, int width, int stride,
+                                double* __restrict__ scratch, unsigned* __restrict__ count,
+                                double* __restrict__ out) {
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    double s = 0.0, c = 0.0;
     const int chunk = (nb + gridDim.x - 1) / gridDim.x;
     const int j0 = blockIdx.x * chunk, j1 = min(j0 + chunk, nb);
-    for (int j = j0 + tid; j < j1; j += kFinThreads)
-        for (int k = 0; k < width; ++k) neumaier_add(s[k], c[k], partials[(size_t)width * j + k]);
-    __shared__ double rs[kMaxWidth][kFinThreads], rc[kMaxWidth][kFinThreads];
-    for (int k = 0; k < width; ++k) {
-        rs[k][tid] = s[k];
-        rc[k][tid] = c[k];
+    for (int j = j0 + lane; j < j1; j += 32) {
+        dd_add(s, c, partials[(size_t)stride * j + k]);
+        if (stride > width) c += partials[(size_t)stride * j + width + k];
     }
-    __syncthreads();
-    for (int w = kFinThreads / 2; w > 0; w /= 2) {   // pairs (s, c) + (s', c') -> (s + s', c + c' + error)
-        if (tid < w) {
-            for (int k = 0; k < width; ++k) {
-                double a = rs[k][tid], cc = rc[k][tid] + rc[k][tid + w];
-                neumaier_add(a, cc, rs[k][tid + w]);
-                rs[k][tid] = a;
-                rc[k][tid] = cc;
-            }
+    warp_dd_sum(s, c);
+    if (gridDim.x > 1) {
+        if (lane == 0) {
+            scratch[2 * (kMaxWidth * blockIdx.x + k)] = s;
+            scratch[2 * (kMaxWidth * blockIdx.x + k) + 1] = c;
+            __threadfence();   // this CTA's pairs are visible before its arrival is counted
         }
         __syncthreads();
-    }
-    if (tid < width) {
-        scratch[2 * (kMaxWidth * blockIdx.x + tid)] = rs[tid][0];
-        scratch[2 * (kMaxWidth * blockIdx.x + tid) + 1] = rc[tid][0];
-    }
-    __threadfence();   // this CTA's pair is visible before its arrival is counted
-    __syncthreads();
-    __shared__ bool last;
-    if (tid == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (tid < width) {
-        double ss = 0.0, cc = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            neumaier_add(ss, cc, __ldcg(scratch + 2 * (kMaxWidth * b + tid)));
-            cc += __ldcg(scratch + 2 * (kMaxWidth * b + tid) + 1);
+        __shared__ bool last;
+        if (threadIdx.x == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        s = c = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32) {
+            dd_add(s, c, __ldcg(scratch + 2 * (kMaxWidth * b + k)));
+            c += __ldcg(scratch + 2 * (kMaxWidth * b + k) + 1);
         }
-        out[tid] = ss + cc;
+        warp_dd_sum(s, c);
+        if (threadIdx.x == 0) *count = 0u;   // ready for the next launch on this stream
     }
-    if (tid == 0) *count = 0u;   // ready for the next launch on this stream
+    if (lane == 0) out[k] = s + c;
 }
 
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA; }
@@ -244,21 +237,21 @@ int sync_status(elbm_handle* h) {
 // stream: written by the kernel itself when out is page-locked mapped memory, else
 // reduced into the totals slot and copied; finalize_to_host also synchronises and reads
 // the status.
-int finalize_async(elbm_handle* h, const double* partials, int nb, double* out, int width = 5) {
+int finalize_async(elbm_handle* h, const double* partials, int nb, double* out, int width = 5, int stride = 5) {
     double* direct = (double*)mapped_host(out, (size_t)width * sizeof(double));
-    const int grid = nb < kFinBlocks ? (nb > 0 ? nb : 1) : kFinBlocks;
-    finalize_kernel<<<grid, kFinThreads, 0, h->stream>>>(partials, nb, width,
-                                                         (double*)(h->auxp + h->aux.fin_scratch),
-                                                         (unsigned*)(h->auxp + h->aux.fin_count),
-                                                         direct ? direct : totals_ptr(h));
+    const int want = (nb + kFinRows - 1) / kFinRows, grid = want < 1 ? 1 : want < kFinBlocks ? want : kFinBlocks;
+    finalize_kernel<<<grid, 32 * width, 0, h->stream>>>(partials, nb, width, stride,
+                                                        (double*)(h->auxp + h->aux.fin_scratch),
+                                                        (unsigned*)(h->auxp + h->aux.fin_count),
+                                                        direct ? direct : totals_ptr(h));
     ++h->launches;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && !direct)
         e = cudaMemcpyAsync(out, totals_ptr(h), width * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA;
 }
-int finalize_to_host(elbm_handle* h, const double* partials, int nb, double* out, int width = 5) {
-    const int rc = finalize_async(h, partials, nb, out, width);
+int finalize_to_host(elbm_handle* h, const double* partials, int nb, double* out, int width = 5, int stride = 5) {
+    const int rc = finalize_async(h, partials, nb, out, width, stride);
     return rc != ELBM_OK ? rc : sync_status(h);
 }
 
@@ -560,7 +553,7 @@ int elbm_conservation(elbm_handle* h, double out[5]) {
     cudaError_t e = h->ops->conservation(diag_params(h), h->pop[h->cur], query_partials(h), &nb, h->stream,
                                          &h->launches);
     if (e != cudaSuccess) return ELBM_ERR_CUDA;
-    return finalize_to_host(h, query_partials(h), nb, out);
+    return finalize_to_host(h, query_partials(h), nb, out, 5, 10);   // sums and their corrections
 }
 
 int elbm_turbulence_stats(elbm_handle* h, double out[13]) {
@@ -570,7 +563,7 @@ int elbm_turbulence_stats(elbm_handle* h, double out[13]) {
     cudaError_t e = h->ops->stats(diag_params(h), h->pop[h->cur], part, &nb, h->stream, &h->launches);
     if (e != cudaSuccess) return ELBM_ERR_CUDA;
     double sums[kStatsSums];
-    const int rc = finalize_to_host(h, part, nb, sums, kStatsSums);
+    const int rc = finalize_to_host(h, part, nb, sums, kStatsSums, kStatsSums);
     if (rc != ELBM_OK) return rc;
     const double N = (double)h->N;
     const double mrho = sums[0] / N, mT = sums[5] / N;

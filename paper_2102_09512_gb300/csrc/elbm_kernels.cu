@@ -336,58 +336,137 @@ __global__ void fields_kernel(const __grid_constant__ KParams p, const P* __rest
     flag_if(bad, status);
 }
 
-// FP64 totals of the current state: one partial per CTA (grid-stride loop).
-__global__ void totals_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop,
-                              double* __restrict__ partials) {
-    double s[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0};
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < p.N;
-         n += (long long)gridDim.x * blockDim.x) {
-        R f[Q], g[Q];
-        load_local(p, pop, n, f, g);
-        double v[5] = {0, 0, 0, 0, 0};
+// Totals of the current state.  A work unit is a run of kTotThreads x kTotRun pairs of one
+// direction's plane, read as it lies in memory, and CTA b takes units b, b + gridDim.x, ...: the
+// device walks through the planes one after another.  A thread sums its share of F = sum f_i and
+// G = sum g_i, and only at a plane's end turns F into the sums of rho and rho c_i f_i.  That is
+// two additions per pair where a sum over each node's moments takes five or more, each of them
+// compensated.  FP32-arithmetic stores: the sums are three-float ones (Tri2) throughout, so no
+// FP64 instruction runs before a CTA's last warp; as an FP64 sum per node the FP64 pipe bounded
+// it (256^3, FP32: 6.08 ms, now 0.66).  FP64 store: plain sums of kTotRun pairs,
+// compensated from there on.  Each CTA writes five sums and their five corrections.
+constexpr int kTotRun = sizeof(R) == 8 ? 16 : 8;   // pairs in flight per thread
+constexpr int kTotThreads = 256;
+struct TotalsF64 {
+    double F = 0, Fc = 0, G = 0, Gc = 0, s[5] = {}, c[5] = {};
+    __device__ __forceinline__ void pairs(const R* f, const R* g) {
+        double a = 0, b = 0;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const double fi = (double)f[i];
-            v[0] += fi;
-            if (cx_of(i) != 0) v[1] += cx_of(i) * fi;
-            if (cy_of(i) != 0) v[2] += cy_of(i) * fi;
-            if (cz_of<kD>(i) != 0) v[3] += cz_of<kD>(i) * fi;
-            v[4] += (double)g[i];
+        for (int k = 0; k < kTotRun; ++k) {
+            a += f[k];
+            b += g[k];
         }
-        if constexpr (DEV) {   // moment sums of the rest state (no momentum)
-            v[0] += (double)p.rest_rho;
-            v[4] += (double)p.rest_E;
-        }
+        dd_add(F, Fc, a);
+        dd_add(G, Gc, b);
+    }
+    __device__ __forceinline__ void plane_end(int i) {
+        const double cx = cx_of(i), cy = cy_of(i), cz = cz_of<kD>(i);
+        F += Fc;
+        dd_add(s[0], c[0], F);
+        if (cx != 0.0) dd_add(s[1], c[1], cx * F);
+        if (cy != 0.0) dd_add(s[2], c[2], cy * F);
+        if (cz != 0.0) dd_add(s[3], c[3], cz * F);
+        dd_add(s[4], c[4], G + Gc);
+        F = Fc = G = Gc = 0.0;
+    }
+    // this warp's sums and corrections, in its lane 0
+    __device__ __forceinline__ void warp_total(int lane, double* out) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {   // Neumaier
-            const double t = s[k] + v[k];
-            c[k] += fabs(s[k]) >= fabs(v[k]) ? (s[k] - t) + v[k] : (v[k] - t) + s[k];
-            s[k] = t;
+        for (int k = 0; k < 5; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double v = __shfl_xor_sync(0xffffffffu, s[k], o);
+                c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
+                dd_add(s[k], c[k], v);
+            }
+            if (lane == 0) {
+                out[k] = s[k];
+                out[5 + k] = c[k];
+            }
         }
     }
+};
+struct TotalsF32 {
+    Tri2 a, t[3];   // (F, G); (rho, rho E), (rho u_x, rho u_y), (rho u_z, -)
+    __device__ __forceinline__ TotalsF32() {
+        a.zero();
 #pragma unroll
-    for (int k = 0; k < 5; ++k) s[k] += c[k];
-    block_sum5(s, partials + 5 * blockIdx.x);
-}
-
-// Velocity of node n from its f values only (rho and rho u).
-__device__ __forceinline__ void node_velocity(const KParams& p, const P* __restrict__ pop, long long n, R u[3]) {
-    R rho = 0, j[3] = {0, 0, 0};
-    R fs[Q], gs[Q];
-    load_local(p, pop, n, fs, gs);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const R f = fs[i];
-        rho += f;
-        if (cx_of(i)) j[0] += cx_of(i) * f;
-        if (cy_of(i)) j[1] += cy_of(i) * f;
-        if (cz_of<kD>(i)) j[2] += cz_of<kD>(i) * f;
+        for (int k = 0; k < 3; ++k) t[k].zero();
     }
-    if constexpr (DEV) rho += R(p.rest_rho);
-    const R inv = qdiv(R(1), rho);
-    u[0] = j[0] * inv;
-    u[1] = j[1] * inv;
-    u[2] = j[2] * inv;
+    __device__ __forceinline__ void pairs(const R* f, const R* g) {
+#pragma unroll
+        for (int k = 0; k < kTotRun; ++k) a.add(make_float2((float)f[k], (float)g[k]));
+    }
+    __device__ __forceinline__ void plane_end(int i) {
+        t[0].add(a);
+        // c_i F: products with -1, 0 and 1 are exact
+        auto scaled = [&](float kx, float ky) {
+            Tri2 m;
+            m.s = make_float2(a.s.x * kx, a.s.x * ky);
+            m.e1 = make_float2(a.e1.x * kx, a.e1.x * ky);
+            m.e2 = make_float2(a.e2.x * kx, a.e2.x * ky);
+            return m;
+        };
+        t[1].add(scaled((float)cx_of(i), (float)cy_of(i)));
+        if (kD == 3) t[2].add(scaled((float)cz_of<kD>(i), 0.f));
+        a.zero();
+    }
+    __device__ __forceinline__ void warp_total(int lane, double* out) {
+#pragma unroll
+        for (int k = 0; k < kD; ++k) t[k].warp_sum();
+        if (lane == 0) {
+            auto put = [&](int k, float a0, float e1, float e2) {
+                out[k] = (double)a0;
+                out[5 + k] = (double)e1 + (double)e2;
+            };
+            put(0, t[0].s.x, t[0].e1.x, t[0].e2.x);
+            put(4, t[0].s.y, t[0].e1.y, t[0].e2.y);
+            put(1, t[1].s.x, t[1].e1.x, t[1].e2.x);
+            put(2, t[1].s.y, t[1].e1.y, t[1].e2.y);
+            put(3, t[2].s.x, t[2].e1.x, t[2].e2.x);
+        }
+    }
+};
+__global__ void __launch_bounds__(kTotThreads, sizeof(R) == 8 ? 4 : 5)
+totals_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int units) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kWarps = kTotThreads / 32;
+    __shared__ double part[kWarps][10];
+    std::conditional_t<sizeof(R) == 8, TotalsF64, TotalsF32> tot;
+    int last = -1;
+    for (long long u = blockIdx.x; u < (long long)Q * units; u += gridDim.x) {   // `units` per plane
+        const int i = (int)(u / units);
+        if (i != last && last >= 0) tot.plane_end(last);
+        last = i;
+        // the plane that holds direction i (swapped in the even AA layout)
+        const P* __restrict__ b = pop + (size_t)(p.aa == 1 ? Q - 1 - i : i) * (size_t)p.N;
+        const long long n = (u - (long long)i * units) * (kTotThreads * kTotRun) + threadIdx.x;
+        R f[kTotRun], g[kTotRun];
+#pragma unroll
+        for (int k = 0; k < kTotRun; ++k) {
+            const long long m = n + (long long)k * kTotThreads;
+            Cd::dec(m < p.N ? b[m] : Cd::enc(R(0), R(0)), f[k], g[k]);
+        }
+        tot.pairs(f, g);
+    }
+    if (last >= 0) tot.plane_end(last);
+    tot.warp_total(lane, part[warp]);
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        const int k = threadIdx.x;
+        double a = 0.0, e = 0.0;
+        for (int w = 0; w < kWarps; ++w) {
+            dd_add(a, e, part[w][k]);
+            e += part[w][5 + k];
+        }
+        if (DEV && blockIdx.x == 0 && (k == 0 || k == 4)) {   // N times the rest state's sums (no momentum)
+            const double r = k == 0 ? (double)p.rest_rho : (double)p.rest_E, n = (double)p.N, v = r * n;
+            dd_add(a, e, v);
+            e += fma(r, n, -v);
+        }
+        partials[10 * blockIdx.x + k] = a;
+        partials[10 * blockIdx.x + 5 + k] = e;
+    }
 }
 
 // Turbulence statistics of the current state (one FP64 partial vector per CTA):
@@ -395,63 +474,177 @@ __device__ __forceinline__ void node_velocity(const KParams& p, const P* __restr
 // and mu(T) |omega|^2, with the velocity gradient by second-order central differences
 // (boundary nodes use the ghost values of the boundary map): dilatation
 // theta = div u, vorticity omega = curl u, mu = mu0 (T/T0)^mu_exp (Eq. mu law).
+//
+// A CTA marches a 32 x 8 column over tz planes: each plane's velocities (tile and halo ring)
+// go through shared memory, those of the planes below and above stay in registers, so the
+// store is read once and a node's moments are computed 1.3 times (from seven reads and seven
+// evaluations, 256^3 FP32 6.1 ms).  For the FP32-arithmetic stores the sums and their terms
+// are unevaluated sums of floats: differences and products of FP32 values are exact as two
+// floats, the viscosity law comes from pow_pos_df and the sums are Tri2 ones.  (With the law in
+// FP64 that pipe bounded the kernel: 256^3 FP32 1.48 ms, without 0.79.)
 constexpr int kStats = kStatsSums;
-__global__ void stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop,
-                             double* __restrict__ partials) {
-    double acc[kStats] = {};
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < p.N;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % p.nx), y = (int)((n / p.nx) % p.ny), z = (int)(n / ((long long)p.nx * p.ny));
+template <int DD>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
+stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int tz) {
+    constexpr int TX = 32, TY = 8, NT = TX * TY;
+    __shared__ R us[2][DD][TY + 2][TX + 2];
+    __shared__ double part[NT / 32][kStats];
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int zb = blockIdx.z * tz, ze = min(zb + tz, p.nz);
+    const int x = x0 + tx, y = y0 + ty;
+    const bool active = x < p.nx && y < p.ny;
+    const int xl = min(x0 + TX, p.nx) - 1 - x0, yl = min(y0 + TY, p.ny) - 1 - y0;
+    // halo ring: rows below and above, columns left and right; (hr, hc) its place in `us`
+    int hx = 0, hy = 0, hr = 0, hc = 0;
+    bool halo = false;
+    if (tid < 2 * TX) {
+        const int side = tid / TX;
+        hc = tx + 1, hr = side ? yl + 2 : 0;
+        hx = x, hy = map_axis(side ? y0 + yl + 1 : y0 - 1, p.ny, p.per_y);
+        halo = tx <= xl;
+    } else if (tid < 2 * TX + 2 * TY) {
+        const int side = (tid - 2 * TX) / TY, k = (tid - 2 * TX) % TY;
+        hr = k + 1, hc = side ? xl + 2 : 0;
+        hy = y0 + k, hx = map_axis(side ? x0 + xl + 1 : x0 - 1, p.nx, p.per_x);
+        halo = k <= yl;
+    }
+    struct Node {
+        R u[3], rho, T;
+    };
+    auto node = [&](int nx_, int ny_, int nz_) {
         R f[Q], g[Q];
-        load_local(p, pop, n, f, g);
+        load_local(p, pop, node_index(p, nx_, ny_, nz_), f, g);
         Moments<R> m;
         node_moments<kD, R, false, DEV>(f, g, p, m);
-        double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};   // G[a][b] = d u_a / d x_b
-        R up[3], um[3];
-        node_velocity(p, pop, node_index(p, map_axis(x + 1, p.nx, p.per_x), y, z), up);
-        node_velocity(p, pop, node_index(p, map_axis(x - 1, p.nx, p.per_x), y, z), um);
+        return Node{{m.ux, m.uy, m.uz}, m.rho, m.T};
+    };
+    auto put = [&](int b, int r, int c, const Node& n) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) G[a][0] = 0.5 * ((double)up[a] - (double)um[a]);
-        node_velocity(p, pop, node_index(p, x, map_axis(y + 1, p.ny, p.per_y), z), up);
-        node_velocity(p, pop, node_index(p, x, map_axis(y - 1, p.ny, p.per_y), z), um);
+        for (int a = 0; a < DD; ++a) us[b][a][r][c] = n.u[a];
+    };
+
+    constexpr bool kF64 = sizeof(R) == 8;
+    double acc[kF64 ? kStats : 1] = {};   // FP64 store
+    Tri2 t[6];                            // FP32 arithmetic: the sums in pairs
 #pragma unroll
-        for (int a = 0; a < 3; ++a) G[a][1] = 0.5 * ((double)up[a] - (double)um[a]);
-        if (kD == 3) {
-            node_velocity(p, pop, node_index(p, x, y, map_axis(z + 1, p.nz, p.per_z)), up);
-            node_velocity(p, pop, node_index(p, x, y, map_axis(z - 1, p.nz, p.per_z)), um);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) G[a][2] = 0.5 * ((double)up[a] - (double)um[a]);
-        }
-        const double theta = G[0][0] + G[1][1] + G[2][2];
-        const double wx = G[2][1] - G[1][2], wy = G[0][2] - G[2][0], wz = G[1][0] - G[0][1];
-        const double rho = m.rho, T = m.T;
-        const double uu = (double)m.ux * m.ux + (double)m.uy * m.uy + (double)m.uz * m.uz;
-        acc[0] += rho;
-        acc[1] += rho * rho;
-        acc[2] += rho * uu;
-        acc[3] += uu;
-        acc[4] += theta * theta;
-        acc[5] += T;
-        acc[6] += T * T;
-        const double w2 = wx * wx + wy * wy + wz * wz;
-        const double mu = p.mu_exp != 0.0 ? p.mu0 * pow(T / p.T0, p.mu_exp) : p.mu0;
-        acc[7] += G[0][0] * G[0][0];
-        acc[8] += w2;
-        acc[9] += (double)m.ux * m.ux;
-        acc[10] += mu * w2;
+    for (int k = 0; k < 6; ++k) t[k].zero();
+    const float eh = (float)p.mu_exp;
+    const Df mu_exp = {eh, kF64 ? 0.f : (float)(p.mu_exp - (double)eh)};
+
+    Node prev = {}, cur = {}, next = {};
+    if (active) {
+        if (DD == 3) prev = node(x, y, map_axis(zb - 1, p.nz, p.per_z));
+        cur = node(x, y, zb);
+        put(0, ty + 1, tx + 1, cur);
     }
-    // block reduction of kStats values, five at a time
-    static_assert(kStats <= 15, "three passes of five values");
-    __shared__ double tail[5];
-    for (int base = 0; base < kStats; base += 5) {
-        double v5[5];
+    if (halo) put(0, hr, hc, node(hx, hy, zb));
+    for (int z = zb; z < ze; ++z) {
+        const int b = (z - zb) & 1;
+        __syncthreads();   // plane z is in us[b]; us[b ^ 1] is free
+        const int zn = map_axis(z + 1, p.nz, p.per_z);
+        if (DD == 3 && active) {
+            next = node(x, y, zn);
+            if (z + 1 < ze) put(b ^ 1, ty + 1, tx + 1, next);
+        }
+        if (DD == 3 && halo && z + 1 < ze) put(b ^ 1, hr, hc, node(hx, hy, zn));
+        if (active) {
+            auto U = [&](int a, int r, int c) { return us[b][a][ty + 1 + r][tx + 1 + c]; };
+            if constexpr (kF64) {
+                double G[3][3] = {};   // twice d u_a / d x_b
 #pragma unroll
-        for (int k = 0; k < 5; ++k) v5[k] = base + k < kStats ? acc[base + k] : 0.0;
-        block_sum5(v5, tail);
-        __syncthreads();
-        if (threadIdx.x == 0)
-            for (int k = 0; k < 5 && base + k < kStats; ++k) partials[(size_t)kStats * blockIdx.x + base + k] = tail[k];
-        __syncthreads();
+                for (int a = 0; a < DD; ++a) {
+                    G[a][0] = U(a, 0, 1) - U(a, 0, -1);
+                    G[a][1] = U(a, 1, 0) - U(a, -1, 0);
+                    if (DD == 3) G[a][2] = next.u[a] - prev.u[a];
+                }
+                const double theta = G[0][0] + G[1][1] + G[2][2];
+                const double wx = G[2][1] - G[1][2], wy = G[0][2] - G[2][0], wz = G[1][0] - G[0][1];
+                const double w2 = wx * wx + wy * wy + wz * wz;
+                const double uu = cur.u[0] * cur.u[0] + cur.u[1] * cur.u[1] + cur.u[2] * cur.u[2];
+                acc[0] += cur.rho;
+                acc[1] = fma(cur.rho, cur.rho, acc[1]);
+                acc[2] = fma(cur.rho, uu, acc[2]);
+                acc[3] += uu;
+                acc[4] = fma(theta, theta, acc[4]);
+                acc[5] += cur.T;
+                acc[6] = fma(cur.T, cur.T, acc[6]);
+                acc[7] = fma(G[0][0], G[0][0], acc[7]);
+                acc[8] += w2;
+                acc[9] = fma(cur.u[0], cur.u[0], acc[9]);
+                if (p.powlaw) acc[10] = fma(pow_pos(cur.T * p.d_invT0, p.mu_exp), w2, acc[10]);
+            } else {
+                Df G[3][3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) G[a][k] = {0.f, 0.f};
+#pragma unroll
+                for (int a = 0; a < DD; ++a) {
+                    G[a][0] = df_diff(U(a, 0, 1), U(a, 0, -1));
+                    G[a][1] = df_diff(U(a, 1, 0), U(a, -1, 0));
+                    if (DD == 3) G[a][2] = df_diff(next.u[a], prev.u[a]);
+                }
+                Df theta = df_add(G[0][0], G[1][1]);
+                const Df wz = df_add(G[1][0], df_neg(G[0][1]));
+                Df w2 = df_sq(wz), uu = df_add(df_prod(cur.u[0], cur.u[0]), df_prod(cur.u[1], cur.u[1]));
+                if (DD == 3) {
+                    theta = df_add(theta, G[2][2]);
+                    w2 = df_add(w2, df_sq(df_add(G[2][1], df_neg(G[1][2]))));
+                    w2 = df_add(w2, df_sq(df_add(G[0][2], df_neg(G[2][0]))));
+                    uu = df_add(uu, df_prod(cur.u[2], cur.u[2]));
+                }
+                const Df r2 = df_prod(cur.rho, cur.rho), ruu = df_scale(uu, cur.rho), th2 = df_sq(theta);
+                const Df T2 = df_prod(cur.T, cur.T), gxx = df_sq(G[0][0]), ux2 = df_prod(cur.u[0], cur.u[0]);
+                t[0].add(make_float2(cur.rho, r2.h), make_float2(0.f, r2.l));
+                t[1].add(make_float2(ruu.h, uu.h), make_float2(ruu.l, uu.l));
+                t[2].add(make_float2(th2.h, cur.T), make_float2(th2.l, 0.f));
+                t[3].add(make_float2(T2.h, gxx.h), make_float2(T2.l, gxx.l));
+                t[4].add(make_float2(w2.h, ux2.h), make_float2(w2.l, ux2.l));
+                if (p.powlaw) {   // T^mu_exp |omega|^2; mu0 T0^-mu_exp comes at the end
+                    Df y;
+                    if (!pow_pos_df(cur.T, mu_exp, y)) {
+                        const double v = pow((double)cur.T, p.mu_exp);
+                        y.h = (float)v;
+                        y.l = (float)(v - (double)y.h);
+                    }
+                    y = df_mul(y, w2);
+                    t[5].add(make_float2(y.h, 0.f), make_float2(y.l, 0.f));
+                }
+            }
+        }
+        prev = cur;
+        cur = next;
+    }
+    const int lane = tid & 31, warp = tid >> 5;
+    if constexpr (kF64) {
+#pragma unroll
+        for (int k = 0; k < kStats; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+            if (lane == 0) part[warp][k] = acc[k];
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            t[k].warp_sum();
+            if (lane == 0) {
+                part[warp][2 * k] = (double)t[k].s.x + ((double)t[k].e1.x + (double)t[k].e2.x);
+                if (k < 5) part[warp][2 * k + 1] = (double)t[k].s.y + ((double)t[k].e1.y + (double)t[k].e2.y);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid < kStats) {
+        // theta, omega and d u_x / d x were summed as twice their values; the last sum lacks mu0 (FP32
+        // arithmetic: mu0 T0^-mu_exp)
+        const bool quad = tid == 4 || tid == 7 || tid == 8 || tid == 10;
+        const int k = tid == 10 && !p.powlaw ? 8 : tid;
+        double v = 0.0;
+        for (int w = 0; w < NT / 32; ++w) v += part[w][k];
+        if (quad) v *= 0.25;
+        if (tid == 10) v *= kF64 || !p.powlaw ? p.mu0 : p.mu0 * pow(p.T0, -p.mu_exp);
+        partials[(size_t)kStats * (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) + tid] = v;
     }
 }
 
@@ -1737,7 +1930,7 @@ constexpr int kTY3 = ELBM_TY3;           // D3Q27 re-read and tensor-copy kernel
 #define ELBM_TYP_F32 8
 #endif
 constexpr int kTYP = (kST == ST_F32) ? ELBM_TYP_F32 : kTY3;
-constexpr int kTotalsBlocks = 2 * 152;   // totals_kernel grid (grid-stride)
+constexpr int kTotalsBlocks = (sizeof(R) == 8 ? 4 : 5) * 152;   // totals_kernel grid (grid-stride)
 // Pipelined D3Q27 kernel per store: two plane buffers.  FP32 pairs make them 145 KB
 // (one CTA per SM, up to 255 registers; a third buffer would leave L1 almost no
 // room and measured 35 % slower); FP16/BF16 pairs are half the size (two CTAs per
@@ -2085,17 +2278,25 @@ int ensemble_occupancy(int ty) {
     return nb;
 }
 
+// Columns of 32 x 8 nodes over segments chosen like those of the fused kernels; a grid has at
+// most as many CTAs as the one-dimensional launches, or one per column (max_blocks bounds both).
 cudaError_t launch_stats(const KParams& p, const void* pop, double* partials, int* nblocks, cudaStream_t s,
                          long long* launches) {
-    stats_kernel<<<kTotalsBlocks, kThreads, 0, s>>>(p, (const P*)pop, partials);
+    const int tx = (p.nx + 31) / 32, ty = (p.ny + 7) / 8;
+    const long long most = blocks_1d_of(p.N) > kTotalsBlocks ? blocks_1d_of(p.N) : kTotalsBlocks;
+    int tz = choose_segment((double)tx * ty, p.nz, 152, 2, 32);
+    while (tz < p.nz && (long long)tx * ty * ((p.nz + tz - 1) / tz) > most) tz = tz < p.nz / 2 ? 2 * tz : p.nz;
+    const dim3 grid(tx, ty, (p.nz + tz - 1) / tz);
+    stats_kernel<kD><<<grid, dim3(32, 8), 0, s>>>(p, (const P*)pop, partials, tz);
     ++*launches;
-    *nblocks = kTotalsBlocks;
+    *nblocks = (int)(grid.x * grid.y * grid.z);
     return cudaGetLastError();
 }
 
 cudaError_t launch_totals(const KParams& p, const void* pop, double* partials, int* nblocks, cudaStream_t s,
                           long long* launches) {
-    totals_kernel<<<kTotalsBlocks, kThreads, 0, s>>>(p, (const P*)pop, partials);
+    constexpr int run = kTotThreads * kTotRun;
+    totals_kernel<<<kTotalsBlocks, kTotThreads, 0, s>>>(p, (const P*)pop, partials, (int)((p.N + run - 1) / run));
     ++*launches;
     *nblocks = kTotalsBlocks;
     return cudaGetLastError();

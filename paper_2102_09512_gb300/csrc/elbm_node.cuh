@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "elbm_powtab.h"
+
 namespace elbm {
 
 enum StoreKind { ST_F64 = 0, ST_F32 = 1, ST_F16DEV = 2, ST_BF16DEV = 3 };
@@ -174,6 +176,168 @@ __device__ __forceinline__ double qdiv(double a, double b) { return a / b; }
 __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double qpow(double a, double b) { return pow(a, b); }
 __device__ __forceinline__ float qpow(float a, float b) { return __powf(a, b); }
+
+// x^e in FP64 for the viscosity law: 2^(e log2 x) from two 128-entry tables and Taylor
+// polynomials of log2(1 + r), |r| < 0.0049, and 2^f - 1, |f| <= 2^-8 (truncation below
+// 2^-60), after Tang's table-driven method; log2 x and its product with e are carried as sums
+// of two doubles.  About 27 FP64 instructions where pow() takes several times as many; on
+// GB300's FP64 pipe (one warp instruction per 16 cycles and SM) that is what a node's
+// viscosity costs.  The remaining error is the rounding of 2^(j/128) and of the result (rms
+// 0.4 ulp; pow() 0.3).  Arguments outside [2^-100, 2^100], non-finite ones and exponents of 2 beyond 60 go
+// to pow().
+__device__ __forceinline__ double pow_pos(double x, double e) {
+    const int hi = __double2hiint(x);
+    if ((unsigned)(hi - 0x39b00000) >= 0x0c800000u) return pow(x, e);
+    const int k = (hi >> 20) - 1023, j = (hi >> 13) & 127;
+    const double2 tab = kLogTab[j];
+    const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
+    const double r = fma(m, tab.x, -1.0);
+    double q = fma(r, 0x1.a61762a7aded9p-3, -0x1.ec709dc3a03fdp-3);
+    q = fma(r, q, 0x1.2776c50ef9bfep-2);
+    q = fma(r, q, -0x1.71547652b82fep-2);
+    q = fma(r, q, 0x1.ec709dc3a03fdp-2);
+    q = fma(r, q, -0x1.71547652b82fep-1);
+    q = fma(r, q, 0x1.71547652b82fep+0);
+    // log2 x = L + l; k + h_j is exact, and not below |r q| in size unless that is tiny
+    const double A = (double)k + tab.y, L = fma(r, q, A), l = fma(r, q, A - L) + kLogLo[j];
+    const double t = e * L, tl = fma(e, l, fma(e, L, -t));
+    if ((__double2hiint(t) & 0x7fffffff) >= 0x404e0000 /* 60 */) return pow(x, e);
+    const double tn = fma(t, 128.0, 0x1.8p52);   // nearest multiple of 1/128 in the low bits
+    const int n = __double2loint(tn);
+    const double f = fma(tn - 0x1.8p52, -0x1p-7, t) + tl;
+    double s = fma(f, 0x1.5d87fe78a6731p-10, 0x1.3b2ab6fba4e77p-7);
+    s = fma(f, s, 0x1.c6b08d704a0c0p-5);
+    s = fma(f, s, 0x1.ebfbdff82c58fp-3);
+    s = fma(f, s, 0x1.62e42fefa39efp-1);
+    const double c = kExpTab[n & 127];
+    const double y = fma(c, f * s, c);
+    return __hiloint2double(__double2hiint(y) + ((n >> 7) << 20), __double2loint(y));
+}
+
+// ---------------------------------------------------------------------------
+// Error-free FP32 sums.  Two floats at a time (FADD2/FFMA2, sm_100 and later): the sums that
+// the diagnostics take over FP32 values run as unevaluated sums of three floats (Knuth's
+// TwoSum; relative error about 2^-70), since one FP64 addition costs as much of the SM as 64
+// FP32 ones.
+// ---------------------------------------------------------------------------
+// (V = float2; templates, so that host programs which include this header for another
+// architecture need not know the two-lane instructions)
+template <class V> __device__ __forceinline__ V sub2(V a, V b) { return __ffma2_rn(b, V{-1.f, -1.f}, a); }
+// a + b = s + err exactly, in both lanes
+template <class V> __device__ __forceinline__ V two_sum2(V a, V b, V& err) {
+    const V s = __fadd2_rn(a, b);
+    const V bb = sub2(s, a);
+    err = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
+}
+template <class V> struct TriOf {   // two running sums s + e1 + e2
+    V s, e1, e2;
+    __device__ __forceinline__ void zero() { s = e1 = e2 = V{0.f, 0.f}; }
+    __device__ __forceinline__ void add(V v) {
+        V r, r1;
+        s = two_sum2(s, v, r);
+        e1 = two_sum2(e1, r, r1);
+        e2 = __fadd2_rn(e2, r1);
+    }
+    // adds v + lo, lo a correction of v
+    __device__ __forceinline__ void add(V v, V lo) {
+        V r;
+        add(v);
+        e1 = two_sum2(e1, lo, r);
+        e2 = __fadd2_rn(e2, r);
+    }
+    __device__ __forceinline__ void add(const TriOf& o) {
+        add(o.s, o.e1);
+        e2 = __fadd2_rn(e2, o.e2);
+    }
+    // sum over the lanes of a warp, in every lane
+    __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            TriOf o;
+            o.s = V{__shfl_xor_sync(0xffffffffu, s.x, d), __shfl_xor_sync(0xffffffffu, s.y, d)};
+            o.e1 = V{__shfl_xor_sync(0xffffffffu, e1.x, d), __shfl_xor_sync(0xffffffffu, e1.y, d)};
+            o.e2 = V{__shfl_xor_sync(0xffffffffu, e2.x, d), __shfl_xor_sync(0xffffffffu, e2.y, d)};
+            add(o);
+        }
+    }
+};
+using Tri2 = TriOf<float2>;
+// FP64 running sum s + c (TwoSum)
+__device__ __forceinline__ void dd_add(double& s, double& c, double v) {
+    const double t = s + v, b = t - s;
+    c += (s - (t - b)) + (v - b);
+    s = t;
+}
+
+// Unevaluated sum h + l of two floats (|l| <= ulp(h)/2): differences and products of FP32
+// values are exact in this form, sums are rounded to about 2^-47.
+struct Df {
+    float h, l;
+};
+__device__ __forceinline__ Df df_diff(float a, float b) {   // a - b, exact
+    const float s = a - b, bb = s - a;
+    return {s, (a - (s - bb)) - (b + bb)};
+}
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+    const float s = a.h + b.h, bb = s - a.h;
+    const float e = ((a.h - (s - bb)) + (b.h - bb)) + (a.l + b.l);
+    const float h = s + e;
+    return {h, e - (h - s)};
+}
+__device__ __forceinline__ Df df_neg(Df a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Df df_prod(float a, float b) {   // a b, exact
+    const float p = __fmul_rn(a, b);
+    return {p, fmaf(a, b, -p)};
+}
+__device__ __forceinline__ Df df_sq(Df a) {
+    const float p = __fmul_rn(a.h, a.h);
+    return {p, fmaf(2.f * a.h, a.l, fmaf(a.h, a.h, -p))};
+}
+__device__ __forceinline__ Df df_mul(Df a, Df b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return {p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ Df df_scale(Df a, float b) {
+    const float p = __fmul_rn(a.h, b);
+    return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
+}
+
+// pow_pos of an FP32 x as a sum of two floats (relative error about 2^-44): the same steps in
+// pairs of floats, about 90 FP32 instructions where one FP64 instruction keeps the SM as busy
+// as 64.  False (and no value) for an x or an exponent of 2 that pow_pos leaves to pow().
+__device__ __forceinline__ bool pow_pos_df(float x, Df e, Df& y) {
+    const int b = __float_as_int(x);
+    if ((unsigned)(b - 0x0d800000) >= 0x64000000u) return false;   // 2^-100 <= x < 2^100
+    const int k = (b >> 23) - 127;
+    const float4 tab = kLogTabF[(b >> 16) & 127];
+    const Df m = df_prod(__int_as_float(b - (k << 23)), tab.x);
+    const float rh = m.h - 1.f;   // exact
+    const float r0 = rh + m.l;
+    const Df r = {r0, m.l - (r0 - rh)};
+    // log2(1 + r) = r (c1 + r (c2 + r q))
+    float q = fmaf(r.h, -0x1.ec709ep-3f, 0x1.2776c6p-2f);
+    q = fmaf(r.h, q, -0x1.715476p-2f);
+    q = fmaf(r.h, q, 0x1.ec709ep-2f);
+    const Df c1 = {0x1.715476p+0f, 0x1.4ae0c0p-26f}, c2 = {-0x1.715476p-1f, -0x1.4ae0c0p-27f};
+    const Df s = df_mul(r, df_add(c1, df_mul(r, df_add(c2, df_prod(r.h, q)))));
+    const Df L = df_add(df_add({(float)k, 0.f}, {tab.y, tab.z}), s);
+    const Df t = df_mul(e, L);
+    if (!(fabsf(t.h) < 60.f)) return false;
+    const float n = rintf(t.h * 128.f);
+    const float f0 = fmaf(n, -0x1p-7f, t.h), fh = f0 + t.l;
+    const Df f = {fh, t.l - (fh - f0)};
+    // 2^f - 1 = f (d1 + f (d2 + f (d3 + f d4)))
+    const Df d1 = {0x1.62e430p-1f, -0x1.05c610p-29f}, d2 = {0x1.ebfbe0p-3f, -0x1.f4e9c6p-33f};
+    const float d = fmaf(f.h, 0x1.3b2ab6p-7f, 0x1.c6b08ep-5f);
+    const Df w = df_mul(f, df_add(d1, df_mul(f, df_add(d2, df_prod(f.h, d)))));
+    const int ni = (int)n;
+    const float2 c = kExpTabF[ni & 127];
+    const Df z = df_add({c.x, c.y}, df_mul({c.x, c.y}, w));
+    const float two = __int_as_float(((ni >> 7) + 127) << 23);
+    y = {z.h * two, z.l * two};
+    return true;
+}
 
 // ---------------------------------------------------------------------------
 // Caloric equation of state (Eqs. U, E; R = 1): U(T) = int_0^T Cv dT and its inverse
