@@ -82,7 +82,9 @@ typedef enum { ELBM_DERIV_UPWIND = 0, ELBM_DERIV_CENTRAL = 1 } elbm_deriv;
 typedef enum {
     ELBM_KERNEL_FUSED = 0,        /* one kernel: halo-recomputed moments + collide + stream;
                                      D3Q27 FP32/FP16/BF16 prefetch each plane into shared
-                                     memory (cp.async), FP64 uses the re-read form; D2Q9
+                                     memory (cp.async); D3Q27 FP64, bound by its arithmetic
+                                     and not by memory, runs the two passes of
+                                     ELBM_KERNEL_TWOPASS, which compute each moment once; D2Q9
                                      marches strips of 128 nodes along y with the next rows
                                      prefetched into shared memory (cp.async), or runs one
                                      32 x 8 tile per CTA on grids too small for the march

@@ -267,7 +267,7 @@ cudaError_t step_one(elbm_handle* h, cudaStream_t st) {
     }
     const void* src = h->pop[h->cur];
     void* dst = h->pop[1 - h->cur];
-    if (h->kernel == ELBM_KERNEL_TWOPASS)
+    if (h->kernel == ELBM_KERNEL_TWOPASS || (h->kernel == ELBM_KERNEL_FUSED && h->ops->fused_is_twopass))
         e = h->ops->step_twopass(h->kp, src, dst, h->auxp + h->aux.qfield, step_partials(h), &h->step_blocks,
                                  status_ptr(h), st, &h->launches);
     else if (h->kernel == ELBM_KERNEL_FUSED_REREAD)

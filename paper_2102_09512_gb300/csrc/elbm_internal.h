@@ -294,6 +294,7 @@ struct Ops {
     cudaError_t (*step_aa)(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
                            cudaStream_t s, long long* launches, int from_l1);
     int march_width;   // D2Q9: strip width of the single-lattice row march of this store
+    int fused_is_twopass;   // the default schedule of this combination is the two-pass one (D3Q27 FP64)
 };
 
 // z-segment length of the fused D3Q27 kernels.  Each CTA marches one (tile, segment)

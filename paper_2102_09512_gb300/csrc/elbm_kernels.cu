@@ -11,6 +11,7 @@
 //   fused3d_kernel       D3Q27 one-kernel step: xy tile + halo marching along z, the pulled
 //                        populations of each plane prefetched into shared memory with
 //                        cp.async one plane ahead
+//   moments64_kernel, collide64_kernel  the two passes in FP64 (the default of D3Q27 FP64)
 //   fused3d_reread_kernel  D3Q27 one-kernel step without the shared-memory plane buffers:
 //                        the populations of a plane are gathered twice (moments of the
 //                        next plane, then the collision), the second time from L2
@@ -179,54 +180,64 @@ __device__ __forceinline__ void node_totals(const Moments<R>& m, R rE, R v[5]) {
     v[4] = rE;
 }
 
-// Per-thread running sum of the node totals over the planes of a z segment:
-// Kahan-compensated in FP64; in FP32 a plain sum (at most p.tz terms of per-node
+// Per-thread running sum of the node totals over the planes of a z segment: in FP64 a
+// Kahan-compensated sum of plain sums of four nodes (compensating every node would cost 20 of
+// the update's FP64 instructions); in FP32 a plain sum (at most p.tz terms of per-node
 // values that are themselves FP32 results), which saves the registers of the
 // compensation terms.
 struct Acc5 {
-    R s[5], c[5];
+    R s[5], c[5], q[5];
+    int n;
     __device__ __forceinline__ void zero() {
+        n = 0;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) s[k] = c[k] = R(0);
+        for (int k = 0; k < 5; ++k) s[k] = c[k] = q[k] = R(0);
     }
-    __device__ __forceinline__ void add(const R v[5]) {
+    __device__ __forceinline__ void kahan() {
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-            if constexpr (sizeof(R) == 8) {
-                const R y = v[k] - c[k];
-                const R t = s[k] + y;
-                c[k] = (t - s[k]) - y;
-                s[k] = t;
-            } else {
-                s[k] += v[k];
-            }
+            const R y = q[k] - c[k];
+            const R t = s[k] + y;
+            c[k] = (t - s[k]) - y;
+            s[k] = t;
         }
+    }
+    __device__ __forceinline__ void add(const R v[5]) {
+        if constexpr (sizeof(R) == 8) {
+            const bool first = (n & 3) == 0;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = first ? v[k] : q[k] + v[k];
+            if ((++n & 3) == 0) kahan();
+        } else {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) s[k] += v[k];
+        }
+    }
+    __device__ __forceinline__ void total(R out[5]) {
+        if constexpr (sizeof(R) == 8)
+            if (n & 3) kahan();
+#pragma unroll
+        for (int k = 0; k < 5; ++k) out[k] = s[k] - c[k];
     }
 };
 
-// Block-wide FP64 sum of 5 values per thread; thread 0 writes out[0..4].
-__device__ __forceinline__ void block_sum5(double v[5], double* __restrict__ out) {
-    __shared__ double red[32][5];
+// Block-wide FP64 sum of 5 values per thread of a block of at most MAXT threads; out[0..4].  The
+// values go through shared memory, so that one warp per value adds them on full warps: 60 FP64
+// warp instructions for 256 threads, where a shuffle tree in every warp takes 240.
+template <int MAXT>
+__device__ __forceinline__ void block_sum5(const double v[5], double* __restrict__ out) {
+    __shared__ double red[5][MAXT];
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    const int nthreads = blockDim.x * blockDim.y * blockDim.z;
-    const int lane = tid & 31, warp = tid >> 5;
+    const int nthreads = blockDim.x * blockDim.y * blockDim.z, lane = tid & 31;
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) red[warp][k] = v[k];
+    for (int k = 0; k < 5; ++k) red[k][tid] = v[k];
     __syncthreads();
-    if (warp == 0) {
-        const int nw = (nthreads + 31) >> 5;
+    for (int k = tid >> 5; k < 5; k += nthreads >> 5) {
+        double t = red[k][lane];
+        for (int j = lane + 32; j < nthreads; j += 32) t += red[k][j];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double t = lane < nw ? red[lane][k] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) out[k] = t;
-        }
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) out[k] = t;
     }
 }
 
@@ -235,10 +246,10 @@ __device__ __forceinline__ void block_sum5(double v[5], double* __restrict__ out
 // tile's whole update on GB300's narrow FP64 pipe), the sum of the warp partials in FP64.
 // With T = double it is block_sum5.  An FP32 warp partial of 32 node values carries a
 // relative rounding error of about 1e-7, below the rounding of the FP32 values summed.
-template <typename T>
+template <typename T, int MAXT = 256>
 __device__ __forceinline__ void block_sum5_warp(T v[5], double* __restrict__ out) {
     if constexpr (sizeof(T) == 8) {
-        block_sum5(v, out);
+        block_sum5<MAXT>(v, out);
     } else {
         __shared__ double red[32][5];
         const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
@@ -717,6 +728,102 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* __res
     block_sum5_warp(tot, partials + 5 * blockIdx.x);
 }
 
+// The two passes in FP64.  The FP64 pipe bounds every FP64 kernel and the memory is idle (8 % of
+// its rate), so the first pass computes the moments once and for all and hands them on, rather
+// than have the second, or a halo, compute them again: rho, T, u and the flux part of q* go to
+// the node's own pairs of the first planes of the destination store, which the same node's
+// thread of the second pass reads before it writes there.  Q~, which neighbours read, goes to
+// the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
+// moments 2.3 times (both with the arithmetic of their time); D2Q9 marches rows instead.
+#if ELBM_ST == 0   // ST_F64
+template <bool PULL>
+__global__ void __launch_bounds__(kThreads1D)
+moments64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, R* __restrict__ qf,
+                 P* __restrict__ dst, double* __restrict__ partials, int* __restrict__ status) {
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    R tot[5] = {0, 0, 0, 0, 0};
+    bool bad = false;
+    if (n < p.N) {
+        const unsigned row = (unsigned)n / (unsigned)p.nx, x = (unsigned)n - row * (unsigned)p.nx;
+        const unsigned z = row / (unsigned)p.ny, y = row - z * (unsigned)p.ny;
+        PullRows r;
+        pull_rows<PULL>(p, (int)x, (int)y, (int)z, r);
+        R f[Q], g[Q];
+        gather(p, src, r, f, g);
+        Moments<R> m;
+        node_moments<kD, R, true, DEV>(f, g, p, m);
+        bad = nonphysical(m);
+        node_totals(m, m.rE, tot);
+        R dq[3];
+        Relax<kD, R, DEV>::flux(m, dq);
+        const R c = fma(R(-3), m.T, R(1));
+        qf[n] = tot[1] * fma(-m.ux, m.ux, c);
+        qf[p.N + n] = tot[2] * fma(-m.uy, m.uy, c);
+        const size_t N = (size_t)p.N;
+        dst[n] = Cd::enc(m.rho, m.T);
+        dst[N + n] = Cd::enc(m.ux, m.uy);
+        if (kD == 3) {
+            qf[2 * p.N + n] = tot[3] * fma(-m.uz, m.uz, c);
+            dst[2 * N + n] = Cd::enc(m.uz, dq[2]);
+            dst[3 * N + n] = Cd::enc(dq[0], dq[1]);
+        } else {
+            dst[2 * N + n] = Cd::enc(dq[0], dq[1]);
+        }
+    }
+    flag_if(bad, status);
+    block_sum5_warp(tot, partials + 5 * blockIdx.x);
+}
+constexpr int kThreads64 = 128;   // second pass: smaller CTAs, so that one's loads overlap another's arithmetic
+template <bool PULL>
+__global__ void __launch_bounds__(kThreads64, 2)
+collide64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* dst, const R* __restrict__ qf) {
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= p.N) return;
+    const unsigned row = (unsigned)n / (unsigned)p.nx, xu = (unsigned)n - row * (unsigned)p.nx;
+    const int x = (int)xu, z = (int)(row / (unsigned)p.ny), y = (int)(row - (unsigned)z * (unsigned)p.ny);
+    const long long N = p.N;
+    PullRows r;
+    pull_rows<PULL>(p, x, y, z, r);
+    R rho, T, ux, uy, uz = R(0), dq[3] = {};
+    Cd::dec(dst[n], rho, T);
+    Cd::dec(dst[N + n], ux, uy);
+    if (kD == 3) {
+        Cd::dec(dst[2 * N + n], uz, dq[2]);
+        Cd::dec(dst[3 * N + n], dq[0], dq[1]);
+    } else {
+        Cd::dec(dst[2 * N + n], dq[0], dq[1]);
+    }
+    const int xm = map_axis(x - 1, p.nx, p.per_x), xp = map_axis(x + 1, p.nx, p.per_x);
+    const int ym = map_axis(y - 1, p.ny, p.per_y), yp = map_axis(y + 1, p.ny, p.per_y);
+    R qxm = qf[node_index(p, xm, y, z)], qxp = qf[node_index(p, xp, y, z)];
+    R qym = qf[N + node_index(p, x, ym, z)], qyp = qf[N + node_index(p, x, yp, z)];
+    if (kD == 2 && p.has_fixed) {
+        if (beyond_fixed(p, 0, x - 1, p.nx)) qxm = fixed_Q(p, 0);
+        if (beyond_fixed(p, 0, x + 1, p.nx)) qxp = fixed_Q(p, 0);
+        if (beyond_fixed(p, 1, y - 1, p.ny)) qym = fixed_Q(p, 1);
+        if (beyond_fixed(p, 1, y + 1, p.ny)) qyp = fixed_Q(p, 1);
+    }
+    const R Dx = dQ(p.deriv, ux, qxm, qf[n], qxp);
+    const R Dy = dQ(p.deriv, uy, qym, qf[N + n], qyp);
+    R Dz = R(0);
+    if (kD == 3) {
+        const int zm = map_axis(z - 1, p.nz, p.per_z), zp = map_axis(z + 1, p.nz, p.per_z);
+        Dz = dQ(p.deriv, uz, qf[2 * N + node_index(p, x, y, zm)], qf[2 * N + n],
+                qf[2 * N + node_index(p, x, y, zp)]);
+    }
+    Relax<kD, R, DEV> rx;
+    rx.init(rho, T, ux, uy, uz, dq, Dx, Dy, Dz, p);
+    const unsigned nn = (unsigned)n;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        R f, g;
+        Cd::dec(*src_ptr(p, src, r, i), f, g);
+        if (kD == 2 && ((r.gmask >> i) & 1u)) fixed_pair(p, i, f, g);
+        (dst + (size_t)i * (size_t)N)[nn] = Cd::enc(rx.f(i, f, p), rx.g(i, g, p));
+    }
+}
+#endif
+
 // ---------------------------------------------------------------------------
 // AA single-store layout (periodic grids, two-pass schedule)
 // ---------------------------------------------------------------------------
@@ -944,7 +1051,7 @@ __device__ __forceinline__ void fused2d_tile(const KParams& p, const P* __restri
         store_node(p, dst, node_index(p, x, y, 0), f, g);
     }
     flag_if(bad, status);
-    if (partial) block_sum5_warp(tot, partial);
+    if (partial) block_sum5_warp<R, TX * TY>(tot, partial);
     __syncthreads();   // the shared arrays are reused by the next tile of a persistent CTA
 }
 
@@ -1241,8 +1348,7 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     cp_async_wait_all();
     flag_if(bad, status);
     R tot[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) tot[k] = acc.s[k] - acc.c[k];
+    acc.total(tot);
     block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
 }
 
@@ -1547,8 +1653,7 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
     cp_async_wait_all();
     flag_if(bad, status);
     R tot[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) tot[k] = acc.s[k] - acc.c[k];
+    acc.total(tot);
     block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
 }
 
@@ -1631,8 +1736,7 @@ fused3d_reread_kernel(const __grid_constant__ KParams p, const P* __restrict__ s
     }
     flag_if(bad, status);
     R tot[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) tot[k] = acc.s[k] - acc.c[k];
+    acc.total(tot);
     block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
 }
 
@@ -1863,8 +1967,7 @@ march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     march2d_segment<W, NB, CAL, FIX>(p, PlanesParam{&pl, src}, x0, y0, ye, march_smem, acc, bad);
     flag_if(bad, status);
     R tot[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) tot[k] = acc.s[k] - acc.c[k];
+    acc.total(tot);
     block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * blockIdx.y));
 }
 
@@ -2038,6 +2141,20 @@ int max_blocks(const KParams& p) {
     return (int)m;
 }
 
+template <bool PULL>
+void launch_two_passes(const KParams& p, const void* src, void* dst, void* qfield, double* partials, int* status,
+                       cudaStream_t s) {
+    const unsigned nb = blocks_1d(p.N);
+#if ELBM_ST == 0
+    moments64_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
+    collide64_kernel<PULL><<<(unsigned)((p.N + kThreads64 - 1) / kThreads64), kThreads64, 0, s>>>(
+        p, (const P*)src, (P*)dst, (const R*)qfield);
+#else
+    moments_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (R*)qfield);
+    collide_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
+#endif
+}
+
 cudaError_t launch_init(const KParams& p, const double* rho, const double* u, const double* T, void* pop,
                         void* spare, void* qfield, double* partials, int* status, cudaStream_t s,
                         long long* launches) {
@@ -2049,8 +2166,7 @@ cudaError_t launch_init(const KParams& p, const double* rho, const double* u, co
     // extraction and totals read each node's own values.
     const unsigned nb = blocks_1d(p.N);
     init_kernel<<<nb, kThreads, 0, s>>>(p, rho, u, T, (P*)spare, status, 0, p.N);
-    moments_kernel<false><<<nb, kThreads, 0, s>>>(p, (const P*)spare, (R*)qfield);
-    collide_kernel<false><<<nb, kThreads, 0, s>>>(p, (const P*)spare, (P*)pop, (const R*)qfield, partials, status);
+    launch_two_passes<false>(p, spare, pop, qfield, partials, status, s);
     *launches += 3;
     return cudaGetLastError();
 }
@@ -2101,8 +2217,7 @@ cudaError_t launch_fields(const KParams& p, const void* pop, double* rho, double
 cudaError_t launch_twopass(const KParams& p, const void* src, void* dst, void* qfield, double* partials,
                            int* nblocks, int* status, cudaStream_t s, long long* launches) {
     const unsigned nb = blocks_1d(p.N);
-    moments_kernel<true><<<nb, kThreads, 0, s>>>(p, (const P*)src, (R*)qfield);
-    collide_kernel<true><<<nb, kThreads, 0, s>>>(p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
+    launch_two_passes<true>(p, src, dst, qfield, partials, status, s);
     *launches += 2;
     *nblocks = (int)nb;
     return cudaGetLastError();
@@ -2332,7 +2447,7 @@ const Ops kOps = {kD,          kST,           sizeof(P) / 2,  sizeof(R),        
                   launch_init, launch_fields, launch_twopass, launch_fused_default, launch_fused_reread,
                   launch_totals, launch_ensemble, ensemble_occupancy, launch_stats,
                   kD == 3 ? (kPipe ? kTYP : kTY3) : 1, fused_occupancy, launch_fused_tma, tma_supported, encode_tmap,
-                  launch_fused_pf, launch_init_nodes, launch_fields_nodes, launch_step_aa, kW2L};
+                  launch_fused_pf, launch_init_nodes, launch_fields_nodes, launch_step_aa, kW2L, kD == 3 && !kPipe};
 
 }  // namespace
 

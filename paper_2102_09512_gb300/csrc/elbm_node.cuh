@@ -177,6 +177,24 @@ __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b
 __device__ __forceinline__ double qpow(double a, double b) { return pow(a, b); }
 __device__ __forceinline__ float qpow(float a, float b) { return __powf(a, b); }
 
+// 1 / x in FP64: the hardware's approximation (about 20 bits) and one step of Householder's
+// third-order iteration x <- x (1 + e + e^2), e = 1 - d x, three FP64 instructions where the
+// compiler's division takes about ten; within 1 ulp.  Outside 2^(+-1000) the division.
+__device__ __forceinline__ double recip(double d) {
+    const int ex = (__double2hiint(d) >> 20) & 0x7ff;
+    if ((unsigned)(ex - 23) >= 2000u) return 1.0 / d;
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
+    const double e = fma(-d, x, 1.0);
+    return fma(x, fma(e, e, e), x);
+}
+// Tests of an FP64 value on its bits: comparisons would take the FP64 pipe.
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool positive64(double x) {   // x > 0 (NaN: by its sign bit)
+    const int hi = __double2hiint(x);
+    return hi >= 0 && (hi | __double2loint(x)) != 0;
+}
+
 // x^e in FP64 for the viscosity law: 2^(e log2 x) from two 128-entry tables and Taylor
 // polynomials of log2(1 + r), |r| < 0.0049, and 2^f - 1, |f| <= 2^-8 (truncation below
 // 2^-60), after Tang's table-driven method; log2 x and its product with e are carried as sums
@@ -448,7 +466,9 @@ __device__ __forceinline__ R g_energy(const R* g, const KParams& p) {
 // u = j / rho and T from E = Cv T + u^2/2.
 template <typename R, bool CAL = true>
 __device__ __forceinline__ void finish_moments(R rho, R jx, R jy, R jz, R rE, const KParams& p, Moments<R>& m) {
-    const R inv = qdiv(R(1), rho);
+    R inv;
+    if constexpr (sizeof(R) == 8) inv = recip(rho);
+    else inv = qdiv(R(1), rho);
     m.rho = rho;
     m.rE = rE;
     m.ux = jx * inv;
@@ -544,12 +564,19 @@ __device__ __forceinline__ R anomaly(R rho, R ua, R T) {
 template <typename R>
 __device__ __forceinline__ R dQ(int deriv, R ua, R qm, R q0, R qp) {
     if (deriv) return R(0.5) * (qp - qm);
+    if constexpr (sizeof(R) == 8) {   // one subtraction, the operands chosen on the sign bit
+        const bool up = positive64(ua);
+        return (up ? q0 : qp) - (up ? qm : q0);
+    }
     return ua > R(0) ? (q0 - qm) : (qp - q0);
 }
 
 // Unphysical-state test used to latch ELBM_ERR_NONPHYSICAL.
 template <typename R>
 __device__ __forceinline__ bool nonphysical(const Moments<R>& m) {
+    if constexpr (sizeof(R) == 8)
+        return !positive64(m.rho) || !positive64(m.T) || !finite64(m.rho) || !finite64(m.T) || !finite64(m.ux) ||
+               !finite64(m.uy) || !finite64(m.uz);
     return !(m.rho > R(0)) || !(m.T > R(0)) || !isfinite(m.rho) || !isfinite(m.T) ||
            !isfinite(m.ux) || !isfinite(m.uy) || !isfinite(m.uz);
 }
@@ -728,6 +755,110 @@ struct Relax {
             const R q = cx != 0 ? dq[0] : (cy != 0 ? dq[1] : dq[2]);
             if (cx + cy + cz < 0) v += h * q;
             else v -= h * q;
+        }
+        return v;
+    }
+};
+
+// The same collision in FP64, arranged for the fewest FP64 instructions (the pipe takes one warp
+// instruction per 16 cycles and SM, so their number is the time: D2Q9 about 320 -> 190 a node,
+// D3Q27 about 860 -> 430 with the two passes below).
+//   - every per-axis factor is carried as twice its value (Psi_{+-1} = P +- xi, Psi_0 = 2 - 2 P),
+//     and 1/8 (D2Q9: 1/4) goes into the density factors;
+//   - the rates are written over P = rho T: w = 2 P / (2 mu + P), w1 = 2 Pr P / (2 mu + Pr P),
+//     (2 - w) / (2 rho w) = mu / (rho P), three reciprocals;
+//   - mu(T) by pow_pos.
+// With u = 0 the factors of opposite directions are equal bit for bit, as in Relax: a gas at
+// rest stays at rest exactly.
+template <int D, bool CAL>
+struct Relax<D, double, false, CAL> {
+    using R = double;
+    double omw, omw1;
+    double X[3], wY[3], Z[3];                 // 2 Psi(u, T + u^2 + k D); wY with the density factor
+    double gx[3], ax[3], A[3], B[3], gz[3], sz[3];
+    double hq[3];                             // (omega - omega_1)/2 (q* - q^eq)
+
+    static __device__ __forceinline__ void phi2(double u, double P, double out[3]) {
+        out[0] = P - u;
+        out[1] = fma(-2.0, P, 2.0);
+        out[2] = P + u;
+    }
+    // q* - q^eq without its derivative part: u . (P - rho T I - rho u u)
+    static __device__ __forceinline__ void flux(const Moments<double>& m, double dq[3]) {
+        const double P = m.rho * m.T, jx = m.rho * m.ux, jy = m.rho * m.uy;
+        const double dxx = fma(-jx, m.ux, m.Pxx - P), dyy = fma(-jy, m.uy, m.Pyy - P), dxy = fma(-jx, m.uy, m.Pxy);
+        dq[0] = fma(m.uy, dxy, m.ux * dxx);
+        dq[1] = fma(m.uy, dyy, m.ux * dxy);
+        dq[2] = 0.0;
+        if (D == 3) {
+            const double jz = m.rho * m.uz;
+            const double dxz = fma(-jx, m.uz, m.Pxz), dyz = fma(-jy, m.uz, m.Pyz), dzz = fma(-jz, m.uz, m.Pzz - P);
+            dq[0] = fma(m.uz, dxz, dq[0]);
+            dq[1] = fma(m.uz, dyz, dq[1]);
+            dq[2] = fma(m.uz, dzz, fma(m.uy, dyz, m.ux * dxz));
+        }
+    }
+    __device__ __forceinline__ void init(const Moments<double>& m, double Dx, double Dy, double Dz, const KParams& p) {
+        double dq[3];
+        flux(m, dq);
+        init(m.rho, m.T, m.ux, m.uy, m.uz, dq, Dx, Dy, Dz, p);
+    }
+    __device__ __forceinline__ void init(double rho, double T, double ux, double uy, double uz, const double dq[3],
+                                         double Dx, double Dy, double Dz, const KParams& p) {
+        double mu = p.mu0;
+        if (p.powlaw) mu *= pow_pos(T * p.d_invT0, p.mu_exp);
+        const double P = rho * T, PrP = p.Pr * P;
+        const double t = P * recip(fma(2.0, mu, P)), t1 = PrP * recip(fma(2.0, mu, PrP));   // w/2, w1/2
+        const double k = mu * recip(rho * P);
+        omw = fma(-2.0, t, 1.0);
+        omw1 = fma(-2.0, t1, 1.0);
+        const double rs = (D == 3 ? 0.25 : 0.5) * rho, wr = t * rs, w1r = t1 * rs;
+        const double T25 = 2.5 * T, TT = T * T;
+        double Y[3], sx[3], gy[3], sy[3];
+        axis(ux, T, T25, TT, k, Dx, X, gx, sx);
+        axis(uy, T, T25, TT, k, Dy, Y, gy, sy);
+        if (D == 3) {
+            axis(uz, T, T25, TT, k, Dz, Z, gz, sz);
+        }
+        const double U = U_of_T<double, CAL>(T, p);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            ax[a] = fma(U, gx[a], sx[a]);
+            wY[a] = wr * Y[a];
+            A[a] = w1r * gy[a];
+            B[a] = w1r * sy[a];
+        }
+        const double h = t - t1;
+        hq[0] = h * fma(ux, 0.5 * Dx, dq[0]);
+        hq[1] = h * fma(uy, 0.5 * Dy, dq[1]);
+        hq[2] = D == 3 ? h * fma(uz, 0.5 * Dz, dq[2]) : 0.0;
+    }
+    // factors of one axis: 2 Psi of f^ex, 2 phi and 2 psi of g^eq (gfactors)
+    static __device__ __forceinline__ void axis(double u, double T, double T25, double TT, double k, double Da,
+                                                double F[3], double phi[3], double ps[3]) {
+        const double u2 = u * u, P = T + u2;
+        phi2(u, fma(k, Da, P), F);
+        phi2(u, P, phi);
+        const double o = u * fma(0.5, u2, T), s = fma(u2, fma(0.5, u2, T25), TT);
+        ps[0] = s - o;
+        ps[1] = fma(-2.0, s, u2);
+        ps[2] = s + o;
+    }
+    // i is a compile-time constant after unrolling; the row products are common subexpressions
+    __device__ __forceinline__ double f(int i, double fi, const KParams&) const {
+        const int a = i % 3, b = (i / 3) % 3, c = i / 9;
+        const double yz = D == 3 ? wY[b] * Z[c] : wY[b];
+        return fma(omw, fi, X[a] * yz);
+    }
+    __device__ __forceinline__ double g(int i, double gi, const KParams&) const {
+        const int a = i % 3, b = (i / 3) % 3, c = i / 9;
+        const double q1 = D == 3 ? A[b] * gz[c] : A[b];
+        const double q2 = D == 3 ? fma(A[b], sz[c], B[b] * gz[c]) : B[b];
+        double v = fma(omw1, gi, fma(ax[a], q1, gx[a] * q2));
+        const int cx = cx_of(i), cy = cy_of(i), cz = cz_of<D>(i);
+        if (cx * cx + cy * cy + cz * cz == 1) {
+            const double q = cx != 0 ? hq[0] : (cy != 0 ? hq[1] : hq[2]);
+            v = cx + cy + cz < 0 ? v + q : v - q;
         }
         return v;
     }

@@ -1,5 +1,5 @@
 """GPU tests of the diagnostics' arithmetic: the table-driven power functions of the
-viscosity law against extended precision, the totals against exactly rounded sums of the
+viscosity law and the FP64 reciprocal against extended precision, the totals against exactly rounded sums of the
 stored populations, and the statistics at grids that are ragged against their tiles."""
 import math
 import os
@@ -29,10 +29,11 @@ POW_PROGRAM = r"""
 #include <cstdio>
 #include <vector>
 #include "elbm_node.cuh"
-__global__ void run(const double* x, const double* e, double* y, double* h, double* l, int n) {
+__global__ void run(const double* x, const double* e, double* y, double* h, double* l, double* q, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     y[i] = elbm::pow_pos(x[i], e[i]);
+    q[i] = elbm::recip(e[i] * x[i]);
     const float eh = (float)e[i];
     elbm::Df r = {-1.f, 0.f};
     if (!elbm::pow_pos_df((float)x[i], {eh, (float)(e[i] - (double)eh)}, r)) r = {-1.f, 0.f};
@@ -41,14 +42,14 @@ __global__ void run(const double* x, const double* e, double* y, double* h, doub
 }
 int main(int argc, char** argv) {
     const int n = atoi(argv[1]);
-    std::vector<double> b(2 * n), o(3 * n);
+    std::vector<double> b(2 * n), o(4 * n);
     if (fread(b.data(), 8, 2 * n, stdin) != (size_t)(2 * n)) return 2;
     double* d;
-    if (cudaMalloc(&d, 5 * n * sizeof(double)) != cudaSuccess) return 3;
+    if (cudaMalloc(&d, 6 * n * sizeof(double)) != cudaSuccess) return 3;
     cudaMemcpy(d, b.data(), 2 * n * sizeof(double), cudaMemcpyHostToDevice);
-    run<<<(n + 255) / 256, 256>>>(d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, n);
-    if (cudaMemcpy(o.data(), d + 2 * n, 3 * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return 4;
-    return fwrite(o.data(), 8, 3 * n, stdout) == (size_t)(3 * n) ? 0 : 5;
+    run<<<(n + 255) / 256, 256>>>(d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, d + 5 * n, n);
+    if (cudaMemcpy(o.data(), d + 2 * n, 4 * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return 4;
+    return fwrite(o.data(), 8, 4 * n, stdout) == (size_t)(4 * n) ? 0 : 5;
 }
 """
 
@@ -57,7 +58,8 @@ def test_power_functions(tmp_path):
     """pow_pos: half an ulp each from the table entry and the final addition and less than a
     half from everything carried in two doubles, so 1.5 ulp; the pair form: its logarithm
     times the exponent is good to 2^-45 of its size (at most 60, in use below 8), so 2^-41
-    relative for |e log2 x| <= 8.  x includes both sides of every table boundary near 1."""
+    relative for |e log2 x| <= 8.  x includes both sides of every table boundary near 1.  recip:
+    the iteration's last addition rounds once, its factors leave less than another half ulp."""
     from paper_2102_09512_gb300 import build as B
     src = tmp_path / "p.cu"
     src.write_text(POW_PROGRAM)
@@ -71,9 +73,11 @@ def test_power_functions(tmp_path):
     e = np.where(np.arange(x.size) % 2, 0.76, rng.uniform(-1.3, 1.3, x.size))
     e[-3:] = 0.76
     out = subprocess.run([exe, str(x.size)], input=np.concatenate([x, e]).tobytes(), stdout=subprocess.PIPE, check=True)
-    y, h, l = np.frombuffer(out.stdout).reshape(3, -1)
+    y, h, l, q = np.frombuffer(out.stdout).reshape(4, -1)
     ref = np.power(x.astype(np.longdouble), e.astype(np.longdouble))
     assert float(np.max(np.abs(y - ref) / np.spacing(np.abs(y)))) <= 1.5
+    r = 1.0 / (e * x)
+    assert np.max(np.abs(q - r) / np.spacing(np.abs(r))) <= 1.0
     assert np.all(h > 0)
     assert float(np.max(np.abs(h.astype(np.longdouble) + l - ref) / ref)) <= 2.0 ** -41
 
