@@ -85,10 +85,11 @@ typedef enum {
                                      memory (cp.async); D3Q27 FP64, bound by its arithmetic
                                      and not by memory, runs the two passes of
                                      ELBM_KERNEL_TWOPASS, which compute each moment once; D2Q9
-                                     marches strips of 128 nodes along y with the next rows
-                                     prefetched into shared memory (cp.async), or runs one
-                                     32 x 8 tile per CTA on grids too small for the march
-                                     to fill the device (see elbm_set_tile_z) */
+                                     runs one strip of 30 nodes or one 32 x 8 tile per CTA on
+                                     small grids and marches strips of 128 nodes (256 for the
+                                     16-bit stores) along y with the next rows prefetched into
+                                     shared memory (cp.async) on larger ones, the two passes in
+                                     FP64 (see elbm_set_tile_z) */
     ELBM_KERNEL_TWOPASS = 1,      /* moment/Q~ pass into the aux buffer, then collide+stream */
     ELBM_KERNEL_FUSED_REREAD = 2, /* one kernel, D3Q27 plane gathered twice (second from L2);
                                      D2Q9: one 32 x 8 tile per CTA, no march */
@@ -227,10 +228,10 @@ int elbm_set_kernel(elbm_handle *h, int kernel);
 /* Length of the segment each CTA of the fused kernel marches over: z planes for
  * D3Q27, rows (y) for D2Q9.  Chosen at elbm_create for the current device (the
  * length that best fills the last wave of CTAs, each segment costing about two
- * planes of prologue); a tuning knob, results agree to rounding.  D2Q9 grids with
- * fewer 128-node strips x row segments than the device has SMs run the fused schedule
- * as one 32 x 8 tile per CTA instead of the march; setting a segment length here
- * selects the march for any grid. */
+ * planes of prologue); a tuning knob, results agree to rounding.  D2Q9 grids of up to
+ * eight 30-node strips or four 32 x 8 tiles per SM, and FP64 ones, run the fused schedule
+ * without the march (see elbm_kernel); setting a segment length here selects the march for
+ * any D2Q9 grid.  No effect on the default schedule of D3Q27 FP64. */
 int elbm_set_tile_z(elbm_handle *h, int tz);
 
 /* Raw copy of the current population store (pop_bytes) to or from host memory,

@@ -267,7 +267,7 @@ cudaError_t step_one(elbm_handle* h, cudaStream_t st) {
     }
     const void* src = h->pop[h->cur];
     void* dst = h->pop[1 - h->cur];
-    if (h->kernel == ELBM_KERNEL_TWOPASS || (h->kernel == ELBM_KERNEL_FUSED && h->ops->fused_is_twopass))
+    if (h->kernel == ELBM_KERNEL_TWOPASS || (h->kernel == ELBM_KERNEL_FUSED && h->kp.sched == kSchedTwoPass))
         e = h->ops->step_twopass(h->kp, src, dst, h->auxp + h->aux.qfield, step_partials(h), &h->step_blocks,
                                  status_ptr(h), st, &h->launches);
     else if (h->kernel == ELBM_KERNEL_FUSED_REREAD)
@@ -353,10 +353,11 @@ int elbm_create(const elbm_params* prm, elbm_handle** out) {
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
         {
             if (D == 3) h->kp.tz = choose_tz(kp, h->ops->fused_tile_y, sms, h->ops->fused_occupancy(h->kp), kp.tz);
-            else plan_d2q9(h->kp, sms, h->ops->fused_occupancy(h->kp), h->ops->march_width);
+            else plan_d2q9(h->kp, sms, h->ops->fused_occupancy(h->kp), h->ops->march_width, p.store == ELBM_F64);
         }
         else
             cudaGetLastError();   // no device: keep the fallback, clear the error
+        if (D == 3 && p.store == ELBM_F64) h->kp.sched = kSchedTwoPass;
     }
     const KParams& k = h->kp;
 
@@ -622,10 +623,10 @@ int elbm_set_tile_z(elbm_handle* h, int tz) {
     KParams k = h->kp;
     const int planes = h->D == 3 ? h->prm.nz : h->prm.ny;   // the marched axis
     k.tz = tz < planes ? tz : planes;
-    k.tile2d = 0;   // D2Q9: an explicit row segment selects the row march
+    if (h->D == 2) k.sched = kSchedMarch;   // an explicit row segment selects the row march
     if (h->ops->max_blocks(k) > h->aux.max_blocks) return ELBM_ERR_ARG;   // partials would not fit
     h->kp.tz = k.tz;
-    h->kp.tile2d = 0;
+    h->kp.sched = k.sched;
     h->drop_graphs();
     return ELBM_OK;
 }

@@ -173,8 +173,13 @@ int step_once(elbm_ensemble* e) {
         for (int k = 0; k < e->n && err == cudaSuccess; ++k) {
             const size_t off = (size_t)e->offset[k] * e->ops->value_bytes * 2;
             int nb = 0;
-            err = e->ops->step_fused(e->kp[k], (const char*)e->pop[c] + off, (char*)e->pop[1 - c] + off,
-                                     (double*)(e->aux + e->a_partials), &nb, e->status(), e->stream, &e->launches);
+            const void* src = (const char*)e->pop[c] + off;
+            void* dst = (char*)e->pop[1 - c] + off;
+            double* part = (double*)(e->aux + e->a_partials);
+            err = e->kp[k].sched == kSchedTwoPass
+                      ? e->ops->step_twopass(e->kp[k], src, dst, e->aux + e->a_qfield, part, &nb, e->status(), e->stream,
+                                             &e->launches)
+                      : e->ops->step_fused(e->kp[k], src, dst, part, &nb, e->status(), e->stream, &e->launches);
         }
     } else if (e->use_graph) {
         if (!e->graph[c]) err = build_graph(e, c, 1, &e->graph[c]);
@@ -233,11 +238,11 @@ int elbm_ensemble_create(const elbm_params* params, int n, elbm_ensemble** out) 
     e->pop_bytes = (size_t)off * ops->value_bytes * 2;
     // aux layout
     // per-CTA partials of the one-launch-per-instance mode: its row segments are chosen
-    // for the device at bind, no shorter than 16 rows, so size for that
+    // for the device at bind, no shorter than kShortestSegment rows, so size for that
     int maxb = 0;
     for (int k = 0; k < n; ++k) {
         KParams shortest = e->kp[k];
-        shortest.tz = shortest.ny < 16 ? shortest.ny : 16;
+        shortest.tz = shortest.ny < kShortestSegment ? shortest.ny : kShortestSegment;
         const int b = std::max(ops->max_blocks(e->kp[k]), ops->max_blocks(shortest));
         if (b > maxb) maxb = b;
     }
@@ -279,7 +284,8 @@ int elbm_ensemble_bind(elbm_ensemble* e, void* pop_a, void* pop_b, void* aux, vo
     e->bound = true;
     // the one-launch-per-instance mode runs each instance as a single lattice would on this device
     const int sms = sm_count();
-    for (KParams& k : e->kp) plan_d2q9(k, sms, e->ops->fused_occupancy(k), e->ops->march_width);
+    for (KParams& k : e->kp) plan_d2q9(k, sms, e->ops->fused_occupancy(k), e->ops->march_width,
+                                           e->store == ELBM_F64);
     cudaError_t c = cudaMemsetAsync(e->status(), 0, sizeof(int), e->stream);
     if (c == cudaSuccess)
         c = cudaMemcpyAsync(e->aux + e->a_params, e->kp.data(), e->kp.size() * sizeof(KParams),

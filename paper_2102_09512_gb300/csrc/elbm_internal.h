@@ -294,18 +294,22 @@ struct Ops {
     cudaError_t (*step_aa)(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
                            cudaStream_t s, long long* launches, int from_l1);
     int march_width;   // D2Q9: strip width of the single-lattice row march of this store
-    int fused_is_twopass;   // the default schedule of this combination is the two-pass one (D3Q27 FP64)
 };
 
-// z-segment length of the fused D3Q27 kernels.  Each CTA marches one (tile, segment)
-// column; the grid runs in waves of sms * per_sm CTAs.  The choice maximises the fill
-// of the last wave times tz / (tz + 2), the second factor charging each segment about
-// two planes of prologue (the Q~ plane below it and the plane above it).  Ties keep
-// the longer segment.  Without device information the fallback is kept.
-inline int choose_segment(double tiles, int nplanes, int sms, int per_sm, int fallback) {
+// Segment length of the marching kernels.  Each CTA marches one (tile, segment) column; the
+// grid runs in waves of sms * per_sm CTAs.  The choice maximises the fill of the last wave times
+// tz / (tz + 2), the second factor charging each segment about two planes of prologue (the Q~
+// plane below it and the plane above it): the shortest run of waves * (tz + 2) planes.  Ties keep
+// the longer segment.  Segments go down to kShortestSegment planes, so that a grid which long ones
+// would leave in a fraction of a wave fills one (D2Q9 1024^2, FP32: 912 CTAs of 9 rows 29.3 us,
+// 512 of 16 rows 32.6; 724^2: 14.7 and 21.4; D3Q27 64^3, FP32: 8 planes 27.5 us, 16 planes 47.5;
+// 32^3: 2 planes 10.4, 16 planes 43.6).  Without device information the fallback is kept.
+constexpr int kShortestSegment = 1;
+inline int choose_segment(double tiles, int nplanes, int sms, int per_sm, int fallback,
+                          int shortest = kShortestSegment) {
     if (sms <= 0 || per_sm <= 0) return fallback < nplanes ? fallback : nplanes;
     const double slots = (double)sms * per_sm;
-    const int lo = nplanes < 16 ? nplanes : 16, hi = 128;
+    const int lo = nplanes < shortest ? nplanes : shortest, hi = 128;
     int best = fallback < nplanes ? fallback : nplanes;
     double best_score = -1.0;
     for (int nseg = 1; nseg <= nplanes; ++nseg) {
@@ -325,20 +329,40 @@ inline int choose_segment(double tiles, int nplanes, int sms, int per_sm, int fa
 }
 inline int choose_tz(const KParams& k, int ty, int sms, int per_sm, int fallback) {
     const double tiles = (double)((k.nx + 31) / 32) * (double)((k.ny + ty - 1) / ty);
-    return choose_segment(tiles, k.nz, sms, per_sm, fallback);
+    // a grid of fewer than 16 planes stays one segment
+    return choose_segment(tiles, k.nz, sms, per_sm, fallback, k.nz < 16 ? k.nz : kShortestSegment);
 }
 // The same choice for the D2Q9 row march: strips of `width` nodes, segments of rows.
 inline int choose_rows(const KParams& k, int sms, int per_sm, int fallback, int width) {
     return choose_segment((double)((k.nx + width - 1) / width), k.ny, sms, per_sm, fallback);
 }
-// D2Q9 schedule for a device of `sms` SMs: the row segment, and whether the grid is too
-// small for the march (fewer strips x segments than SMs), in which case the default fused
-// schedule runs the one-tile-per-CTA kernel instead.  Without device information the
-// march with the fallback segment is kept.
-inline void plan_d2q9(KParams& k, int sms, int per_sm, int width) {
+
+// D2Q9 small-grid kernels: a strip of kRowW nodes of a row per CTA, kRowMost strips at most
+// (one partial vector each).
+constexpr int kRowW = 30;
+constexpr int kRowMost = 8 * 152;
+inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW - 1) / kRowW) * k.ny; }
+
+// What the default schedule of a D2Q9 grid runs on a device of `sms` SMs, and the row segment of
+// the march.  Measured on 152 SMs, us a step (Sod parameters, zero-gradient x ends):
+//   FP32     strips  tiles  march        FP64   strips  tiles  two passes
+//   800x4      2.7    3.4    5.8         800x4     5.5   11.3    13.6
+//   180^2      3.3    3.8     -          1700x8   10.5   17.9    14.4
+//   256^2      4.5    4.6    6.5         128^2    16.1   17.9    13.6
+//   384^2      7.4    5.8    7.8         256^2    46.6   33.0    45.0
+//   512^2     11.6   10.1    9.5         384^2    94.4   63.2    64.2
+//   724^2     20.6   17.6   14.6         512^2     173    109     101
+//   1024^2      -    37.2   29.3         1448^2     -     848     750   (march 880)
+// (16-bit stores as FP32).  So: strips while there are at most eight to an SM (FP64, where each
+// keeps four warps busy: four), tiles while there are at most four to an SM, else the march,
+// for FP64 the two passes, which the FP64 pipe bounds and no wave of CTAs leaves idle.
+constexpr int kSchedMarch = 0, kSchedTile = 1, kSchedRow = 2, kSchedTwoPass = 3;
+inline void plan_d2q9(KParams& k, int sms, int per_sm, int width, bool f64) {
     k.tz = choose_rows(k, sms, per_sm, k.tz, width);
-    const long long ctas = (long long)((k.nx + width - 1) / width) * ((k.ny + k.tz - 1) / k.tz);
-    k.tile2d = sms > 0 && ctas < sms;
+    const long long strips = row_strips(k), tiles = (long long)((k.nx + 31) / 32) * ((k.ny + 7) / 8);
+    if (sms > 0 && strips <= (f64 ? 4LL : 8LL) * sms && strips <= kRowMost) k.sched = kSchedRow;
+    else if (sms > 0 && tiles <= 4LL * sms) k.sched = kSchedTile;
+    else k.sched = f64 ? kSchedTwoPass : kSchedMarch;
 }
 
 constexpr int kTmapStage = 0, kTmapPrefetch = 1;   // encode_tmap kinds

@@ -295,6 +295,21 @@ __device__ __forceinline__ void cp_async_wait_pending() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Programmatic dependent launch.  The step kernels are launched by launch_dependent: the next
+// one's CTAs may be set up as soon as every CTA of this one has called launch_dependents, and
+// wait for its end, with its writes visible, before they touch memory (wait_for_previous, in every
+// CTA, so that the wait carries over from launch to launch).  Launched one after another
+// without it, kernels start on a raster of about 2.05 us.  Most kernels call it late, a marching
+// one when its column is done: CTAs set up beside a whole grid that is still running are
+// spread unevenly (D2Q9 724^2, FP32: 22.6 us a step without dependent launches, 34.7 with early
+// ones).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void dependent_launch_point() {
+    launch_dependents();
+    wait_for_previous();
+}
+
 // ---------------------------------------------------------------------------
 // initial state and field extraction
 // ---------------------------------------------------------------------------
@@ -666,6 +681,7 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
 template <bool PULL>
 __global__ void moments_kernel(const __grid_constant__ KParams p, const P* __restrict__ src,
                                R* __restrict__ qf) {
+    dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const int x = (int)(n % p.nx);
@@ -687,6 +703,7 @@ template <bool PULL>
 __global__ void collide_kernel(const __grid_constant__ KParams p, const P* __restrict__ src,
                                P* __restrict__ dst, const R* __restrict__ qf,
                                double* __restrict__ partials, int* __restrict__ status) {
+    dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     R tot[5] = {0, 0, 0, 0, 0};
     bool bad = false;
@@ -740,6 +757,7 @@ template <bool PULL>
 __global__ void __launch_bounds__(kThreads1D)
 moments64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, R* __restrict__ qf,
                  P* __restrict__ dst, double* __restrict__ partials, int* __restrict__ status) {
+    wait_for_previous();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     R tot[5] = {0, 0, 0, 0, 0};
     bool bad = false;
@@ -770,6 +788,7 @@ moments64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, R
             dst[2 * N + n] = Cd::enc(dq[0], dq[1]);
         }
     }
+    launch_dependents();
     flag_if(bad, status);
     block_sum5_warp(tot, partials + 5 * blockIdx.x);
 }
@@ -777,6 +796,7 @@ constexpr int kThreads64 = 128;   // second pass: smaller CTAs, so that one's lo
 template <bool PULL>
 __global__ void __launch_bounds__(kThreads64, 2)
 collide64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* dst, const R* __restrict__ qf) {
+    wait_for_previous();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const unsigned row = (unsigned)n / (unsigned)p.nx, xu = (unsigned)n - row * (unsigned)p.nx;
@@ -811,6 +831,7 @@ collide64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P
         Dz = dQ(p.deriv, uz, qf[2 * N + node_index(p, x, y, zm)], qf[2 * N + n],
                 qf[2 * N + node_index(p, x, y, zp)]);
     }
+    launch_dependents();
     Relax<kD, R, DEV> rx;
     rx.init(rho, T, ux, uy, uz, dq, Dx, Dy, Dz, p);
     const unsigned nn = (unsigned)n;
@@ -870,6 +891,7 @@ __device__ __forceinline__ void aa_store(const KParams& p, P* A, const PullRows&
 // Pass 1 of an AA step: Q~_aaa of every node from its post-stream populations.
 template <bool FROM_L1>
 __global__ void aa_moments_kernel(const __grid_constant__ KParams p, P* A, R* __restrict__ qf) {
+    dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const int x = (int)(n % p.nx), y = (int)((n / p.nx) % p.ny), z = (int)(n / ((long long)p.nx * p.ny));
@@ -896,6 +918,7 @@ template <bool FROM_L1>
 __global__ void __launch_bounds__(kThreads1D, kAaMinBlocks)
 aa_collide_kernel(const __grid_constant__ KParams p, P* A, const R* __restrict__ qf,
                                   double* __restrict__ partials, int* __restrict__ status) {
+    dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     R tot[5] = {0, 0, 0, 0, 0};
     bool bad = false;
@@ -1038,6 +1061,7 @@ __device__ __forceinline__ void fused2d_tile(const KParams& p, const P* __restri
             store_halo_q(q);
         }
     }
+    if constexpr (ONE_WAIT) launch_dependents();
     __syncthreads();
 
     R tot[5] = {0, 0, 0, 0, 0};
@@ -1059,9 +1083,250 @@ template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY)
 fused2d_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst,
                double* __restrict__ partials, int* __restrict__ status) {
+    wait_for_previous();
     fused2d_tile<TY, CAL, true>(p, src, dst, blockIdx.x, blockIdx.y, partials + 5 * (blockIdx.x + gridDim.x * blockIdx.y),
                      status);
 }
+
+// D2Q9 step of a small grid: a warp owns kRowW = 30 nodes of a row; its first and last lane hold
+// the nodes at either end, for their Q~_xxx alone.  Nothing goes through shared memory but
+// the totals: Q~_xxx of the x neighbours comes by shuffle, and of the two y neighbours only the
+// upwind one is evaluated (both for the central derivative).  The pairs of all three nodes
+// are requested before any arithmetic, so a warp waits for memory once.  A grid of a few
+// thousand nodes is all latency, and in FP64 the arithmetic of a warp keeps its SM's pipe busy
+// for about 16 cycles an instruction: one warp to a CTA spreads 3,200 nodes over 108 SMs
+// where the 32 x 8 tiles used 25 (800 x 4, FP64: 14.4 us a step; this kernel 4.5).
+template <bool CAL, bool FIX>
+__global__ void __launch_bounds__(128)
+fused2d_row_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst, int strips,
+                   double* __restrict__ partials, int* __restrict__ status) {
+    __shared__ R red[4][5][32];
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int y = warp / strips, x = (warp - y * strips) * kRowW - 1 + lane;
+    const bool have = y < p.ny && x <= p.nx;                        // a node of the strip or an end
+    const bool node = have && lane >= 1 && lane <= kRowW && x < p.nx;
+    const int xc = map_axis(x, p.nx, p.per_x);
+    const int yd = map_axis(y - 1, p.ny, p.per_y), yu = map_axis(y + 1, p.ny, p.per_y);
+    auto request = [&](int yy, P pk[Q]) {
+        PullRows r;
+        pull_rows(p, xc, yy, 0, r);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) pk[i] = *src_ptr(p, src, r, i);
+    };
+    auto decode = [&](const P pk[Q], int yy, R f[Q], R g[Q]) {
+        const unsigned gm = fixed_mask<FIX>(p, xc, yy);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            Cd::dec(pk[i], f[i], g[i]);
+            if ((gm >> i) & 1u) fixed_pair(p, i, f[i], g[i]);
+        }
+    };
+    wait_for_previous();
+    P pc[Q], pd[Q], pu[Q];
+    if (have) request(y, pc);
+    if (node) {
+        request(yd, pd);
+        request(yu, pu);
+    }
+    R f[Q], g[Q], qx = R(0);
+    Moments<R> m;
+    if (have) {
+        decode(pc, y, f, g);
+        node_moments<kD, R, true, DEV, CAL>(f, g, p, m);
+        qx = FIX && p.has_fixed && beyond_fixed(p, 0, x, p.nx) ? fixed_Q(p, 0) : anomaly(m.rho, m.ux, m.T);
+    }
+    launch_dependents();
+    const R qxm = __shfl_up_sync(0xffffffffu, qx, 1), qxp = __shfl_down_sync(0xffffffffu, qx, 1);
+    R tot[5] = {0, 0, 0, 0, 0};
+    bool bad = false;
+    if (node) {
+        bad = nonphysical(m);
+        const R q0 = anomaly(m.rho, m.uy, m.T);
+        auto neighbour_q = [&](const P pk[Q], int yy, int y_unmapped) {
+            if (FIX && p.has_fixed && beyond_fixed(p, 1, y_unmapped, p.ny)) return fixed_Q(p, 1);
+            R hf[Q], hg[Q];
+            decode(pk, yy, hf, hg);
+            Moments<R> hm;
+            node_moments<kD, R, false, DEV, CAL>(hf, hg, p, hm);
+            return anomaly(hm.rho, hm.uy, hm.T);
+        };
+        R Dy;
+        if (p.deriv) {
+            Dy = R(0.5) * (neighbour_q(pu, yu, y + 1) - neighbour_q(pd, yd, y - 1));
+        } else {
+            const bool up = m.uy > R(0);
+            P pn[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) pn[i] = up ? pd[i] : pu[i];
+            const R qn = neighbour_q(pn, up ? yd : yu, up ? y - 1 : y + 1);
+            Dy = up ? q0 - qn : qn - q0;
+        }
+        const R Dx = dQ(p.deriv, m.ux, qxm, qx, qxp);
+        node_totals(m, m.rE, tot);
+        collide<kD, R, DEV, CAL>(f, g, m, Dx, Dy, R(0), p);
+        store_node(p, dst, node_index(p, x, y, 0), f, g);
+    }
+    flag_if(bad, status);
+    // totals of the warp: lane 4k + j adds eight of the 32 values of sum k
+#pragma unroll
+    for (int k = 0; k < 5; ++k) red[wb][k][lane] = tot[k];
+    __syncwarp();
+    const int k = lane >> 2, j = lane & 3;
+    R t = R(0);
+    if (k < 5) {
+        const R* v = red[wb][k] + j;
+        t = ((v[0] + v[4]) + (v[8] + v[12])) + ((v[16] + v[20]) + (v[24] + v[28]));
+    }
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    if (k < 5 && j == 0) partials[5 * warp + k] = (double)t;
+}
+
+// The same strip in FP64, where one warp alone would take 10.5 us: an SM's quarter finishes an FP64
+// warp instruction in 64 cycles, whatever lanes it has, and starts the next one only then, so
+// a warp's instructions run one after another (measured: 64.6 cycles each at any degree of
+// independence, 16.2 with four warps).  So four warps share a node's arithmetic: the moments
+// of the node and of its two y neighbours; then the rates, the factors of either axis and the
+// flux of q*; then one row of three directions each, and the totals.  About 86 instructions deep
+// instead of 205.
+#if ELBM_ST == 0 && ELBM_D == 2
+template <bool CAL, bool FIX>
+__global__ void __launch_bounds__(128)
+fused2d_split_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst, int strips,
+                     double* __restrict__ partials, int* __restrict__ status) {
+    enum { RHO, TT_, UX, UY, RE, QXL, QX, QXR, QY, QD, QU, PX, GX, AX = GX + 3, PY = AX + 3, GY, SY = GY + 3, KK = SY + 3,
+           WR, W1R, OMW, OMW1, HH, DX, DY, FX, FY, NV };
+    __shared__ double v[NV][34];   // column lane + 1 of a node; QXL and QXR are QX shifted by one
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, col = lane + 1;
+    const int y = blockIdx.x / strips, x = (blockIdx.x - y * strips) * kRowW - 1 + lane;
+    const bool have = x <= p.nx;                                    // a node of the strip or an end
+    const bool node = have && lane >= 1 && lane <= kRowW && x < p.nx;
+    const int xc = map_axis(x, p.nx, p.per_x);
+    // warps 0 and 3: the node's row; 1: the row below; 2: above
+    const int yw = wb == 1 ? y - 1 : wb == 2 ? y + 1 : y, yy = map_axis(yw, p.ny, p.per_y);
+    wait_for_previous();
+    double f[Q], g[Q];
+    Moments<double> m;
+    if (wb == 0 || wb == 3 ? have : node) {
+        PullRows r;
+        pull_rows(p, xc, yy, 0, r);
+        r.gmask = fixed_mask<FIX>(p, xc, yy);
+        gather(p, src, r, f, g);
+        if (wb == 3) {
+            double rho, jx, jy, jz, P6[6];
+            f_moments<kD, double, true, false>(f, p, rho, jx, jy, jz, P6);
+            m.Pxx = P6[0];
+            m.Pyy = P6[1];
+            m.Pxy = P6[3];
+        } else {
+            node_moments<kD, double, false, false, CAL>(f, g, p, m);
+            if (wb == 0) {
+                v[RHO][col] = m.rho;
+                v[TT_][col] = m.T;
+                v[UX][col] = m.ux;
+                v[UY][col] = m.uy;
+                v[RE][col] = m.rE;
+                const double q =
+                    FIX && p.has_fixed && beyond_fixed(p, 0, x, p.nx) ? fixed_Q(p, 0) : anomaly(m.rho, m.ux, m.T);
+                v[QX][col] = v[QXL][col + 1] = v[QXR][col - 1] = q;
+                v[QY][col] = anomaly(m.rho, m.uy, m.T);
+            } else {
+                v[wb == 1 ? QD : QU][col] = FIX && p.has_fixed && beyond_fixed(p, 1, yw, p.ny)
+                                                ? fixed_Q(p, 1)
+                                                : anomaly(m.rho, m.uy, m.T);
+            }
+        }
+    }
+    __syncthreads();
+    if (node) {
+        m.rho = v[RHO][col];
+        m.T = v[TT_][col];
+        m.ux = v[UX][col];
+        m.uy = v[UY][col];
+        m.rE = v[RE][col];
+        m.uz = 0.0;
+        using Rx = Relax<kD, double, false, CAL>;
+        if (wb == 0) {
+            double k, omw, omw1, wr, w1r, h;
+            Rx::rates(m.rho, m.T, p, k, omw, omw1, wr, w1r, h);
+            v[KK][col] = k;
+            v[WR][col] = wr;
+            v[W1R][col] = w1r;
+            v[OMW][col] = omw;
+            v[OMW1][col] = omw1;
+            v[HH][col] = h;
+        } else if (wb < 3) {
+            const double u = wb == 1 ? m.ux : m.uy, u2 = u * u, Pa = m.T + u2;
+            double phi[3], ps[3];
+            Rx::phi2(u, Pa, phi);
+            Rx::psi2(u, u2, m.T, 2.5 * m.T, m.T * m.T, ps);
+            const double U = U_of_T<double, CAL>(m.T, p);
+            v[wb == 1 ? PX : PY][col] = Pa;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                v[(wb == 1 ? GX : GY) + a][col] = phi[a];
+                v[(wb == 1 ? AX : SY) + a][col] = wb == 1 ? fma(U, phi[a], ps[a]) : ps[a];
+            }
+        } else {
+            double dq[3];
+            Rx::flux(m, dq);
+            const double Dx = dQ(p.deriv, m.ux, v[QXL][col], v[QX][col], v[QXR][col]);
+            const double Dy = dQ(p.deriv, m.uy, v[QD][col], v[QY][col], v[QU][col]);
+            v[DX][col] = Dx;
+            v[DY][col] = Dy;
+            v[FX][col] = fma(m.ux, 0.5 * Dx, dq[0]);
+            v[FY][col] = fma(m.uy, 0.5 * Dy, dq[1]);
+        }
+    }
+    __syncthreads();
+    launch_dependents();
+    if (wb < 3) {   // row c_y = wb - 1
+        if (node) {
+            const double k = v[KK][col], omw = v[OMW][col], omw1 = v[OMW1][col];
+            double X[3], Y[3];
+            Relax<kD, double, false, CAL>::phi2(m.ux, fma(k, v[DX][col], v[PX][col]), X);
+            Relax<kD, double, false, CAL>::phi2(m.uy, fma(k, v[DY][col], v[PY][col]), Y);
+            const double wY = v[WR][col] * (wb == 0 ? Y[0] : wb == 1 ? Y[1] : Y[2]);
+            const double A = v[W1R][col] * v[GY + wb][col], B = v[W1R][col] * v[SY + wb][col];
+            const double hq = v[HH][col] * v[wb == 1 ? FX : FY][col];
+            PullRows r;
+            pull_rows(p, x, y, 0, r);
+            r.gmask = fixed_mask<FIX>(p, x, y);
+            const unsigned n = (unsigned)(x + p.nx * y);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int i = a + 3 * wb;
+                double fi, gi;
+                Cd::dec((src + (size_t)i * (size_t)p.N)[(unsigned)((wb == 0 ? r.row[0][1] : wb == 1 ? r.row[1][1] : r.row[2][1]) + r.xs[a])], fi, gi);
+                if ((r.gmask >> i) & 1u) {
+                    fi = p.fixd[i][0];
+                    gi = p.fixd[i][1];
+                }
+                double go = fma(omw1, gi, fma(v[AX + a][col], A, v[GX + a][col] * B));
+                // unit-speed directions: (+-1, 0) in the middle row, (0, +-1) in the outer ones
+                if (wb == 1 ? a != 1 : a == 1) go = (wb == 1 ? a == 0 : wb == 0) ? go + hq : go - hq;
+                (dst + (size_t)i * (size_t)p.N)[n] = Cd::enc(fma(omw, fi, X[a] * wY), go);
+            }
+        }
+    } else {
+        flag_if(node && nonphysical(m), status);
+        // lane 4k + j adds eight of the 32 values of sum k: rho, rho u_x, rho u_y, rho u_z, rho E
+        __syncwarp();
+        v[QX][col] = node ? m.rho * m.ux : 0.0;
+        v[QY][col] = node ? m.rho * m.uy : 0.0;
+        v[QD][col] = node ? m.rho : 0.0;
+        v[QU][col] = node ? m.rE : 0.0;
+        __syncwarp();
+        const int k = lane >> 2, j = lane & 3;
+        const double* w = v[k == 0 ? QD : k == 1 ? QX : k == 2 ? QY : QU] + 1 + j;
+        double t = ((w[0] + w[4]) + (w[8] + w[12])) + ((w[16] + w[20]) + (w[24] + w[28]));
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if (k < 5 && j == 0) partials[5 * blockIdx.x + k] = k == 3 ? 0.0 : t;
+    }
+}
+#endif
 
 // Persistent D2Q9 ensemble step: the tiles of all instances form one work list
 // (instance k owns tiles [tile_start[k], tile_start[k+1]), tiles_x[k] per row); CTA
@@ -1070,6 +1335,7 @@ fused2d_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* 
 template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY)
 ensemble2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int* __restrict__ status) {
+    wait_for_previous();
     __shared__ int s_start[kMaxEnsemble + 1];
     __shared__ int s_tx[kMaxEnsemble];
     const int tid = threadIdx.x + TX * threadIdx.y;
@@ -1184,6 +1450,7 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     auto QX = [&](int b, int row, int col) -> R& { return qxs[(b * TY + row) * (TX + 2) + col]; };
     auto QY = [&](int b, int row, int col) -> R& { return qys[(b * (TY + 2) + row) * TX + col]; };
 
+    wait_for_previous();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int zb = blockIdx.z * p.tz, ze = min(zb + p.tz, p.nz);
@@ -1345,6 +1612,7 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
         qz_prev = qz_cur;
         qz_cur = qz_next;
     }
+    launch_dependents();
     cp_async_wait_all();
     flag_if(bad, status);
     R tot[5];
@@ -1471,6 +1739,7 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
     auto QX = [&](int b, int row, int col) -> R& { return qxs[(b * TY + row) * (TX + 2) + col]; };
     auto QY = [&](int b, int row, int col) -> R& { return qys[(b * (TY + 2) + row) * TX + col]; };
 
+    wait_for_previous();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int zb = blockIdx.z * p.tz, ze = min(zb + p.tz, p.nz);
@@ -1641,6 +1910,7 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
         qz_prev = qz_cur;
         qz_cur = qz_next;
     }
+    launch_dependents();
     if (gave_up) {
         // the last phase of each buffer may still have copies in flight
 #pragma unroll
@@ -1663,6 +1933,7 @@ template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY, 2)
 fused3d_reread_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst,
                       double* __restrict__ partials, int* __restrict__ status) {
+    wait_for_previous();
     __shared__ R qx[2][TY][TX + 2];
     __shared__ R qy[2][TY + 2][TX];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
@@ -1734,6 +2005,7 @@ fused3d_reread_kernel(const __grid_constant__ KParams p, const P* __restrict__ s
         qz_prev = qz_cur;
         qz_cur = qz_next;
     }
+    launch_dependents();
     flag_if(bad, status);
     R tot[5];
     acc.total(tot);
@@ -1960,11 +2232,13 @@ __global__ void ELBM_MARCH_BOUNDS(W)
 march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* __restrict__ src,
                double* __restrict__ partials, int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
+    wait_for_previous();
     const int x0 = blockIdx.x * W, y0 = blockIdx.y * p.tz, ye = min(y0 + p.tz, p.ny);
     Acc5 acc;
     acc.zero();
     bool bad = false;
     march2d_segment<W, NB, CAL, FIX>(p, PlanesParam{&pl, src}, x0, y0, ye, march_smem, acc, bad);
+    launch_dependents();
     flag_if(bad, status);
     R tot[5];
     acc.total(tot);
@@ -1979,6 +2253,7 @@ __global__ void __launch_bounds__(W)
 ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int seg,
                         int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
+    wait_for_previous();
     __shared__ int s_start[kMaxEnsemble + 1];
     __shared__ int s_tx[kMaxEnsemble];
     for (int k = threadIdx.x; k <= a.n; k += W) s_start[k] = a.tile_start[k];
@@ -1998,12 +2273,29 @@ ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __re
         march2d_segment<W, NB, CAL, true>(p, PlanesBase{src + off, dst + off, (size_t)p.N, src + off}, bx * W, y0,
                                 min(y0 + seg, p.ny), march_smem, acc, bad);
     }
+    launch_dependents();
     flag_if(bad, status);
 }
 
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
+// Launch with programmatic dependent launch allowed on the kernel before it in the stream.
+template <class... Args, class... Act>
+cudaError_t launch_dependent(void (*kern)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Act... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Args>(args)...);
+}
+
 constexpr int kThreads = kThreads1D;
 constexpr int kTY2 = 8;                  // D2Q9 tile kernel: 32 x 8 tiles
 constexpr int kW2 = kMarchW2;            // D2Q9 row march: strips of kW2 nodes
@@ -2138,6 +2430,7 @@ int max_blocks(const KParams& p) {
     const long long c = (long long)gt.x * gt.y * gt.z;
     if (c > m) m = c;
     if (m < kTotalsBlocks) m = kTotalsBlocks;
+    if (kD == 2 && row_strips(p) <= kRowMost && m < row_strips(p)) m = row_strips(p);
     return (int)m;
 }
 
@@ -2146,12 +2439,11 @@ void launch_two_passes(const KParams& p, const void* src, void* dst, void* qfiel
                        cudaStream_t s) {
     const unsigned nb = blocks_1d(p.N);
 #if ELBM_ST == 0
-    moments64_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
-    collide64_kernel<PULL><<<(unsigned)((p.N + kThreads64 - 1) / kThreads64), kThreads64, 0, s>>>(
-        p, (const P*)src, (P*)dst, (const R*)qfield);
+    launch_dependent(moments64_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
+    launch_dependent(collide64_kernel<PULL>, (unsigned)((p.N + kThreads64 - 1) / kThreads64), kThreads64, 0, s, p, (const P*)src, (P*)dst, (const R*)qfield);
 #else
-    moments_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (R*)qfield);
-    collide_kernel<PULL><<<nb, kThreads, 0, s>>>(p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
+    launch_dependent(moments_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (R*)qfield);
+    launch_dependent(collide_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
 #endif
 }
 
@@ -2196,11 +2488,11 @@ cudaError_t launch_step_aa(const KParams& p, void* A, void* qfield, double* part
                            cudaStream_t s, long long* launches, int from_l1) {
     const unsigned nb = blocks_1d(p.N);
     if (from_l1) {
-        aa_moments_kernel<true><<<nb, kThreads, 0, s>>>(p, (P*)A, (R*)qfield);
-        aa_collide_kernel<true><<<nb, kThreads, 0, s>>>(p, (P*)A, (const R*)qfield, partials, status);
+        launch_dependent(aa_moments_kernel<true>, nb, kThreads, 0, s, p, (P*)A, (R*)qfield);
+        launch_dependent(aa_collide_kernel<true>, nb, kThreads, 0, s, p, (P*)A, (const R*)qfield, partials, status);
     } else {
-        aa_moments_kernel<false><<<nb, kThreads, 0, s>>>(p, (P*)A, (R*)qfield);
-        aa_collide_kernel<false><<<nb, kThreads, 0, s>>>(p, (P*)A, (const R*)qfield, partials, status);
+        launch_dependent(aa_moments_kernel<false>, nb, kThreads, 0, s, p, (P*)A, (R*)qfield);
+        launch_dependent(aa_collide_kernel<false>, nb, kThreads, 0, s, p, (P*)A, (const R*)qfield, partials, status);
     }
     *launches += 2;
     *nblocks = (int)nb;
@@ -2235,8 +2527,18 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
                              cudaStream_t s, bool reread, const CUtensorMap* pmap = nullptr) {
     const dim3 grid = fused_grid(p);
     if constexpr (DD == 2) {
-        if (reread || p.tile2d) {   // the tile kernel: one 32 x kTY2 tile per CTA, no march
-            fused2d_kernel<kTY2, CAL><<<tile2d_grid(p), dim3(TX, kTY2), 0, s>>>(p, (const P*)src, (P*)dst, partials,
+        if (!reread && p.sched == kSchedRow) {
+#if ELBM_ST == 0 && ELBM_D == 2
+            auto kern = p.has_fixed ? fused2d_split_kernel<CAL, true> : fused2d_split_kernel<CAL, false>;
+            constexpr int threads = 128;
+#else
+            auto kern = p.has_fixed ? fused2d_row_kernel<CAL, true> : fused2d_row_kernel<CAL, false>;
+            constexpr int threads = 32;
+#endif
+            return launch_dependent(kern, dim3((unsigned)row_strips(p)), dim3(threads), 0, s, p, (const P*)src, (P*)dst,
+                                    (p.nx + kRowW - 1) / kRowW, partials, status);
+        } else if (reread || p.sched == kSchedTile) {   // the tile kernel: one 32 x kTY2 tile per CTA, no march
+            launch_dependent(fused2d_kernel<kTY2, CAL>, tile2d_grid(p), dim3(TX, kTY2), 0, s, p, (const P*)src, (P*)dst, partials,
                                                                                status);
         } else {
             auto kern = p.has_fixed ? march2d_kernel<kW2L, kNBM, CAL, true> : march2d_kernel<kW2L, kNBM, CAL, false>;
@@ -2244,7 +2546,8 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
                                                  (int)MarchCfgL::smem_bytes);
             if (e != cudaSuccess) return e;
             DirPlanes pl = dir_planes(p, src, dst);
-            kern<<<grid, kW2L, MarchCfgL::smem_bytes, s>>>(p, pl, (const P*)src, partials, status);
+            e = launch_dependent(kern, dim3(grid), kW2L, MarchCfgL::smem_bytes, s, p, pl, (const P*)src, partials, status);
+            if (e != cudaSuccess) return e;
         }
     } else {
         bool launched = false;
@@ -2259,13 +2562,14 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
                 DirPlanes pl = dir_planes(p, src, dst);
                 CUtensorMap none;
                 std::memset(&none, 0, sizeof(none));
-                kern<<<grid, dim3(TX, kTYP), PipeCfg::smem_bytes, s>>>(p, pl, (const P*)src, partials, status,
+                e = launch_dependent(kern, dim3(grid), dim3(TX, kTYP), PipeCfg::smem_bytes, s, p, pl, (const P*)src, partials, status,
                                                                        pmap ? *pmap : none, pmap ? kPref : 0);
+            if (e != cudaSuccess) return e;
                 launched = true;
             }
         }
         if (!launched)
-            fused3d_reread_kernel<kTY3, CAL><<<grid3_ty3(p), dim3(TX, kTY3), 0, s>>>(p, (const P*)src, (P*)dst, partials,
+            launch_dependent(fused3d_reread_kernel<kTY3, CAL>, grid3_ty3(p), dim3(TX, kTY3), 0, s, p, (const P*)src, (P*)dst, partials,
                                                                               status);
     }
     return cudaGetLastError();
@@ -2280,7 +2584,8 @@ cudaError_t launch_tma_cal(const KParams& p, const void* src, void* dst, const C
                                              (int)TmaCfg::smem_bytes);
         if (e != cudaSuccess) return e;
         DirPlanes pl = dir_planes(p, src, dst);
-        kern<<<grid3_ty3(p), dim3(TX, kTY3), TmaCfg::smem_bytes, s>>>(p, pl, *map, (const P*)src, partials, status);
+        e = launch_dependent(kern, dim3(grid3_ty3(p)), dim3(TX, kTY3), TmaCfg::smem_bytes, s, p, pl, *map, (const P*)src, partials, status);
+            if (e != cudaSuccess) return e;
         return cudaGetLastError();
     } else {
         return cudaErrorInvalidValue;
@@ -2306,7 +2611,9 @@ cudaError_t launch_fused(const KParams& p, const void* src, void* dst, double* p
     const cudaError_t e = p.eos ? launch_fused_cal<DD, true>(p, src, dst, partials, status, s, reread, pmap)
                                 : launch_fused_cal<DD, false>(p, src, dst, partials, status, s, reread, pmap);
     ++*launches;
-    const dim3 grid = DD == 2 ? ((reread || p.tile2d) ? tile2d_grid(p) : fused_grid(p))
+    const dim3 grid = DD == 2 ? (!reread && p.sched == kSchedRow ? dim3((unsigned)row_strips(p), 1, 1)
+                                 : (reread || p.sched == kSchedTile)   ? tile2d_grid(p)
+                                                          : fused_grid(p))
                               : ((reread && kPipe) ? grid3_ty3(p) : fused_grid(p));
     *nblocks = (int)(grid.x * grid.y * grid.z);
     return e;
@@ -2336,7 +2643,8 @@ cudaError_t launch_ensemble_march(const EnsembleArgs& a, const void* src, void* 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)MarchCfg::smem_bytes);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kW2, MarchCfg::smem_bytes, s>>>(a, (const P*)src, (P*)dst, seg, status);
+    e = launch_dependent(kern, dim3(grid), kW2, MarchCfg::smem_bytes, s, a, (const P*)src, (P*)dst, seg, status);
+            if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -2352,15 +2660,15 @@ cudaError_t launch_ensemble(const EnsembleArgs& a, const void* src, void* dst, i
                              : launch_ensemble_march<false>(a, src, dst, status, ty, grid, s);
         }
         if (a.caloric) {
-            if (ty == 4) ensemble2d_kernel<4, true><<<grid, dim3(TX, 4), 0, s>>>(a, (const P*)src, (P*)dst, status);
+            if (ty == 4) launch_dependent(ensemble2d_kernel<4, true>, grid, dim3(TX, 4), 0, s, a, (const P*)src, (P*)dst, status);
             else if (ty == 16)
-                ensemble2d_kernel<16, true><<<grid, dim3(TX, 16), 0, s>>>(a, (const P*)src, (P*)dst, status);
-            else ensemble2d_kernel<8, true><<<grid, dim3(TX, 8), 0, s>>>(a, (const P*)src, (P*)dst, status);
+                launch_dependent(ensemble2d_kernel<16, true>, grid, dim3(TX, 16), 0, s, a, (const P*)src, (P*)dst, status);
+            else launch_dependent(ensemble2d_kernel<8, true>, grid, dim3(TX, 8), 0, s, a, (const P*)src, (P*)dst, status);
         } else {
-            if (ty == 4) ensemble2d_kernel<4, false><<<grid, dim3(TX, 4), 0, s>>>(a, (const P*)src, (P*)dst, status);
+            if (ty == 4) launch_dependent(ensemble2d_kernel<4, false>, grid, dim3(TX, 4), 0, s, a, (const P*)src, (P*)dst, status);
             else if (ty == 16)
-                ensemble2d_kernel<16, false><<<grid, dim3(TX, 16), 0, s>>>(a, (const P*)src, (P*)dst, status);
-            else ensemble2d_kernel<8, false><<<grid, dim3(TX, 8), 0, s>>>(a, (const P*)src, (P*)dst, status);
+                launch_dependent(ensemble2d_kernel<16, false>, grid, dim3(TX, 16), 0, s, a, (const P*)src, (P*)dst, status);
+            else launch_dependent(ensemble2d_kernel<8, false>, grid, dim3(TX, 8), 0, s, a, (const P*)src, (P*)dst, status);
         }
         ++*launches;
         return cudaGetLastError();
@@ -2447,7 +2755,7 @@ const Ops kOps = {kD,          kST,           sizeof(P) / 2,  sizeof(R),        
                   launch_init, launch_fields, launch_twopass, launch_fused_default, launch_fused_reread,
                   launch_totals, launch_ensemble, ensemble_occupancy, launch_stats,
                   kD == 3 ? (kPipe ? kTYP : kTY3) : 1, fused_occupancy, launch_fused_tma, tma_supported, encode_tmap,
-                  launch_fused_pf, launch_init_nodes, launch_fields_nodes, launch_step_aa, kW2L, kD == 3 && !kPipe};
+                  launch_fused_pf, launch_init_nodes, launch_fields_nodes, launch_step_aa, kW2L};
 
 }  // namespace
 

@@ -33,8 +33,8 @@ struct KParams {
     double Pr, mu0, T0, mu_exp;
     int deriv;                   // 0 upwind, 1 central
     int tz;                      // segment length of the fused kernels (D3Q27: z planes, D2Q9: rows)
-    int tile2d;                  // D2Q9: the default fused schedule runs the one-tile-per-CTA kernel
-                                 // (grids whose row march would not fill the device)
+    int sched;                   // what the default fused schedule runs: 0 the marching kernel, 1 (D2Q9) one
+                                 // tile per CTA, 2 (D2Q9) one strip per CTA, 3 the two passes
     int aa;                      // layout of the store read by the diagnostics: 0 in place; AA single
                                  // store: 1 swapped at the node, 2 pushed to the neighbour
     float2 rest2[27];            // rest-state pair (f_i, g_i) of every direction, deviation stores
@@ -803,16 +803,26 @@ struct Relax<D, double, false, CAL> {
         flux(m, dq);
         init(m.rho, m.T, m.ux, m.uy, m.uz, dq, Dx, Dy, Dz, p);
     }
-    __device__ __forceinline__ void init(double rho, double T, double ux, double uy, double uz, const double dq[3],
-                                         double Dx, double Dy, double Dz, const KParams& p) {
+    // k = (2 - w)/(2 rho w), 1 - w, 1 - w1, the density factors of f^ex and g^eq (w and w1 times
+    // rho over the scale of the doubled factors) and (w - w1)/2
+    static __device__ __forceinline__ void rates(double rho, double T, const KParams& p, double& k, double& omw,
+                                                 double& omw1, double& wr, double& w1r, double& h) {
         double mu = p.mu0;
         if (p.powlaw) mu *= pow_pos(T * p.d_invT0, p.mu_exp);
         const double P = rho * T, PrP = p.Pr * P;
         const double t = P * recip(fma(2.0, mu, P)), t1 = PrP * recip(fma(2.0, mu, PrP));   // w/2, w1/2
-        const double k = mu * recip(rho * P);
+        k = mu * recip(rho * P);
         omw = fma(-2.0, t, 1.0);
         omw1 = fma(-2.0, t1, 1.0);
-        const double rs = (D == 3 ? 0.25 : 0.5) * rho, wr = t * rs, w1r = t1 * rs;
+        const double rs = (D == 3 ? 0.25 : 0.5) * rho;
+        wr = t * rs;
+        w1r = t1 * rs;
+        h = t - t1;
+    }
+    __device__ __forceinline__ void init(double rho, double T, double ux, double uy, double uz, const double dq[3],
+                                         double Dx, double Dy, double Dz, const KParams& p) {
+        double k, wr, w1r, h;
+        rates(rho, T, p, k, omw, omw1, wr, w1r, h);
         const double T25 = 2.5 * T, TT = T * T;
         double Y[3], sx[3], gy[3], sy[3];
         axis(ux, T, T25, TT, k, Dx, X, gx, sx);
@@ -828,7 +838,6 @@ struct Relax<D, double, false, CAL> {
             A[a] = w1r * gy[a];
             B[a] = w1r * sy[a];
         }
-        const double h = t - t1;
         hq[0] = h * fma(ux, 0.5 * Dx, dq[0]);
         hq[1] = h * fma(uy, 0.5 * Dy, dq[1]);
         hq[2] = D == 3 ? h * fma(uz, 0.5 * Dz, dq[2]) : 0.0;
@@ -839,6 +848,9 @@ struct Relax<D, double, false, CAL> {
         const double u2 = u * u, P = T + u2;
         phi2(u, fma(k, Da, P), F);
         phi2(u, P, phi);
+        psi2(u, u2, T, T25, TT, ps);
+    }
+    static __device__ __forceinline__ void psi2(double u, double u2, double T, double T25, double TT, double ps[3]) {
         const double o = u * fma(0.5, u2, T), s = fma(u2, fma(0.5, u2, T25), TT);
         ps[0] = s - o;
         ps[1] = fma(-2.0, s, u2);

@@ -1,0 +1,73 @@
+"""GPU tests of what the default schedule runs on small D2Q9 grids and of the rule that chooses
+it: one strip of 30 nodes per CTA (FP64: its arithmetic shared by four warps), tiles, short row
+segments and the FP64 two passes, at the sizes where a strip is full, one node short or one
+node over, and in every option of the collision.  Bounds as in test_gpu_parity.py."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2102_09512_gb300 import cases as C
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"f64": 1e-12, "f32": 1e-5, "f16dev": 1e-3, "bf16dev": 8e-3}
+U0 = (0.09, -0.07, 0.0)
+
+
+@pytest.fixture(scope="module")
+def E():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2102_09512_gb300 import build as B
+    B.build()
+    O.build()
+    from paper_2102_09512_gb300 import elbm
+    return elbm
+
+
+def rel_l2(a, b):
+    return float(np.linalg.norm(np.ravel(a) - np.ravel(b)) / np.linalg.norm(np.ravel(b)))
+
+
+def case(nx, ny, bc, cv=None, mu_exp=0.0):
+    c = C.random_smooth(2, nx, ny, 1, seed=171 + nx, mu0=0.01, mu_exp=mu_exp, du=0.05, u0=U0, bc=bc)
+    c.fixed = (1.0, U0[0], U0[1], 0.0, 0.15)
+    c.cv = cv
+    return c
+
+
+def check(E, c, store, steps, deriv=0, kernel=0):
+    s = O.init(O.Params(D=2, nx=c.nx, ny=c.ny, nz=1, gamma=c.gamma, Pr=c.Pr, mu0=c.mu0, T0=c.T0, mu_exp=c.mu_exp, bc=c.bc,
+                        fixed=c.fixed, cv=c.cv, deriv=deriv), c.rho, c.u, c.T)
+    O.step(s, steps)
+    g = E.Solver.from_case(c, store=store, deriv=deriv)
+    g.set_kernel(kernel)
+    g.step(steps)
+    for a, b in zip(g.fields(), O.fields(s)):
+        assert rel_l2(a, b) <= TOL[store], (store, c.nx, c.ny, c.bc)
+    if store in ("f64", "f32"):   # the 16-bit stores round the state after its totals were taken
+        t, ref = g.step_totals(), g.conservation()
+        assert np.allclose(t, ref, rtol=0, atol=(1e-13 if store == "f64" else 2e-6) * abs(ref[0]))
+    g.close()
+
+
+@pytest.mark.parametrize("store", list(TOL))
+@pytest.mark.parametrize("bc", [(0,) * 6, (1, 1, 1, 1, 0, 0), (2, 1, 0, 0, 0, 0), (2, 1, 2, 1, 0, 0)])
+@pytest.mark.parametrize("nx,ny", [(1, 5), (2, 1), (29, 4), (30, 3), (31, 2), (60, 5), (91, 1)])
+def test_strips(E, nx, ny, bc, store):
+    check(E, case(nx, ny, bc), store, 25)
+
+
+@pytest.mark.parametrize("store", ["f64", "f32"])
+@pytest.mark.parametrize("deriv,cv,mu_exp", [(1, None, 0.0), (0, (1.0, 4.0, -4.0, 5.0), 0.0), (0, None, 0.76)])
+def test_strip_options(E, store, deriv, cv, mu_exp):
+    check(E, case(47, 6, (1, 1, 0, 0, 0, 0), cv, mu_exp), store, 25, deriv)
+
+
+@pytest.mark.parametrize("store", ["f64", "f32", "f16dev"])
+@pytest.mark.parametrize("nx,ny", [(150, 200), (180, 203), (608, 256), (616, 257), (700, 333)])
+@pytest.mark.parametrize("kernel", [0, 1])
+def test_sizes_around_the_rule(E, nx, ny, store, kernel):
+    """Strip and tile counts on either side of the rule's limits, and just above them, where
+    the march runs segments of a few rows and FP64 its two passes."""
+    check(E, case(nx, ny, (0,) * 6 if nx % 2 else (1, 1, 0, 0, 0, 0)), store, 6, kernel=kernel)
