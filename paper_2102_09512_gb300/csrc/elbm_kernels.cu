@@ -29,6 +29,7 @@
 
 #include "elbm_internal.h"
 #include "elbm_node.cuh"
+#include "elbm_pair.cuh"
 
 #ifndef ELBM_D
 #error "ELBM_D must be defined (2 or 3)"
@@ -2218,6 +2219,238 @@ __device__ __forceinline__ void march2d_segment(const KParams& p, const PL& pl, 
     __syncthreads();   // the shared buffers are reused by the next segment of a persistent CTA
 }
 
+// The same march for the 16-bit stores, which instruction issue bounds (615 instructions a
+// node): a thread has the nodes x0 + 2t and x0 + 2t + 1, their arithmetic as two-lane FP32
+// instructions (elbm_pair.cuh).  Both nodes' pairs lie side by side in a row buffer ([direction]
+// [slot], slots 2t and 2t + 1, W and W + 1 the strip's ends), so one 8-byte access takes them out;
+// where the stores' rows start on 8-byte boundaries (nx even) one 8-byte copy brings those of
+// c_x = 0 in and one 8-byte store writes both.
+#if ELBM_ST >= 2 && ELBM_D == 2
+template <int W>
+struct MarchPair {
+    static constexpr int NT = W / 2, NS = W + 2, QW = W + 4;   // Q~_xxx: the strip from column 2 on, its ends beside it
+    static constexpr size_t buf_bytes = ((size_t)2 * Q * NS * sizeof(P) + 15) / 16 * 16;
+    static constexpr size_t smem_bytes = buf_bytes + (size_t)2 * QW * sizeof(float);
+};
+template <int W, bool CAL, bool FIX, class PL>
+__device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL& pl, int x0, int y0, int ye,
+                                                     unsigned char* smem, float2 acc[4], bool& bad) {
+    using MC = MarchPair<W>;
+    constexpr int NS = MC::NS, QW = MC::QW;
+    P* buf = reinterpret_cast<P*>(smem);                            // [2][Q][NS]
+    float* qxs = reinterpret_cast<float*>(smem + MC::buf_bytes);    // [2][QW]
+    const int t = threadIdx.x, x = x0 + 2 * t;
+    const bool act0 = x < p.nx, act1 = x + 1 < p.nx;
+    const int xl = min(x0 + W, p.nx) - 1 - x0;   // last local column of the strip
+    // rows of both stores on 8-byte boundaries
+    const bool even = p.nx % 2 == 0 &&
+                      ((reinterpret_cast<unsigned long long>(pl.s(0)) | reinterpret_cast<unsigned long long>(pl.d(0))) & 7) == 0;
+    const bool has_halo = t < 2;
+    const int hux = t == 0 ? x0 - 1 : x0 + xl + 1, hx = map_axis(hux, p.nx, p.per_x);
+    const bool fixed_faces = FIX && p.has_fixed;
+    const bool hfixed = has_halo && fixed_faces && beyond_fixed(p, 0, hux, p.nx);
+    const int xm = map_axis(x - 1, p.nx, p.per_x), xp = map_axis(x + 1, p.nx, p.per_x);
+    const int xq = act1 ? map_axis(x + 2, p.nx, p.per_x) : 0;
+
+    auto issue_row = [&](int yq, int sb, bool with_halo) {   // yq already mapped
+        P* bb = buf + (size_t)sb * Q * NS;
+        const int row[3] = {p.nx * map_axis(yq + 1, p.ny, p.per_y), p.nx * yq, p.nx * map_axis(yq - 1, p.ny, p.per_y)};
+        if (act0) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const int a = i % 3;
+                const unsigned r = (unsigned)row[i / 3];
+                P* d = bb + i * NS + 2 * t;
+                const P* s = pl.s(i);
+                if (a == 1 && even) {
+                    cp_async<8>(d, s + (r + (unsigned)x));
+                } else {
+                    cp_async<4>(d, s + (r + (unsigned)(a == 0 ? xp : a == 1 ? x : xm)));
+                    if (act1) cp_async<4>(d + 1, s + (r + (unsigned)(a == 0 ? xq : a == 1 ? x + 1 : x)));
+                }
+            }
+        }
+        if (with_halo && has_halo && !hfixed) {
+            PullRows r;
+            pull_rows(p, hx, yq, 0, r);
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                cp_async<4>(bb + i * NS + W + t, pl.s(i) + (unsigned)(r.row[(i / 3) % 3][1] + r.xs[i % 3]));
+        }
+        cp_async_commit();
+    };
+    // stored pairs of one node with the fixed state's in place of those marked in gm
+    auto node_fixed = [&](const P* v, int stride, unsigned gm, Moments<float>& m) {
+        float f[Q], g[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            Cd::dec(v[i * stride], f[i], g[i]);
+            if ((gm >> i) & 1u) fixed_pair(p, i, f[i], g[i]);
+        }
+        node_moments<kD, float, true, true, CAL>(f, g, p, m);
+    };
+    auto pair_moments = [&](int sb, int y, MomentsPair& m) {
+        const P* bb = buf + (size_t)sb * Q * NS + 2 * t;
+        if (FIX) {
+            const unsigned g0 = fixed_mask<FIX>(p, x, y), g1 = fixed_mask<FIX>(p, x + 1, y);
+            if (g0 | g1) {
+                Moments<float> a, b;
+                node_fixed(bb, NS, g0, a);
+                node_fixed(bb + 1, NS, g1, b);
+                m.rho = make_float2(a.rho, b.rho);
+                m.ux = make_float2(a.ux, b.ux);
+                m.uy = make_float2(a.uy, b.uy);
+                m.T = make_float2(a.T, b.T);
+                m.rE = make_float2(a.rE, b.rE);
+                m.Pxx = make_float2(a.Pxx, b.Pxx);
+                m.Pyy = make_float2(a.Pyy, b.Pyy);
+                m.Pxy = make_float2(a.Pxy, b.Pxy);
+                return;
+            }
+        }
+        uint2 raw[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) raw[i] = *reinterpret_cast<const uint2*>(bb + i * NS);
+        node_moments_pair<kD, kST, CAL>(
+            [&](int i, int k) { return *reinterpret_cast<const P*>(k ? &raw[i].y : &raw[i].x); }, p, m);
+    };
+    auto halo_q = [&](int sb, int y) {
+        if (hfixed) return fixed_Q(p, 0);
+        const P* bb = buf + (size_t)sb * Q * NS + W + t;
+        Moments<float> m;
+        const unsigned gm = fixed_mask<FIX>(p, hx, y);
+        if (FIX && gm) node_fixed(bb, NS, gm, m);
+        else node_moments_stored<kD, kST, false, CAL>([&](int i) { return bb[i * NS]; }, p, m);
+        return anomaly(m.rho, m.ux, m.T);
+    };
+    float* const my_qx = qxs + 2 + 2 * t;
+    float* const halo_qx = qxs + (t == 0 ? 1 : xl + 3);
+    // Q~ of this thread's nodes: xxx to shared memory row b, yyy returned
+    auto put_q = [&](int b, const MomentsPair& m, bool x_too) {
+        const float2 c = anomaly_c(m.T);
+        if (x_too) {
+            const float2 v = anomaly2(m.rho, m.ux, c);
+            if (act1) *reinterpret_cast<float2*>(my_qx + b * QW) = v;
+            else my_qx[b * QW] = v.x;
+        }
+        return anomaly2(m.rho, m.uy, c);
+    };
+
+    float2 qy_prev = both(0.f), qy_cur = both(0.f), qy_next = both(0.f);
+    if (act0) {
+        if (fixed_faces && beyond_fixed(p, 1, y0 - 1, p.ny)) {
+            qy_prev = both(fixed_Q(p, 1));
+        } else {
+            const int yd = map_axis(y0 - 1, p.ny, p.per_y);
+            qy_prev.x = direct_anomaly_y<CAL>(p, pl.base, x, yd);
+            if (act1) qy_prev.y = direct_anomaly_y<CAL>(p, pl.base, x + 1, yd);
+        }
+    }
+    issue_row(y0, 0, true);
+    issue_row(map_axis(y0 + 1, p.ny, p.per_y), 1, y0 + 1 < ye);
+    MomentsPair m_cur, m_next;
+    cp_async_wait_pending<1>();
+    __syncthreads();
+    if (act0) {
+        pair_moments(0, y0, m_cur);
+        qy_cur = put_q(0, m_cur, true);
+    }
+    if (has_halo) halo_qx[0] = halo_q(0, y0);
+
+    for (int y = y0; y < ye; ++y) {
+        const int bq = (y - y0) & 1, sn = bq ^ 1;   // buffers of rows y and y+1
+        const bool last = y + 1 == ye;
+        cp_async_wait_all();
+        __syncthreads();
+        uint2 pk[Q];   // the pulled pairs of row y, as stored
+        if (act0) {
+            const P* bb = buf + (size_t)bq * Q * NS + 2 * t;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) pk[i] = *reinterpret_cast<const uint2*>(bb + i * NS);
+        }
+        if (y + 2 <= ye) issue_row(map_axis(y + 2, p.ny, p.per_y), bq, y + 2 < ye);
+        const int yn = map_axis(y + 1, p.ny, p.per_y);
+        if (act0) {
+            if (fixed_faces && beyond_fixed(p, 1, y + 1, p.ny)) {
+                qy_next = both(fixed_Q(p, 1));   // the last row of the grid: nothing after it
+            } else {
+                pair_moments(sn, yn, m_next);
+                qy_next = put_q(sn, m_next, !last);
+            }
+        }
+        if (!last && has_halo) halo_qx[sn * QW] = halo_q(sn, yn);
+        if (act0) {
+            auto bad_lane = [](float rho, float T, float ux, float uy) {
+                return !(rho > 0.f) || !(T > 0.f) || !isfinite(rho) || !isfinite(T) || !isfinite(ux) || !isfinite(uy);
+            };
+            bad |= bad_lane(m_cur.rho.x, m_cur.T.x, m_cur.ux.x, m_cur.uy.x) ||
+                   (act1 && bad_lane(m_cur.rho.y, m_cur.T.y, m_cur.ux.y, m_cur.uy.y));
+            const float* qx = my_qx + bq * QW;
+            const float2 q0 = *reinterpret_cast<const float2*>(qx);
+            const float2 Dx = dQ2(p.deriv, m_cur.ux, make_float2(qx[-1], q0.x), q0, make_float2(q0.y, qx[2]));
+            const float2 Dy = dQ2(p.deriv, m_cur.uy, qy_prev, qy_cur, qy_next);
+            acc[0] = add2(acc[0], m_cur.rho);
+            acc[1] = fma2(m_cur.rho, m_cur.ux, acc[1]);
+            acc[2] = fma2(m_cur.rho, m_cur.uy, acc[2]);
+            acc[3] = add2(acc[3], m_cur.rE);
+            RelaxPair<kD, CAL> rx;
+            rx.init(m_cur, Dx, Dy, both(0.f), p);
+            const unsigned n = (unsigned)(x + p.nx * y);
+            const unsigned g0 = fixed_mask<FIX>(p, x, y), g1 = fixed_mask<FIX>(p, x + 1, y);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                float2 f, g;
+                Cd::dec(*reinterpret_cast<const P*>(&pk[i].x), f.x, g.x);
+                Cd::dec(*reinterpret_cast<const P*>(&pk[i].y), f.y, g.y);
+                if ((g0 >> i) & 1u) fixed_pair(p, i, f.x, g.x);
+                if ((g1 >> i) & 1u) fixed_pair(p, i, f.y, g.y);
+                f = rx.f(i, f);
+                g = rx.g(i, g);
+                const P o0 = Cd::enc(f.x, g.x), o1 = Cd::enc(f.y, g.y);
+                P* d = pl.d(i) + n;
+                if (even) {
+                    uint2 o;
+                    o.x = *reinterpret_cast<const unsigned*>(&o0);
+                    o.y = *reinterpret_cast<const unsigned*>(&o1);
+                    *reinterpret_cast<uint2*>(d) = o;
+                } else {
+                    d[0] = o0;
+                    if (act1) d[1] = o1;
+                }
+            }
+        }
+        m_cur = m_next;
+        qy_prev = qy_cur;
+        qy_cur = qy_next;
+    }
+    cp_async_wait_all();
+    __syncthreads();   // the shared buffers are reused by the next segment of a persistent CTA
+}
+// Sixteen warps of 128 registers per SM (uncapped 145 registers, twelve warps: 4096^2 272 us a
+// step, twenty warps: 598, it spills).  4096^2, FP16: 301 us with a node a thread, 249 with two;
+// strips of 128 nodes 269, 512 nodes 253.
+template <int W> constexpr int kPairCtas = 1024 / W;
+template <int W, bool CAL, bool FIX>
+__global__ void __launch_bounds__(W / 2, kPairCtas<W>)
+march2d_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* __restrict__ src,
+                    double* __restrict__ partials, int* __restrict__ status) {
+    extern __shared__ __align__(16) unsigned char march_smem[];
+    wait_for_previous();
+    const int x0 = blockIdx.x * W, y0 = blockIdx.y * p.tz, ye = min(y0 + p.tz, p.ny);
+    float2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = both(0.f);
+    bool bad = false;
+    march2d_pair_segment<W, CAL, FIX>(p, PlanesParam{&pl, src}, x0, y0, ye, march_smem, acc, bad);
+    launch_dependents();
+    flag_if(bad, status);
+    const bool act1 = x0 + 2 * (int)threadIdx.x + 1 < p.nx;
+    auto lanes = [&](float2 a) { return act1 ? a.x + a.y : a.x; };
+    float tot[5] = {lanes(acc[0]), lanes(acc[1]), lanes(acc[2]), 0.f, lanes(acc[3])};
+    block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * blockIdx.y));
+}
+#endif
+
 // One lattice: CTA (bx, by) marches strip bx over rows [by * p.tz, min((by + 1) * p.tz, ny)).
 #ifndef ELBM_MARCH_MINB
 #define ELBM_MARCH_MINB 0
@@ -2248,20 +2481,34 @@ march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
 // Persistent ensemble step on the row march: the work list holds (instance, strip, segment)
 // units (instance k owns units [tile_start[k], tile_start[k+1]), tiles_x[k] strips per
 // segment row); CTA b takes units b, b + gridDim.x, ...  No totals are kept.
+// Threads and shared memory of a march CTA: two nodes a thread for the 16-bit stores.
+#if ELBM_ST >= 2 && ELBM_D == 2
+template <int W, int NB> constexpr int march_threads = W / 2;
+template <int W, int NB> constexpr int march_min_ctas = kPairCtas<W>;
+template <int W, int NB> constexpr size_t march_smem_bytes = MarchPair<W>::smem_bytes;
+#else
+template <int W, int NB> constexpr int march_threads = W;
+template <int W, int NB> constexpr int march_min_ctas = 1;
+template <int W, int NB> constexpr size_t march_smem_bytes = March2<W, NB>::smem_bytes;
+#endif
 template <int W, int NB, bool CAL>
-__global__ void __launch_bounds__(W)
+__global__ void __launch_bounds__(march_threads<W, NB>, march_min_ctas<W, NB>)
 ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int seg,
                         int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
     wait_for_previous();
     __shared__ int s_start[kMaxEnsemble + 1];
     __shared__ int s_tx[kMaxEnsemble];
-    for (int k = threadIdx.x; k <= a.n; k += W) s_start[k] = a.tile_start[k];
-    for (int k = threadIdx.x; k < a.n; k += W) s_tx[k] = a.tiles_x[k];
+    for (int k = threadIdx.x; k <= a.n; k += blockDim.x) s_start[k] = a.tile_start[k];
+    for (int k = threadIdx.x; k < a.n; k += blockDim.x) s_tx[k] = a.tiles_x[k];
     __syncthreads();
     bool bad = false;
+#if ELBM_ST >= 2 && ELBM_D == 2
+    float2 acc[4] = {};
+#else
     Acc5 acc;
     acc.zero();
+#endif
     int k = 0;
     for (int u = blockIdx.x; u < a.ntiles; u += gridDim.x) {
         while (u >= s_start[k + 1]) ++k;   // u increases, so k only moves forward
@@ -2270,8 +2517,12 @@ ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __re
         const KParams& p = a.params[k];
         const long long off = a.offset[k];
         const int y0 = by * seg;
-        march2d_segment<W, NB, CAL, true>(p, PlanesBase{src + off, dst + off, (size_t)p.N, src + off}, bx * W, y0,
-                                min(y0 + seg, p.ny), march_smem, acc, bad);
+        const PlanesBase pl{src + off, dst + off, (size_t)p.N, src + off};
+#if ELBM_ST >= 2 && ELBM_D == 2
+        march2d_pair_segment<W, CAL, true>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
+#else
+        march2d_segment<W, NB, CAL, true>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
+#endif
     }
     launch_dependents();
     flag_if(bad, status);
@@ -2303,16 +2554,13 @@ constexpr int kW2 = kMarchW2;            // D2Q9 row march: strips of kW2 nodes
 #define ELBM_MARCH_NB 2
 #endif
 constexpr int kNBM = ELBM_MARCH_NB;      // row buffers of the march (2: one row in flight, 3: two)
-using MarchCfg = March2<kW2, kNBM>;
 // Strip width of the single-lattice D2Q9 march: 256 nodes for the 16-bit stores, whose
-// march is issue-bound and pays for the strip's two halo nodes half as often per node
-// (FP16 at 4096^2: 52.8 -> 55.2 GLUPS), kW2 for FP32 and FP64, which are bandwidth-bound
+// march is issue-bound and pays for the strip's two halo nodes half as often per node, kW2 for FP32 and FP64, which are bandwidth-bound
 // (256 measured 39.2 against 44.9 GLUPS in FP32).  The persistent ensemble keeps kW2.
 #ifndef ELBM_MARCH_W16
 #define ELBM_MARCH_W16 256
 #endif
 constexpr int kW2L = sizeof(P) == 4 ? ELBM_MARCH_W16 : kW2;
-using MarchCfgL = March2<kW2L, kNBM>;
 #ifndef ELBM_TY3
 #define ELBM_TY3 8
 #endif
@@ -2522,6 +2770,17 @@ cudaError_t launch_twopass(const KParams& p, const void* src, void* dst, void* q
 #endif
 constexpr int kPref = ELBM_PREF;   // planes of L2 prefetch ahead of the cp.async copies (with a tensor map)
 
+// The row march of this store for grid p (D2Q9).
+template <int DD, bool CAL>
+auto march_kernel(const KParams& p) {
+    static_assert(DD == 2, "D2Q9");
+#if ELBM_ST >= 2 && ELBM_D == 2
+    return p.has_fixed ? march2d_pair_kernel<kW2L, CAL, true> : march2d_pair_kernel<kW2L, CAL, false>;
+#else
+    return p.has_fixed ? march2d_kernel<kW2L, kNBM, CAL, true> : march2d_kernel<kW2L, kNBM, CAL, false>;
+#endif
+}
+
 template <int DD, bool CAL>
 cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, double* partials, int* status,
                              cudaStream_t s, bool reread, const CUtensorMap* pmap = nullptr) {
@@ -2541,12 +2800,12 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
             launch_dependent(fused2d_kernel<kTY2, CAL>, tile2d_grid(p), dim3(TX, kTY2), 0, s, p, (const P*)src, (P*)dst, partials,
                                                                                status);
         } else {
-            auto kern = p.has_fixed ? march2d_kernel<kW2L, kNBM, CAL, true> : march2d_kernel<kW2L, kNBM, CAL, false>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)MarchCfgL::smem_bytes);
+            auto kern = march_kernel<DD, CAL>(p);
+            constexpr size_t smem = march_smem_bytes<kW2L, kNBM>;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             DirPlanes pl = dir_planes(p, src, dst);
-            e = launch_dependent(kern, dim3(grid), kW2L, MarchCfgL::smem_bytes, s, p, pl, (const P*)src, partials, status);
+            e = launch_dependent(kern, dim3(grid), march_threads<kW2L, kNBM>, smem, s, p, pl, (const P*)src, partials, status);
             if (e != cudaSuccess) return e;
         }
     } else {
@@ -2640,10 +2899,10 @@ template <bool CAL>
 cudaError_t launch_ensemble_march(const EnsembleArgs& a, const void* src, void* dst, int* status, int seg, int grid,
                                   cudaStream_t s) {
     auto kern = ensemble_march2d_kernel<kW2, kNBM, CAL>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)MarchCfg::smem_bytes);
+    constexpr size_t smem = march_smem_bytes<kW2, kNBM>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_dependent(kern, dim3(grid), kW2, MarchCfg::smem_bytes, s, a, (const P*)src, (P*)dst, seg, status);
+    e = launch_dependent(kern, dim3(grid), march_threads<kW2, kNBM>, smem, s, a, (const P*)src, (P*)dst, seg, status);
             if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -2685,9 +2944,9 @@ int ensemble_occupancy(int ty) {
         cudaError_t e;
         if (ty > 16) {
             auto kern = ensemble_march2d_kernel<kW2, kNBM, false>;
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg::smem_bytes) !=
-                    cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kW2, MarchCfg::smem_bytes) != cudaSuccess)
+            constexpr size_t smem = march_smem_bytes<kW2, kNBM>;
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, march_threads<kW2, kNBM>, smem) != cudaSuccess)
                 return 0;
             return nb;
         }
@@ -2741,10 +3000,10 @@ int fused_occupancy_impl(const KParams& p) {
             cudaSuccess)
             return 0;
     } else {
-        auto kern = p.has_fixed ? march2d_kernel<kW2L, kNBM, false, true> : march2d_kernel<kW2L, kNBM, false, false>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfgL::smem_bytes) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kW2L, MarchCfgL::smem_bytes) != cudaSuccess)
+        auto kern = march_kernel<DD, false>(p);
+        constexpr size_t smem = march_smem_bytes<kW2L, kNBM>;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, march_threads<kW2L, kNBM>, smem) != cudaSuccess)
             return 0;
     }
     return n;

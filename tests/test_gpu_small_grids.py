@@ -71,3 +71,22 @@ def test_sizes_around_the_rule(E, nx, ny, store, kernel):
     """Strip and tile counts on either side of the rule's limits, and just above them, where
     the march runs segments of a few rows and FP64 its two passes."""
     check(E, case(nx, ny, (0,) * 6 if nx % 2 else (1, 1, 0, 0, 0, 0)), store, 6, kernel=kernel)
+
+
+@pytest.mark.parametrize("store", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("bc", [(0,) * 6, (1, 1, 1, 1, 0, 0), (2, 1, 2, 1, 0, 0)])
+@pytest.mark.parametrize("nx,ny,tz", [(257, 40, 7), (512, 33, 16), (255, 9, 1), (6, 30, 10), (1, 12, 5), (770, 21, None)])
+def test_row_march(E, nx, ny, tz, bc, store):
+    """The row march (two nodes a thread for the 16-bit stores) forced on strips that end on a
+    pair, between the nodes of one and one node over, with rows on and off 8-byte boundaries and
+    fixed faces, and segments of one row."""
+    c = case(nx, ny, bc)
+    s = O.init(O.Params(D=2, nx=nx, ny=ny, nz=1, gamma=c.gamma, Pr=c.Pr, mu0=c.mu0, T0=c.T0, mu_exp=0.0, bc=bc,
+                        fixed=c.fixed), c.rho, c.u, c.T)
+    O.step(s, 20)
+    g = E.Solver.from_case(c, store=store)
+    g.set_tile_z(ny if tz is None else tz)
+    g.step(20)
+    for a, b in zip(g.fields(), O.fields(s)):
+        assert rel_l2(a, b) <= TOL[store], (store, nx, ny, bc)
+    g.close()
