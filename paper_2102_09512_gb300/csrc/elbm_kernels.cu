@@ -1408,13 +1408,6 @@ struct PipeBytes {
     static constexpr size_t value = Pipe<TY, NB>::smem_bytes;
 };
 
-// The collision's per-direction updates of f and g as one two-lane FP32 operation (FFMA2):
-// FP16 19.9 -> 20.4 GLUPS at 256^3, FP32 unchanged (the same results bit for bit).
-#ifndef ELBM_FFMA2
-#define ELBM_FFMA2 1
-#endif
-constexpr bool kFFMA2 = ELBM_FFMA2;
-
 // Store of a post-collision pair.  With ELBM_STCS the store is marked streaming (evict
 // first), so that the step's writes do not push the planes prefetched ahead out of L2.
 #ifndef ELBM_STCS
@@ -1594,18 +1587,21 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
             node_totals(m_cur, m_cur.rE, v);
             acc.add(v);
             // collide and store pair by pair, decoding each just before its update
-            Relax<kD, R, DEV, CAL> rx;
-            rx.init(m_cur, Dx, Dy, Dz, p);
             const unsigned n = (unsigned)node_index(p, x, y, z);
+            if constexpr (DEV) {
+                RelaxDev<CAL> rx;
+                rx.init(m_cur, Dx, Dy, Dz, p);
+                rx.apply([&](int i, R& f, R& g) { Cd::dec(pk[i], f, g); },
+                         [&](int i, R f, R g) { store_pair(pl.dst[i] + n, Cd::enc(f, g)); });
+            } else {
+                Relax<kD, R, DEV, CAL> rx;
+                rx.init(m_cur, Dx, Dy, Dz, p);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                R f, g;
-                Cd::dec(pk[i], f, g);
-                if constexpr (kFFMA2) {
+                for (int i = 0; i < Q; ++i) {
+                    R f, g;
+                    Cd::dec(pk[i], f, g);
                     const float2 o = rx.fg(i, make_float2(f, g), p);
                     store_pair(pl.dst[i] + n, Cd::enc(o.x, o.y));
-                } else {
-                    store_pair(pl.dst[i] + n, Cd::enc(rx.f(i, f, p), rx.g(i, g, p)));
                 }
             }
         }
@@ -1892,18 +1888,21 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
             R v[5];
             node_totals(m_cur, m_cur.rE, v);
             acc.add(v);
-            Relax<kD, R, DEV, CAL> rx;
-            rx.init(m_cur, Dx, Dy, Dz, p);
             const unsigned n = (unsigned)node_index(p, x, y, z);
+            if constexpr (DEV) {
+                RelaxDev<CAL> rx;
+                rx.init(m_cur, Dx, Dy, Dz, p);
+                rx.apply([&](int i, R& f, R& g) { Cd::dec(pk[i], f, g); },
+                         [&](int i, R f, R g) { store_pair(pl.dst[i] + n, Cd::enc(f, g)); });
+            } else {
+                Relax<kD, R, DEV, CAL> rx;
+                rx.init(m_cur, Dx, Dy, Dz, p);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                R f, g;
-                Cd::dec(pk[i], f, g);
-                if constexpr (kFFMA2) {
+                for (int i = 0; i < Q; ++i) {
+                    R f, g;
+                    Cd::dec(pk[i], f, g);
                     const float2 o = rx.fg(i, make_float2(f, g), p);
                     store_pair(pl.dst[i] + n, Cd::enc(o.x, o.y));
-                } else {
-                    store_pair(pl.dst[i] + n, Cd::enc(rx.f(i, f, p), rx.g(i, g, p)));
                 }
             }
         }
@@ -2116,12 +2115,6 @@ __device__ __forceinline__ void march2d_segment(const KParams& p, const PL& pl, 
     // fixed state's (pulled across a fixed face)
     auto row_moments = [&](int sb, int slot, unsigned gm, Moments<R>& m, auto full) {
         const P* bb = buf + (size_t)sb * Q * NS + slot;
-        if constexpr (DEV) {
-            if (!gm) {   // sums straight from the stored pairs
-                node_moments_stored<kD, kST, decltype(full)::value, CAL>([&](int i) { return bb[i * NS]; }, p, m);
-                return;
-            }
-        }
         R f[Q], g[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) Cd::dec(bb[i * NS], f[i], g[i]);
@@ -2484,15 +2477,15 @@ march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
 // Threads and shared memory of a march CTA: two nodes a thread for the 16-bit stores.
 #if ELBM_ST >= 2 && ELBM_D == 2
 template <int W, int NB> constexpr int march_threads = W / 2;
-template <int W, int NB> constexpr int march_min_ctas = kPairCtas<W>;
+#define ELBM_ENSEMBLE_BOUNDS(W) __launch_bounds__(W / 2, kPairCtas<W>)
 template <int W, int NB> constexpr size_t march_smem_bytes = MarchPair<W>::smem_bytes;
 #else
 template <int W, int NB> constexpr int march_threads = W;
-template <int W, int NB> constexpr int march_min_ctas = 1;
+#define ELBM_ENSEMBLE_BOUNDS(W) __launch_bounds__(W)
 template <int W, int NB> constexpr size_t march_smem_bytes = March2<W, NB>::smem_bytes;
 #endif
 template <int W, int NB, bool CAL>
-__global__ void __launch_bounds__(march_threads<W, NB>, march_min_ctas<W, NB>)
+__global__ void ELBM_ENSEMBLE_BOUNDS(W)
 ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int seg,
                         int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];

@@ -12,12 +12,6 @@
 
 namespace elbm {
 
-// V = float2; templates, so that host programs which include this header for another architecture
-// need not know the two-lane instructions.
-template <class V> __device__ __forceinline__ V add2(V a, V b) { return __fadd2_rn(a, b); }
-template <class V> __device__ __forceinline__ V mul2(V a, V b) { return __fmul2_rn(a, b); }
-template <class V> __device__ __forceinline__ V fma2(V a, V b, V c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 both(float c) { return make_float2(c, c); }
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(qdiv(1.f, a.x), qdiv(1.f, a.y)); }
 
 struct MomentsPair {
