@@ -96,7 +96,11 @@ struct elbm_ensemble {
         a.n = n;
         a.ntiles = tile_start[tyi][n];
         a.caloric = 0;
-        for (const KParams& k : kp) a.caloric |= k.eos;
+        a.fixed = 0;
+        for (const KParams& k : kp) {
+            a.caloric |= k.eos;
+            a.fixed |= k.has_fixed;
+        }
         return a;
     }
     void drop_graphs() {

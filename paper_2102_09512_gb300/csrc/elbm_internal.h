@@ -237,6 +237,7 @@ struct EnsembleArgs {
     const int* tiles_x;         // [n] tiles per row of instance k
     int n, ntiles;
     int caloric;                // some instance has a Cv(T) model (selects the kernel form)
+    int fixed;                  // some instance has a fixed-state face (likewise)
 };
 
 // Launchers for one (lattice, store) combination.  Each returns the first CUDA

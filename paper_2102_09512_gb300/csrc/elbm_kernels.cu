@@ -2471,6 +2471,8 @@ march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     block_sum5_warp(tot, partials + 5 * (blockIdx.x + gridDim.x * blockIdx.y));
 }
 
+// Compiled with and without fixed-state faces, as march2d_kernel (64 lattices, 8 steps: 7124 us with
+// the face tests always in, 6506 without).
 // Persistent ensemble step on the row march: the work list holds (instance, strip, segment)
 // units (instance k owns units [tile_start[k], tile_start[k+1]), tiles_x[k] strips per
 // segment row); CTA b takes units b, b + gridDim.x, ...  No totals are kept.
@@ -2484,7 +2486,7 @@ template <int W, int NB> constexpr int march_threads = W;
 #define ELBM_ENSEMBLE_BOUNDS(W) __launch_bounds__(W)
 template <int W, int NB> constexpr size_t march_smem_bytes = March2<W, NB>::smem_bytes;
 #endif
-template <int W, int NB, bool CAL>
+template <int W, int NB, bool CAL, bool FIX>
 __global__ void ELBM_ENSEMBLE_BOUNDS(W)
 ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int seg,
                         int* __restrict__ status) {
@@ -2512,9 +2514,9 @@ ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __re
         const int y0 = by * seg;
         const PlanesBase pl{src + off, dst + off, (size_t)p.N, src + off};
 #if ELBM_ST >= 2 && ELBM_D == 2
-        march2d_pair_segment<W, CAL, true>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
+        march2d_pair_segment<W, CAL, FIX>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
 #else
-        march2d_segment<W, NB, CAL, true>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
+        march2d_segment<W, NB, CAL, FIX>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
 #endif
     }
     launch_dependents();
@@ -2891,7 +2893,7 @@ cudaError_t launch_fused_pf(const KParams& p, const void* src, void* dst, const 
 template <bool CAL>
 cudaError_t launch_ensemble_march(const EnsembleArgs& a, const void* src, void* dst, int* status, int seg, int grid,
                                   cudaStream_t s) {
-    auto kern = ensemble_march2d_kernel<kW2, kNBM, CAL>;
+    auto kern = a.fixed ? ensemble_march2d_kernel<kW2, kNBM, CAL, true> : ensemble_march2d_kernel<kW2, kNBM, CAL, false>;
     constexpr size_t smem = march_smem_bytes<kW2, kNBM>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -2936,7 +2938,7 @@ int ensemble_occupancy(int ty) {
     if constexpr (kD == 2) {
         cudaError_t e;
         if (ty > 16) {
-            auto kern = ensemble_march2d_kernel<kW2, kNBM, false>;
+            auto kern = ensemble_march2d_kernel<kW2, kNBM, false, false>;
             constexpr size_t smem = march_smem_bytes<kW2, kNBM>;
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, march_threads<kW2, kNBM>, smem) != cudaSuccess)
