@@ -261,11 +261,11 @@ long long elbm_launch_count(const elbm_handle *h);
 /* Velocity c_i = (c[0], c[1], c[2]) of direction i of a lattice (Eq. d3q27vel). */
 int elbm_velocity(int lattice, int i, int c[3]);
 
-/* One time step, src -> dst, of the two-pass schedule, for callers that cannot
- * allocate device memory (for example a solver embedded in an application that owns
- * the whole device memory pool and lends the library only the populations it
- * updates).  No handle and no auxiliary buffer: the scratch this step needs (the Q~
- * field, the per-CTA partials and the status word) lives in a fixed static device
+/* One time step, src -> dst, for callers that cannot allocate device memory (for example
+ * a solver embedded in an application that owns the whole device memory pool and lends
+ * the library only the populations it updates).  Grids below 2^14 nodes run the two-pass
+ * schedule, larger ones the default schedule of a handle (results agree to rounding).  No handle and no auxiliary buffer: the scratch this step needs (the Q~
+ * field and the per-CTA partials) lives in a fixed static device
  * array of 16 MiB that every GPU loading the library holds until the process exits.
  * The paper has no counterpart; this is an interface choice of the library.
  *   params  problem statement, validated as by elbm_create;
@@ -281,9 +281,9 @@ int elbm_velocity(int lattice, int i, int c[3]);
  * it up again, so make the first call after a reset before any capture as well.
  * Calls no cudaMalloc, cudaFree or other allocating routine.  All calls share the
  * array, so calls whose kernels overlap on the GPU (different streams, or several
- * host threads) race on it; serialise them.  The status word is cleared by each
- * call and device-detected non-physical states are not reported here (read them
- * through the handle API, e.g. elbm_conservation on a bound handle). */
+ * host threads) race on it; serialise them.  Device-detected non-physical states are
+ * not reported here (read them through the handle API, e.g. elbm_conservation on a
+ * bound handle). */
 int elbm_step_noalloc(const elbm_params *params, const void *src, void *dst, void *stream);
 
 /* Frees the handle (not the caller's buffers). */

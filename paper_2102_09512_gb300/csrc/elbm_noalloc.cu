@@ -1,5 +1,5 @@
-// elbm_step_noalloc: one time step of the two-pass schedule for callers that cannot
-// allocate device memory.
+// elbm_step_noalloc: one time step for callers that cannot allocate device memory, on the
+// two-pass schedule or, from kNoallocFused nodes on, on the one-kernel schedules of a handle.
 //
 // Some callers of this library are not allowed to call cudaMalloc: a solver embedded
 // in a host application that owns the whole device memory pool and hands the library
@@ -81,6 +81,21 @@ const Ops* ops_for(int D, int store) {
     return nullptr;
 }
 
+// Grids of at least this many nodes run the default schedule of a handle (FP64 D3Q27: the two
+// passes, which are its default), which needs no Q~ field: D3Q27 FP32 96^3 71 us a step where the
+// two passes take 125, 61 x 45 x 53 18.6 and 18.8.
+constexpr long long kNoallocFused = 1LL << 14;
+
+// Resident CTAs per SM of the fused kernel a problem would run, looked up once per device (a
+// property of the compiled kernel): the query costs as much as a launch.
+int fused_per_sm(const Ops* ops, const KParams& k, int D, int store, int dev) {
+    static int known[kMaxDevices][2][4][2] = {};   // + 1; guarded by g_setup_mutex
+    std::lock_guard<std::mutex> lock(g_setup_mutex);
+    int& v = known[dev][D - 2][store][k.has_fixed ? 1 : 0];
+    if (v == 0) v = ops->fused_occupancy(k) + 1;
+    return v - 1;
+}
+
 // Device address of the scratch array on the current device: looked up on the first call
 // made on the device, and again on the first call after its context changed (a reset).
 int scratch_address(void** out) {
@@ -120,11 +135,26 @@ extern "C" int elbm_step_noalloc(const elbm_params* prm, const void* src, void* 
     if (rc != ELBM_OK) return rc;
     char* s = (char*)base;
     cudaStream_t st = (cudaStream_t)stream;
-    int* status = (int*)(s + lay.status);
-    if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return ELBM_ERR_CUDA;
+    // No status word: nothing reads it here, and clearing it would part one step's kernels from the next's.
     int nb = 0;
     long long launches = 0;
-    cudaError_t e = ops->step_twopass(k, src, dst, s + lay.qfield, (double*)(s + lay.partials), &nb, status, st,
-                                      &launches);
+    if (k.N >= kNoallocFused) {
+        int dev = -1, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return ELBM_ERR_CUDA;
+        const int per_sm = fused_per_sm(ops, k, D, p.store, dev);
+        if (D == 2) plan_d2q9(k, sms, per_sm, ops->march_width, p.store == ELBM_F64);
+        else if (p.store == ELBM_F64) k.sched = kSchedTwoPass;
+        else k.tz = choose_tz(k, ops->fused_tile_y, sms, per_sm, k.tz);
+        // the fused kernels' partials may run into the Q~ field, which they do not use
+        const size_t room = (kNoallocScratchBytes - lay.partials) / (5 * sizeof(double));
+        if (k.sched != kSchedTwoPass && (size_t)ops->max_blocks(k) <= room) {
+            const cudaError_t e = ops->step_fused(k, src, dst, (double*)(s + lay.partials), &nb, nullptr, st, &launches);
+            return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA;
+        }
+    }
+    const cudaError_t e = ops->step_twopass(k, src, dst, s + lay.qfield, (double*)(s + lay.partials), &nb, nullptr, st,
+                                            &launches);
     return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA;
 }
