@@ -303,12 +303,14 @@ __device__ __forceinline__ void cp_async_wait_pending() {
 // without it, kernels start on a raster of about 2.05 us.  Most kernels call it late, a marching
 // one when its column is done: CTAs set up beside a whole grid that is still running are
 // spread unevenly (D2Q9 724^2, FP32: 22.6 us a step without dependent launches, 34.7 with early
-// ones).
+// ones).  The pointers such a kernel reads are not const __restrict__: the compiler would load
+// through the non-coherent path, which is for data that nobody writes while the grid exists, and a
+// dependent grid exists while the one before it still writes.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void dependent_launch_point() {
-    launch_dependents();
     wait_for_previous();
+    launch_dependents();
 }
 
 // ---------------------------------------------------------------------------
@@ -680,7 +682,7 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
 // ---------------------------------------------------------------------------
 // Pass 1: Q~_aaa at every node from the pulled (post-stream) populations.
 template <bool PULL>
-__global__ void moments_kernel(const __grid_constant__ KParams p, const P* __restrict__ src,
+__global__ void moments_kernel(const __grid_constant__ KParams p, const P* src,
                                R* __restrict__ qf) {
     dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -701,8 +703,8 @@ __global__ void moments_kernel(const __grid_constant__ KParams p, const P* __res
 
 // Pass 2: pull, moments, derivative of Q~ from the field, collide, store.
 template <bool PULL>
-__global__ void collide_kernel(const __grid_constant__ KParams p, const P* __restrict__ src,
-                               P* __restrict__ dst, const R* __restrict__ qf,
+__global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
+                               P* __restrict__ dst, const R* qf,
                                double* __restrict__ partials, int* __restrict__ status) {
     dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -756,7 +758,7 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* __res
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
 __global__ void __launch_bounds__(kThreads1D)
-moments64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, R* __restrict__ qf,
+moments64_kernel(const __grid_constant__ KParams p, const P* src, R* __restrict__ qf,
                  P* __restrict__ dst, double* __restrict__ partials, int* __restrict__ status) {
     wait_for_previous();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -796,7 +798,7 @@ moments64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, R
 constexpr int kThreads64 = 128;   // second pass: smaller CTAs, so that one's loads overlap another's arithmetic
 template <bool PULL>
 __global__ void __launch_bounds__(kThreads64, 2)
-collide64_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* dst, const R* __restrict__ qf) {
+collide64_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, const R* qf) {
     wait_for_previous();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
@@ -917,7 +919,7 @@ __global__ void aa_moments_kernel(const __grid_constant__ KParams p, P* A, R* __
 constexpr int kAaMinBlocks = sizeof(R) == 4 ? 2 : 1;
 template <bool FROM_L1>
 __global__ void __launch_bounds__(kThreads1D, kAaMinBlocks)
-aa_collide_kernel(const __grid_constant__ KParams p, P* A, const R* __restrict__ qf,
+aa_collide_kernel(const __grid_constant__ KParams p, P* A, const R* qf,
                                   double* __restrict__ partials, int* __restrict__ status) {
     dependent_launch_point();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1082,7 +1084,7 @@ __device__ __forceinline__ void fused2d_tile(const KParams& p, const P* __restri
 
 template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY)
-fused2d_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst,
+fused2d_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst,
                double* __restrict__ partials, int* __restrict__ status) {
     wait_for_previous();
     fused2d_tile<TY, CAL, true>(p, src, dst, blockIdx.x, blockIdx.y, partials + 5 * (blockIdx.x + gridDim.x * blockIdx.y),
@@ -1099,7 +1101,7 @@ fused2d_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* 
 // where the 32 x 8 tiles used 25 (800 x 4, FP64: 14.4 us a step; this kernel 4.5).
 template <bool CAL, bool FIX>
 __global__ void __launch_bounds__(128)
-fused2d_row_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst, int strips,
+fused2d_row_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, int strips,
                    double* __restrict__ partials, int* __restrict__ status) {
     __shared__ R red[4][5][32];
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
@@ -1194,7 +1196,7 @@ fused2d_row_kernel(const __grid_constant__ KParams p, const P* __restrict__ src,
 #if ELBM_ST == 0 && ELBM_D == 2
 template <bool CAL, bool FIX>
 __global__ void __launch_bounds__(128)
-fused2d_split_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst, int strips,
+fused2d_split_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, int strips,
                      double* __restrict__ partials, int* __restrict__ status) {
     enum { RHO, TT_, UX, UY, RE, QXL, QX, QXR, QY, QD, QU, PX, GX, AX = GX + 3, PY = AX + 3, GY, SY = GY + 3, KK = SY + 3,
            WR, W1R, OMW, OMW1, HH, DX, DY, FX, FY, NV };
@@ -1335,7 +1337,7 @@ fused2d_split_kernel(const __grid_constant__ KParams p, const P* __restrict__ sr
 // offset[k] of both stores; its parameters are params[k].  No totals are kept.
 template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY)
-ensemble2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int* __restrict__ status) {
+ensemble2d_kernel(const EnsembleArgs a, const P* src, P* __restrict__ dst, int* __restrict__ status) {
     wait_for_previous();
     __shared__ int s_start[kMaxEnsemble + 1];
     __shared__ int s_tx[kMaxEnsemble];
@@ -1431,7 +1433,7 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, i
 template <int TY, int NB, int MINB, bool EARLY, int DD, bool CAL>
 __global__ void __launch_bounds__(TX * TY, MINB)
 fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl,
-               const P* __restrict__ src, double* __restrict__ partials, int* __restrict__ status,
+               const P* src, double* __restrict__ partials, int* __restrict__ status,
                const __grid_constant__ CUtensorMap pmap, int pref) {
     using PP = Pipe<TY, NB>;
     static_assert(NB == 2, "plane z+2 is prefetched into the slots of plane z");
@@ -1722,7 +1724,7 @@ constexpr bool kPrefTma = ELBM_PREF_TMA;
 template <int TY, int MINB, int DD, bool CAL>
 __global__ void __launch_bounds__(TX * TY, MINB)
 fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl,
-                   const __grid_constant__ CUtensorMap tmap, const P* __restrict__ src,
+                   const __grid_constant__ CUtensorMap tmap, const P* src,
                    double* __restrict__ partials, int* __restrict__ status) {
     using TT = Tma<TY>;
     static_assert(sizeof(R) == 4 && DD == 3, "the TMA-staged kernel is D3Q27 in FP32 arithmetic");
@@ -1931,7 +1933,7 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
 // from a first gather, then gathers plane z again (an L2 hit) to collide it.
 template <int TY, bool CAL>
 __global__ void __launch_bounds__(TX * TY, 2)
-fused3d_reread_kernel(const __grid_constant__ KParams p, const P* __restrict__ src, P* __restrict__ dst,
+fused3d_reread_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst,
                       double* __restrict__ partials, int* __restrict__ status) {
     wait_for_previous();
     __shared__ R qx[2][TY][TX + 2];
@@ -2425,7 +2427,7 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
 template <int W> constexpr int kPairCtas = 1024 / W;
 template <int W, bool CAL, bool FIX>
 __global__ void __launch_bounds__(W / 2, kPairCtas<W>)
-march2d_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* __restrict__ src,
+march2d_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* src,
                     double* __restrict__ partials, int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
     wait_for_previous();
@@ -2455,7 +2457,7 @@ march2d_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ D
 #endif
 template <int W, int NB, bool CAL, bool FIX>
 __global__ void ELBM_MARCH_BOUNDS(W)
-march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* __restrict__ src,
+march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl, const P* src,
                double* __restrict__ partials, int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
     wait_for_previous();
@@ -2488,7 +2490,7 @@ template <int W, int NB> constexpr size_t march_smem_bytes = March2<W, NB>::smem
 #endif
 template <int W, int NB, bool CAL, bool FIX>
 __global__ void ELBM_ENSEMBLE_BOUNDS(W)
-ensemble_march2d_kernel(const EnsembleArgs a, const P* __restrict__ src, P* __restrict__ dst, int seg,
+ensemble_march2d_kernel(const EnsembleArgs a, const P* src, P* __restrict__ dst, int seg,
                         int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
     wait_for_previous();
