@@ -110,10 +110,11 @@ typedef enum {
  * other (every schedule).  AA: one store updated in place, its layout alternating with the
  * step parity (after an even number of steps the pairs of a node sit at the node with each
  * direction in the opposite direction's plane; after an odd number, each pair sits at the
- * node it streams to next), on the two-pass schedule: the first pass writes the Q~ field,
- * the second reads and writes exactly the slots each node read, so no two threads touch one
- * slot.  Half the population memory (D3Q27 FP32 at 1024^3: 232 GB instead of 464 GB), 1.5x
- * the bytes per update of the fused schedule.  Periodic grids only (a zero-gradient or fixed
+ * node it streams to next): the first kernel of a step writes Q~ (of every node; D3Q27 with
+ * FP32 arithmetic and more than 64 MB of store: of the nodes at the faces of the second
+ * one's tiles), the second reads and writes exactly the slots each node read, so no two
+ * threads touch one slot.  Half the population memory (D3Q27 FP32 at 1024^3: 232 GB instead
+ * of 464 GB), 1.5x the bytes per update of the fused schedule.  Periodic grids only (a zero-gradient or fixed
  * face makes two nodes read one slot that one of them writes). */
 typedef enum { ELBM_LAYOUT_PINGPONG = 0, ELBM_LAYOUT_AA = 1 } elbm_layout;
 

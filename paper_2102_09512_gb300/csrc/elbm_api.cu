@@ -26,6 +26,7 @@ struct elbm_handle {
     CUtensorMap tmap[2];     // tensor maps of pop[0], pop[1] (TMA-staged D3Q27 kernel)
     CUtensorMap pfmap[2];    // ... with the L2-prefetch boxes of the default fused kernel
     bool tmap_ready;
+    bool aa_map_ready;       // AA layout: pfmap[0] holds the single store's prefetch map
     char* auxp;
     cudaStream_t stream;
     bool bound;
@@ -261,7 +262,7 @@ cudaError_t step_one(elbm_handle* h, cudaStream_t st) {
     cudaError_t e;
     if (h->layout == ELBM_LAYOUT_AA) {   // the layout alternates: L0 after an even number of steps
         e = h->ops->step_aa(h->kp, h->pop[0], h->auxp + h->aux.qfield, step_partials(h), &h->step_blocks,
-                            status_ptr(h), st, &h->launches, (int)(h->steps % 2));
+                            status_ptr(h), st, &h->launches, (int)(h->steps % 2), h->aa_map_ready ? &h->pfmap[0] : nullptr);
         if (e == cudaSuccess) ++h->steps;
         return e;
     }
@@ -393,6 +394,7 @@ int elbm_bind(elbm_handle* h, void* pop_a, void* pop_b, void* aux, void* stream)
                         h->ops->encode_tmap(h->kp, pop_b, &h->tmap[1], kTmapStage) == 1 &&
                         h->ops->encode_tmap(h->kp, pop_a, &h->pfmap[0], kTmapPrefetch) == 1 &&
                         h->ops->encode_tmap(h->kp, pop_b, &h->pfmap[1], kTmapPrefetch) == 1;
+    h->aa_map_ready = aa && h->ops->encode_tmap(h->kp, pop_a, &h->pfmap[0], kTmapPrefetchAa) == 1;
     h->auxp = (char*)aux;
     h->stream = (cudaStream_t)stream;
     h->cur = 0;
@@ -407,7 +409,7 @@ int elbm_bind(elbm_handle* h, void* pop_a, void* pop_b, void* aux, void* stream)
 int aa_collide_initial(elbm_handle* h) {
     int nb = 0;
     return cuda_status(h->ops->step_aa(h->kp, h->pop[0], h->auxp + h->aux.qfield, query_partials(h), &nb,
-                                       status_ptr(h), h->stream, &h->launches, 1));
+                                       status_ptr(h), h->stream, &h->launches, 1, h->aa_map_ready ? &h->pfmap[0] : nullptr));
 }
 
 int elbm_set_fields_device(elbm_handle* h, const double* rho, const double* u, const double* T) {

@@ -278,7 +278,7 @@ struct Ops {
     int (*tma_supported)(const KParams& p);   // the grid suits the TMA-staged D3Q27 kernel
     // tensor map of a store: 1 made, 0 not applicable, -1 the driver refused.  kind
     // kTmapStage: the boxes the TMA-staged kernel copies; kTmapPrefetch: the boxes the
-    // default fused kernel prefetches into L2
+    // default fused kernel prefetches into L2; kTmapPrefetchAa: those of its in-place form
     int (*encode_tmap)(const KParams& p, const void* base, CUtensorMap* out, int kind);
     // the default fused step given src's prefetch tensor map (L2 prefetch of the planes ahead)
     cudaError_t (*step_fused_pf)(const KParams& p, const void* src, void* dst, const CUtensorMap* src_map,
@@ -293,7 +293,7 @@ struct Ops {
     // L1 (from_l1 = 1: node-local reads, swapped writes) or from layout L0 (pulled reads,
     // pushed writes)
     cudaError_t (*step_aa)(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
-                           cudaStream_t s, long long* launches, int from_l1);
+                           cudaStream_t s, long long* launches, int from_l1, const CUtensorMap* pmap);
     int march_width;   // D2Q9: strip width of the single-lattice row march of this store
 };
 
@@ -366,7 +366,7 @@ inline void plan_d2q9(KParams& k, int sms, int per_sm, int width, bool f64) {
     else k.sched = f64 ? kSchedTwoPass : kSchedMarch;
 }
 
-constexpr int kTmapStage = 0, kTmapPrefetch = 1;   // encode_tmap kinds
+constexpr int kTmapStage = 0, kTmapPrefetch = 1, kTmapPrefetchAa = 2;   // encode_tmap kinds
 
 const Ops* ops_d2_f64();
 const Ops* ops_d2_f32();

@@ -1405,10 +1405,69 @@ __device__ __forceinline__ const P* dir_src(const DirPlanes& pl, const PullRows&
     return pl.src[i] + (unsigned)(r.row[b][c] + r.xs[a]);
 }
 
+// AA single store (src = dst): direction j's pair where direction k is pulled from.
+__device__ __forceinline__ P* aa_slot(const DirPlanes& pl, const PullRows& r, int j, int k) {
+    const int a = k % 3, b = (k / 3) % 3, c = (kD == 3) ? k / 9 : 1;
+    return pl.dst[j] + (unsigned)(r.row[b][c] + r.xs[a]);
+}
+
 template <int TY, int NB>
 struct PipeBytes {
     static constexpr size_t value = Pipe<TY, NB>::smem_bytes;
 };
+
+// Q~ of the nodes at the faces of the fused kernel's tiles and segments, where other CTAs of
+// the in-place march read it: Q~_yyy in the first and last row of every tile, Q~_xxx in its first
+// and last column, Q~_zzz in the first and last plane of every segment (30 % of the nodes with 32
+// x 8 tiles).  The columns touch a line of 128 bytes in every 16 (FP32) or 32 nodes, so this reads
+// about the whole store, at the memory's rate (256^3 FP32 0.5 ms); rows and columns of a plane
+// are adjacent CTAs, whose shared lines come from memory once.
+struct AaEdges {
+    int tx, ty, tz;               // tile and segment
+    int nr, nc, ns;               // rows, columns, planes of the three sets
+    unsigned br, bc;              // CTAs of a plane's rows and columns
+};
+template <bool FROM_L1>
+__global__ void __launch_bounds__(kThreads1D)
+aa_edges_kernel(const __grid_constant__ KParams p, const __grid_constant__ AaEdges e, P* A, R* __restrict__ qf) {
+    wait_for_previous();
+    // entry k of the set 0 | t - 1, t | 2 t - 1, 2 t | ... | n - 1
+    auto member = [](int k, int t, int n) { return k % 2 == 0 ? k / 2 * t : min((k + 1) / 2 * t, n) - 1; };
+    const unsigned per = e.br + e.bc, pz = blockIdx.x / per;
+    int x, y, z = p.nz, comp;
+    if (pz < (unsigned)p.nz) {
+        unsigned k = blockIdx.x - pz * per;
+        comp = k < e.br ? 1 : 0;
+        k = (comp ? k : k - e.br) * kThreads1D + threadIdx.x;
+        const unsigned w = comp ? p.nx : e.nc, line = k / w;
+        if (comp) {
+            x = (int)(k - line * w);
+            y = member((int)line, e.ty, p.ny);
+        } else {
+            x = member((int)(k - line * w), e.tx, p.nx);
+            y = (int)line;
+        }
+        if (line < (unsigned)(comp ? e.nr : p.ny)) z = (int)pz;
+    } else {
+        const long long k = (long long)(blockIdx.x - per * (unsigned)p.nz) * kThreads1D + threadIdx.x, line = k / p.nx;
+        x = (int)(k - line * p.nx);
+        const int q = (int)(line / p.ny);
+        y = (int)(line - (long long)q * p.ny);
+        if (q < e.ns) z = member(q, e.tz, p.nz);
+        comp = 2;
+    }
+    if (z < p.nz) {
+        const long long n = node_index(p, x, y, z);
+        PullRows r;
+        if (!FROM_L1) pull_rows(p, x, y, z, r);
+        R f[Q], g[Q];
+        aa_gather<FROM_L1>(p, A, r, n, f, g);
+        Moments<R> m;
+        node_moments<kD, R, false, DEV>(f, g, p, m);
+        qf[(long long)comp * p.N + n] = anomaly(m.rho, comp == 0 ? m.ux : comp == 1 ? m.uy : m.uz, m.T);
+    }
+    launch_dependents();
+}
 
 // Store of a post-collision pair.  With ELBM_STCS the store is marked streaming (evict
 // first), so that the step's writes do not push the planes prefetched ahead out of L2.
@@ -1430,11 +1489,15 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, i
                  : "memory");
 }
 
-template <int TY, int NB, int MINB, bool EARLY, int DD, bool CAL>
+// AA = 1, 2: the same march in place on the AA single store (pl.src = pl.dst), from layout L0 or
+// L1.  A node's slots are read and written by its own thread alone, so what the kernel may not do
+// is read other CTAs' nodes: Q~ of the halo ring and of the planes on either side of the segment
+// comes from qf, where aa_edges_kernel put it before.
+template <int TY, int NB, int MINB, bool EARLY, int DD, bool CAL, int AA>
 __global__ void __launch_bounds__(TX * TY, MINB)
 fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPlanes pl,
                const P* src, double* __restrict__ partials, int* __restrict__ status,
-               const __grid_constant__ CUtensorMap pmap, int pref) {
+               const __grid_constant__ CUtensorMap pmap, int pref, const R* qf) {
     using PP = Pipe<TY, NB>;
     static_assert(NB == 2, "plane z+2 is prefetched into the slots of plane z");
     static_assert(sizeof(R) == 4 && DD == 3, "the pipelined kernel is D3Q27 in FP32");
@@ -1462,12 +1525,19 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     auto issue_plane = [&](int q, int sb, bool with_halo) {
         P* bb = buf + (size_t)sb * Q * NS;
         if (active) {
-            PullRows r;
-            pull_rows(p, x, y, q, r);
+            if constexpr (AA == 2) {
+                const unsigned n = (unsigned)node_index(p, x, y, q);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) cp_async<sizeof(P)>(bb + i * NS + tid, dir_src(pl, r, i));
+                for (int i = 0; i < Q; ++i) cp_async<sizeof(P)>(bb + i * NS + tid, pl.src[i] + n);
+            } else {
+                PullRows r;
+                pull_rows(p, x, y, q, r);
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+                    cp_async<sizeof(P)>(bb + i * NS + tid, AA ? aa_slot(pl, r, opp(i), i) : dir_src(pl, r, i));
+            }
         }
-        if (with_halo && has_halo) {
+        if (AA == 0 && with_halo && has_halo) {
             PullRows r;
             pull_rows(p, hx, hy, q, r);
 #pragma unroll
@@ -1501,6 +1571,12 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
     // the neighbours' columns, which in FP32 cost 15 % more DRAM reads and 11 % of the step.
     const int pf_lane = tid - (NT - 32);
     auto prefetch_plane = [&](int q) {
+        if (AA && pf_lane >= 0 && pf_lane < Q) {   // box TX x TY: the tile's rows where they are pulled from
+            const int i = pf_lane, b = (i / 3) % 3, c = i / 9;
+            if (AA == 2) tma_prefetch_3d(&pmap, x0, y0, i * p.nz + q);
+            else tma_prefetch_3d(&pmap, x0, max(y0 + 1 - b, 0), opp(i) * p.nz + map_axis(q + 1 - c, p.nz, p.per_z));
+            return;
+        }
         if (pf_lane >= 0 && pf_lane < Q) {
             const int i = pf_lane, b = (i / 3) % 3, c = i / 9;
             // x0 is a multiple of TX (x0 * pair size a multiple of 16 bytes); rows clamped
@@ -1514,10 +1590,18 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
 
     // prologue: Q~_zzz below the segment, planes zb and zb+1 in flight, moments of zb
     R qz_prev = R(0), qz_cur = R(0), qz_next = R(0);
-    if (active) qz_prev = direct_anomaly_z<CAL>(p, src, x, y, map_axis(zb - 1, p.nz, p.per_z));
-    for (int d = 2; d < 2 + pref && zb + d <= ze; ++d) prefetch_plane(map_axis(zb + d, p.nz, p.per_z));
+    // AA: Q~ at this thread's node or halo node of a plane, from qf
+    auto field_qz = [&](int q) { return qf[2 * p.N + node_index(p, x, y, map_axis(q, p.nz, p.per_z))]; };
+    auto field_halo = [&](int q) { return qf[(haxis == 1 ? p.N : 0) + node_index(p, hx, hy, q)]; };
+    const int zt = AA ? ze - 1 : ze;   // last plane whose pairs are needed
+    if (active) {
+        if constexpr (AA) qz_prev = field_qz(zb - 1);
+        else qz_prev = direct_anomaly_z<CAL>(p, src, x, y, map_axis(zb - 1, p.nz, p.per_z));
+    }
+    for (int d = 2; d < 2 + pref && zb + d <= zt; ++d) prefetch_plane(map_axis(zb + d, p.nz, p.per_z));
     issue_plane(zb, 0, true);
-    issue_plane(map_axis(zb + 1, p.nz, p.per_z), 1 % NB, zb + 1 < ze);
+    if (zb + 1 <= zt) issue_plane(map_axis(zb + 1, p.nz, p.per_z), 1 % NB, zb + 1 < ze);
+    else cp_async_commit();
     Moments<R> m_cur, m_next;
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
@@ -1527,11 +1611,18 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
         QY(0, ty + 1, tx) = anomaly(m_cur.rho, m_cur.uy, m_cur.T);
         qz_cur = anomaly(m_cur.rho, m_cur.uz, m_cur.T);
     }
+    auto put_halo = [&](int b, R q) {
+        if (haxis == 1) QY(b, hsy, hsx) = q;
+        else QX(b, hsy, hsx) = q;
+    };
     if (has_halo) {
-        Moments<R> hm;
-        slot_moments(0, NT + tid, hm, Lite());
-        if (haxis == 1) QY(0, hsy, hsx) = anomaly(hm.rho, hm.uy, hm.T);
-        else QX(0, hsy, hsx) = anomaly(hm.rho, hm.ux, hm.T);
+        if constexpr (AA) {
+            put_halo(0, field_halo(zb));
+        } else {
+            Moments<R> hm;
+            slot_moments(0, NT + tid, hm, Lite());
+            put_halo(0, anomaly(hm.rho, haxis == 1 ? hm.uy : hm.ux, hm.T));
+        }
     }
 
     for (int z = zb; z < ze; ++z) {
@@ -1547,17 +1638,21 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
         // moments of plane z+1, so the copy overlaps them too (both planes are live
         // in registers meanwhile, which only a one-CTA-per-SM launch affords)
         P pk[Q];   // the pulled pairs of plane z, as stored
-        if (pref > 0 && z + 2 + pref <= ze) prefetch_plane(map_axis(z + 2 + pref, p.nz, p.per_z));
+        if (pref > 0 && z + 2 + pref <= zt) prefetch_plane(map_axis(z + 2 + pref, p.nz, p.per_z));
         if (EARLY) {
             if (active) {
                 const P* bb = buf + (size_t)sz * Q * NS + tid;
 #pragma unroll
                 for (int i = 0; i < Q; ++i) pk[i] = bb[i * NS];
             }
-            if (z + 2 <= ze) issue_plane(map_axis(z + 2, p.nz, p.per_z), sz, z + 2 < ze);
+            if (z + 2 <= zt) issue_plane(map_axis(z + 2, p.nz, p.per_z), sz, z + 2 < ze);
         }
 
-        if (active) {
+        R halo_next = R(0);
+        if (AA && !last && has_halo) halo_next = field_halo(z + 1);
+        if (AA && last) {
+            if (active) qz_next = field_qz(ze);
+        } else if (active) {
             slot_moments(sn, tid, m_next, Full());
             qz_next = anomaly(m_next.rho, m_next.uz, m_next.T);
             if (!last) {
@@ -1566,10 +1661,13 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
             }
         }
         if (!last && has_halo) {
-            Moments<R> hm;
-            slot_moments(sn, NT + tid, hm, Lite());
-            if (haxis == 1) QY(bq ^ 1, hsy, hsx) = anomaly(hm.rho, hm.uy, hm.T);
-            else QX(bq ^ 1, hsy, hsx) = anomaly(hm.rho, hm.ux, hm.T);
+            if constexpr (AA) {
+                put_halo(bq ^ 1, halo_next);
+            } else {
+                Moments<R> hm;
+                slot_moments(sn, NT + tid, hm, Lite());
+                put_halo(bq ^ 1, anomaly(hm.rho, haxis == 1 ? hm.uy : hm.ux, hm.T));
+            }
         }
 
         if (!EARLY) {
@@ -1578,7 +1676,7 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
 #pragma unroll
                 for (int i = 0; i < Q; ++i) pk[i] = bb[i * NS];
             }
-            if (z + 2 <= ze) issue_plane(map_axis(z + 2, p.nz, p.per_z), sz, z + 2 < ze);
+            if (z + 2 <= zt) issue_plane(map_axis(z + 2, p.nz, p.per_z), sz, z + 2 < ze);
         }
         if (active) {
             bad |= nonphysical(m_cur);
@@ -1590,11 +1688,14 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
             acc.add(v);
             // collide and store pair by pair, decoding each just before its update
             const unsigned n = (unsigned)node_index(p, x, y, z);
+            PullRows w;   // AA from L0: the new pairs go to where opposite directions are pulled from
+            if constexpr (AA == 1) pull_rows(p, x, y, z, w);
+            auto out = [&](int i) { return AA == 0 ? pl.dst[i] + n : AA == 2 ? pl.dst[opp(i)] + n : aa_slot(pl, w, i, opp(i)); };
             if constexpr (DEV) {
                 RelaxDev<CAL> rx;
                 rx.init(m_cur, Dx, Dy, Dz, p);
                 rx.apply([&](int i, R& f, R& g) { Cd::dec(pk[i], f, g); },
-                         [&](int i, R f, R g) { store_pair(pl.dst[i] + n, Cd::enc(f, g)); });
+                         [&](int i, R f, R g) { store_pair(out(i), Cd::enc(f, g)); });
             } else {
                 Relax<kD, R, DEV, CAL> rx;
                 rx.init(m_cur, Dx, Dy, Dz, p);
@@ -1603,7 +1704,7 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
                     R f, g;
                     Cd::dec(pk[i], f, g);
                     const float2 o = rx.fg(i, make_float2(f, g), p);
-                    store_pair(pl.dst[i] + n, Cd::enc(o.x, o.y));
+                    store_pair(out(i), Cd::enc(o.x, o.y));
                 }
             }
         }
@@ -2622,13 +2723,13 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 int encode_tmap(const KParams& p, const void* base, CUtensorMap* out, int kind) {
-    if (!tma_supported(p) || (kind != kTmapStage && kind != kTmapPrefetch)) return 0;
+    if (!tma_supported(p) || (kind != kTmapStage && kind != kTmapPrefetch && kind != kTmapPrefetchAa)) return 0;
     static const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();   // resolved once, thread-safe
     if (!encode) return -1;
     const cuuint64_t dims[3] = {(cuuint64_t)p.nx, (cuuint64_t)p.ny, (cuuint64_t)p.nz * Q};
     const cuuint64_t strides[2] = {(cuuint64_t)p.nx * sizeof(P), (cuuint64_t)p.nx * p.ny * sizeof(P)};
     const cuuint32_t box[3] = {(cuuint32_t)(kind == kTmapStage ? TmaCfg::BW : TX),
-                               (cuuint32_t)(kind == kTmapStage ? TmaCfg::RB : kTYP + 2), 1u};
+                               (cuuint32_t)(kind == kTmapStage ? TmaCfg::RB : kind == kTmapPrefetch ? kTYP + 2 : kTYP), 1u};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     const CUtensorMapDataType dt = sizeof(P) == 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
 #ifndef ELBM_TMAP_PROMO
@@ -2727,10 +2828,49 @@ cudaError_t launch_fields_nodes(const KParams& p, const void* pop, double* rho, 
     return cudaGetLastError();
 }
 
+#ifndef ELBM_PREF
+#define ELBM_PREF 1
+#endif
+constexpr int kPref = ELBM_PREF;   // planes of L2 prefetch ahead of the cp.async copies (with a tensor map)
+
 // One AA step on the single store A: from layout L1 (node-local reads, swapped writes) or
-// from L0 (pulled reads, pushed writes).
+// from L0 (pulled reads, pushed writes).  Stores larger than the L2 cache, D3Q27, FP32
+// arithmetic: the edges' Q~, then the march in place; the store is read 1.5 times less than by the
+// two passes, which take smaller grids (whose second pass finds the store in the cache).
+template <int DD>
+cudaError_t launch_aa_march(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
+                            cudaStream_t s, int from_l1, const CUtensorMap* pmap) {
+    if constexpr (DD == 3 && kPipe) {
+        const dim3 grid = fused_grid(p);
+        AaEdges e;
+        e.tx = TX, e.ty = kTYP, e.tz = p.tz;
+        e.nr = 2 * (int)grid.y, e.nc = 2 * (int)grid.x, e.ns = 2 * (int)grid.z;
+        e.br = (unsigned)blocks_1d_of((long long)e.nr * p.nx);
+        e.bc = (unsigned)blocks_1d_of((long long)e.nc * p.ny);
+        const unsigned bs = (unsigned)blocks_1d_of((long long)e.ns * p.nx * p.ny);
+        auto edges = from_l1 ? aa_edges_kernel<true> : aa_edges_kernel<false>;
+        cudaError_t c = launch_dependent(edges, dim3((e.br + e.bc) * (unsigned)p.nz + bs), dim3(kThreads), 0, s, p, e, (P*)A, (R*)qfield);
+        if (c != cudaSuccess) return c;
+        auto kern = p.eos ? (from_l1 ? fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, true, 2>
+                                     : fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, true, 1>)
+                          : (from_l1 ? fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, false, 2>
+                                     : fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, false, 1>);
+        c = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PipeCfg::smem_bytes);
+        if (c != cudaSuccess) return c;
+        CUtensorMap none;
+        std::memset(&none, 0, sizeof(none));
+        *nblocks = (int)(grid.x * grid.y * grid.z);
+        return launch_dependent(kern, grid, dim3(TX, kTYP), PipeCfg::smem_bytes, s, p, dir_planes(p, A, A), (const P*)A,
+                                partials, status, pmap ? *pmap : none, pmap ? kPref : 0, (const R*)qfield);
+    } else {
+        return cudaErrorInvalidValue;
+    }
+}
 cudaError_t launch_step_aa(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
-                           cudaStream_t s, long long* launches, int from_l1) {
+                           cudaStream_t s, long long* launches, int from_l1, const CUtensorMap* pmap) {
+    *launches += 2;
+    if (kD == 3 && kPipe && (double)p.N * Q * sizeof(P) > 64e6)
+        return launch_aa_march<kD>(p, A, qfield, partials, nblocks, status, s, from_l1, pmap);
     const unsigned nb = blocks_1d(p.N);
     if (from_l1) {
         launch_dependent(aa_moments_kernel<true>, nb, kThreads, 0, s, p, (P*)A, (R*)qfield);
@@ -2739,7 +2879,6 @@ cudaError_t launch_step_aa(const KParams& p, void* A, void* qfield, double* part
         launch_dependent(aa_moments_kernel<false>, nb, kThreads, 0, s, p, (P*)A, (R*)qfield);
         launch_dependent(aa_collide_kernel<false>, nb, kThreads, 0, s, p, (P*)A, (const R*)qfield, partials, status);
     }
-    *launches += 2;
     *nblocks = (int)nb;
     return cudaGetLastError();
 }
@@ -2762,11 +2901,6 @@ cudaError_t launch_twopass(const KParams& p, const void* src, void* dst, void* q
 
 // A template so that the branch of the other lattice is never instantiated; CAL as in
 // the kernels (the caloric form only for handles with a Cv(T) model).
-#ifndef ELBM_PREF
-#define ELBM_PREF 1
-#endif
-constexpr int kPref = ELBM_PREF;   // planes of L2 prefetch ahead of the cp.async copies (with a tensor map)
-
 // The row march of this store for grid p (D2Q9).
 template <int DD, bool CAL>
 auto march_kernel(const KParams& p) {
@@ -2809,7 +2943,7 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
         bool launched = false;
         if constexpr (kPipe) {
             if (!reread) {
-                auto kern = fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, CAL>;
+                auto kern = fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, CAL, 0>;
                 // the dynamic shared-memory limit is a per-function attribute; setting it
                 // again is cheap and keeps this correct for every device of the process
                 cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2819,7 +2953,8 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
                 CUtensorMap none;
                 std::memset(&none, 0, sizeof(none));
                 e = launch_dependent(kern, dim3(grid), dim3(TX, kTYP), PipeCfg::smem_bytes, s, p, pl, (const P*)src, partials, status,
-                                                                       pmap ? *pmap : none, pmap ? kPref : 0);
+                                                                       pmap ? *pmap : none, pmap ? kPref : 0,
+                                     (const R*)nullptr);
             if (e != cudaSuccess) return e;
                 launched = true;
             }
@@ -2987,7 +3122,7 @@ template <int DD>
 int fused_occupancy_impl(const KParams& p) {
     int n = 0;
     if constexpr (DD == 3 && kPipe) {
-        auto kern = fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, false>;
+        auto kern = fused3d_kernel<kTYP, kNB, kMinB, kEarly, DD, false, 0>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PipeCfg::smem_bytes) !=
                 cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TX * kTYP, PipeCfg::smem_bytes) != cudaSuccess)
