@@ -347,22 +347,26 @@ inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW
 // What the default schedule of a D2Q9 grid runs on a device of `sms` SMs, and the row segment of
 // the march.  Measured on 152 SMs, us a step (Sod parameters, zero-gradient x ends):
 //   FP32     strips  tiles  march        FP64   strips  tiles  two passes
-//   800x4      2.7    3.4    5.8         800x4     5.5   11.3    13.6
-//   180^2      3.3    3.8     -          1700x8   10.5   17.9    14.4
-//   256^2      4.5    4.6    6.5         128^2    16.1   17.9    13.6
-//   384^2      7.4    5.8    7.8         256^2    46.6   33.0    45.0
-//   512^2     11.6   10.1    9.5         384^2    94.4   63.2    64.2
-//   724^2     20.6   17.6   14.6         512^2     173    109     101
-//   1024^2      -    37.2   29.3         1448^2     -     848     750   (march 880)
-// (16-bit stores as FP32).  So: strips while there are at most eight to an SM (FP64, where each
-// keeps four warps busy: four), tiles while there are at most four to an SM, else the march,
-// for FP64 the two passes, which the FP64 pipe bounds and no wave of CTAs leaves idle.
+//   800x4      2.6    3.4    5.8         800x4     5.4   11.3      13.6
+//   180^2      3.3    3.8     -          800x20   13.0   17.9      14.4
+//   256^2      4.5    4.6    6.5         128^2    16.0   17.9      14.5
+//   384^2      7.4    5.8    7.8         160^2    18.1   17.9      18.3
+//   512^2     11.6   10.1    9.5         220^2      -    32.9      27.5
+//   724^2     20.6   17.6   14.6         256^2    46.6   33.0      33.0
+//   1024^2      -    37.2   29.3         384^2    94.4   63.2      60.8
+//                                        512^2    173    109       102
+//                                        1448^2     -    848       752   (march 880)
+// (16-bit stores as FP32).  So: strips while there are at most eight to an SM, tiles while there
+// are at most four, else the march.  FP64: strips while there are at most four to an SM, each
+// of which keeps four warps busy; then the two passes, which the FP64 pipe bounds and no wave of
+// CTAs leaves idle; but tiles where one to an SM does and the passes need a second warp to a
+// quarter of an SM (more than 128 nodes to an SM).
 constexpr int kSchedMarch = 0, kSchedTile = 1, kSchedRow = 2, kSchedTwoPass = 3;
 inline void plan_d2q9(KParams& k, int sms, int per_sm, int width, bool f64) {
     k.tz = choose_rows(k, sms, per_sm, k.tz, width);
     const long long strips = row_strips(k), tiles = (long long)((k.nx + 31) / 32) * ((k.ny + 7) / 8);
     if (sms > 0 && strips <= (f64 ? 4LL : 8LL) * sms && strips <= kRowMost) k.sched = kSchedRow;
-    else if (sms > 0 && tiles <= 4LL * sms) k.sched = kSchedTile;
+    else if (sms > 0 && (f64 ? tiles <= sms && k.N > 128LL * sms : tiles <= 4LL * sms)) k.sched = kSchedTile;
     else k.sched = f64 ? kSchedTwoPass : kSchedMarch;
 }
 

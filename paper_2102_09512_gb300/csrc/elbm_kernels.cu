@@ -1098,12 +1098,13 @@ fused2d_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ 
 // are requested before any arithmetic, so a warp waits for memory once.  A grid of a few
 // thousand nodes is all latency, and in FP64 the arithmetic of a warp keeps its SM's pipe busy
 // for about 16 cycles an instruction: one warp to a CTA spreads 3,200 nodes over 108 SMs
-// where the 32 x 8 tiles used 25 (800 x 4, FP64: 14.4 us a step; this kernel 4.5).
+// where the 32 x 8 tiles used 25 (800 x 4, FP32: 3.4 us a step, this kernel 2.6).
+constexpr int kRowSmem = 5 * 32 * (int)sizeof(R);   // its static shared memory, bytes
 template <bool CAL, bool FIX>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32)
 fused2d_row_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, int strips,
                    double* __restrict__ partials, int* __restrict__ status) {
-    __shared__ R red[4][5][32];
+    __shared__ R red[1][5][32];
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int y = warp / strips, x = (warp - y * strips) * kRowW - 1 + lane;
@@ -1194,12 +1195,14 @@ fused2d_row_kernel(const __grid_constant__ KParams p, const P* src, P* __restric
 // flux of q*; then one row of three directions each, and the totals.  About 86 instructions deep
 // instead of 205.
 #if ELBM_ST == 0 && ELBM_D == 2
+constexpr int kSplitSmem = 35 * 34 * (int)sizeof(double);   // its static shared memory, bytes
 template <bool CAL, bool FIX>
 __global__ void __launch_bounds__(128)
 fused2d_split_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, int strips,
                      double* __restrict__ partials, int* __restrict__ status) {
     enum { RHO, TT_, UX, UY, RE, QXL, QX, QXR, QY, QD, QU, PX, GX, AX = GX + 3, PY = AX + 3, GY, SY = GY + 3, KK = SY + 3,
            WR, W1R, OMW, OMW1, HH, DX, DY, FX, FY, NV };
+    static_assert(NV * 34 * sizeof(double) == kSplitSmem, "static shared memory");
     __shared__ double v[NV][34];   // column lane + 1 of a node; QXL and QXR are QX shifted by one
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, col = lane + 1;
     const int y = blockIdx.x / strips, x = (blockIdx.x - y * strips) * kRowW - 1 + lane;
@@ -2780,13 +2783,39 @@ int max_blocks(const KParams& p) {
     return (int)m;
 }
 
+// Dynamic shared memory that makes an SM hold ceil(ctas / 152) CTAs of `stat` bytes of their own
+// and no more (an SM has 228 KB, 1 KB of which goes with each CTA).  The next kernel's CTAs are set
+// up while this one's still run: counted against the same limits, they went two and three to
+// an SM while others had none, and in FP64 such CTAs share one pipe.  us a step, zero-gradient
+// 2D grids and periodic boxes, without this limit and with it:
+//   strips, FP64  800x4  6.46  5.38    800x9 9.58  7.66    800x15 13.18 10.33    800x20 16.05 12.99
+//   strips, FP32  800x4  2.66  2.60   800x15 2.94  2.74    800x20  3.05  2.81    800x43  3.37  3.31
+//   FP64 passes   140^2  35.2  18.0    220^2 40.6  27.5     256^2  45.2  33.0     320^2  55.4  47.0
+//                  24^3  35.1  27.8     28^3 45.0  35.7      32^3  44.1  35.4      36^3  65.1  55.4
+// From nine CTAs to an SM on the grid takes several waves anyway: no limit.  (The march, whose rows
+// reuse the first-level cache that this takes away, is slower with it: FP32 1024^2 28.0 -> 35.0;
+// the tiles and the D3Q27 kernel do not change.)  The function's attribute is set to the same value
+// every time: another thread's launch, or a graph captured before, may need more than this one.
+constexpr int kSms = 152, kSmShared = 228 * 1024;
+template <class... Args>
+size_t spread_smem(void (*kern)(Args...), long long ctas, int stat) {
+    const long long k = (ctas + kSms - 1) / kSms;
+    if (k > 8) return 0;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmShared / 2);
+    return (size_t)(kSmShared / (k + 1) - stat);
+}
+
 template <bool PULL>
 void launch_two_passes(const KParams& p, const void* src, void* dst, void* qfield, double* partials, int* status,
                        cudaStream_t s) {
     const unsigned nb = blocks_1d(p.N);
 #if ELBM_ST == 0
-    launch_dependent(moments64_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
-    launch_dependent(collide64_kernel<PULL>, (unsigned)((p.N + kThreads64 - 1) / kThreads64), kThreads64, 0, s, p, (const P*)src, (P*)dst, (const R*)qfield);
+    const unsigned nc = (unsigned)((p.N + kThreads64 - 1) / kThreads64);
+    constexpr int stat = 5 * kThreads1D * (int)sizeof(double);   // of the totals
+    const size_t sm = nc > 8 * kSms ? 0 : spread_smem(moments64_kernel<PULL>, nb, stat);
+    const size_t sc = spread_smem(collide64_kernel<PULL>, nc, 0);
+    launch_dependent(moments64_kernel<PULL>, nb, kThreads, sm, s, p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
+    launch_dependent(collide64_kernel<PULL>, nc, kThreads64, sc, s, p, (const P*)src, (P*)dst, (const R*)qfield);
 #else
     launch_dependent(moments_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (R*)qfield);
     launch_dependent(collide_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
@@ -2920,12 +2949,14 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
         if (!reread && p.sched == kSchedRow) {
 #if ELBM_ST == 0 && ELBM_D == 2
             auto kern = p.has_fixed ? fused2d_split_kernel<CAL, true> : fused2d_split_kernel<CAL, false>;
-            constexpr int threads = 128;
+            constexpr int threads = 128, stat = kSplitSmem;
 #else
             auto kern = p.has_fixed ? fused2d_row_kernel<CAL, true> : fused2d_row_kernel<CAL, false>;
-            constexpr int threads = 32;
+            constexpr int threads = 32, stat = kRowSmem;
 #endif
-            return launch_dependent(kern, dim3((unsigned)row_strips(p)), dim3(threads), 0, s, p, (const P*)src, (P*)dst,
+            const long long strips = row_strips(p);
+            const size_t share = spread_smem(kern, strips, stat);
+            return launch_dependent(kern, dim3((unsigned)strips), dim3(threads), share, s, p, (const P*)src, (P*)dst,
                                     (p.nx + kRowW - 1) / kRowW, partials, status);
         } else if (reread || p.sched == kSchedTile) {   // the tile kernel: one 32 x kTY2 tile per CTA, no march
             launch_dependent(fused2d_kernel<kTY2, CAL>, tile2d_grid(p), dim3(TX, kTY2), 0, s, p, (const P*)src, (P*)dst, partials,

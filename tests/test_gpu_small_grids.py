@@ -90,3 +90,27 @@ def test_row_march(E, nx, ny, tz, bc, store):
     for a, b in zip(g.fields(), O.fields(s)):
         assert rel_l2(a, b) <= TOL[store], (store, nx, ny, bc)
     g.close()
+
+
+@pytest.mark.parametrize("store", ["f64", "f32"])
+def test_one_grid_s_share_of_an_sm_beside_another_s(E, store):
+    """The shared memory that spreads a grid's CTAs goes with the grid's size: grids of 1, 2 and 8
+    CTAs to an SM, one more than that, FP64 two passes on either side of their limits, stepped
+    in turn and from graphs captured before the others ran, match each alone."""
+    sizes = [(30, 152), (30, 153), (60, 152), (29, 1216), (152, 128), (153, 128), (190, 205), (389, 400)]
+    cases = [case(nx, ny, (1, 1, 0, 0, 0, 0)) for nx, ny in sizes]
+    alone = []
+    for c in cases:
+        g = E.Solver.from_case(c, store=store)
+        g.step(8)
+        alone.append(g.pop_a.clone())
+        g.close()
+    gs = [E.Solver.from_case(c, store=store) for c in cases]
+    for g in gs[::2]:
+        g.set_step_graph(2)
+    for _ in range(4):
+        for g in gs:
+            g.step(2)
+    for g, a in zip(gs, alone):
+        assert bool((g.pop_a == a).all())
+        g.close()
