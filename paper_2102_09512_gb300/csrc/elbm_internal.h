@@ -235,6 +235,7 @@ struct EnsembleArgs {
     const long long* offset;    // [n] element offset of instance k in both stores
     const int* tile_start;      // [n+1] prefix sums of the instances' tile counts
     const int* tiles_x;         // [n] tiles per row of instance k
+    const int* order;           // [n] row march: the instance of the k-th entry of the two lists above
     int n, ntiles;
     int caloric;                // some instance has a Cv(T) model (selects the kernel form)
     int fixed;                  // some instance has a fixed-state face (likewise)

@@ -2578,10 +2578,11 @@ march2d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
 }
 
 // Compiled with and without fixed-state faces, as march2d_kernel (64 lattices, 8 steps: 7124 us with
-// the face tests always in, 6506 without).
+// the face tests always in, 6506 without, both with segments of 32 rows).
 // Persistent ensemble step on the row march: the work list holds (instance, strip, segment)
-// units (instance k owns units [tile_start[k], tile_start[k+1]), tiles_x[k] strips per
-// segment row); CTA b takes units b, b + gridDim.x, ...  No totals are kept.
+// units (instance order[k] owns units [tile_start[k], tile_start[k+1]), tiles_x[k] strips per
+// segment row, the rows shared evenly between its segments); CTA b takes the b-th unit of every round
+// of gridDim.x, counted from the end in every other round.  No totals are kept.
 // Threads and shared memory of a march CTA: two nodes a thread for the 16-bit stores.
 #if ELBM_ST >= 2 && ELBM_D == 2
 template <int W, int NB> constexpr int march_threads = W / 2;
@@ -2594,14 +2595,11 @@ template <int W, int NB> constexpr size_t march_smem_bytes = March2<W, NB>::smem
 #endif
 template <int W, int NB, bool CAL, bool FIX>
 __global__ void ELBM_ENSEMBLE_BOUNDS(W)
-ensemble_march2d_kernel(const EnsembleArgs a, const P* src, P* __restrict__ dst, int seg,
-                        int* __restrict__ status) {
+ensemble_march2d_kernel(const EnsembleArgs a, const P* src, P* __restrict__ dst, int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char march_smem[];
     wait_for_previous();
     __shared__ int s_start[kMaxEnsemble + 1];
-    __shared__ int s_tx[kMaxEnsemble];
     for (int k = threadIdx.x; k <= a.n; k += blockDim.x) s_start[k] = a.tile_start[k];
-    for (int k = threadIdx.x; k < a.n; k += blockDim.x) s_tx[k] = a.tiles_x[k];
     __syncthreads();
     bool bad = false;
 #if ELBM_ST >= 2 && ELBM_D == 2
@@ -2611,13 +2609,15 @@ ensemble_march2d_kernel(const EnsembleArgs a, const P* src, P* __restrict__ dst,
     acc.zero();
 #endif
     int k = 0;
-    for (int u = blockIdx.x; u < a.ntiles; u += gridDim.x) {
+    for (int u0 = 0, back = 0; u0 < a.ntiles; u0 += gridDim.x, back ^= 1) {
+        const int u = u0 + (back ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
+        if (u >= a.ntiles) continue;
         while (u >= s_start[k + 1]) ++k;   // u increases, so k only moves forward
-        const int local = u - s_start[k];
-        const int bx = local % s_tx[k], by = local / s_tx[k];
-        const KParams& p = a.params[k];
-        const long long off = a.offset[k];
-        const int y0 = by * seg;
+        const int local = u - s_start[k], tx = a.tiles_x[k], inst = a.order[k];
+        const int bx = local % tx, by = local / tx, nseg = (s_start[k + 1] - s_start[k]) / tx;
+        const KParams& p = a.params[inst];
+        const long long off = a.offset[inst];
+        const int seg = (p.ny + nseg - 1) / nseg, y0 = by * seg;
         const PlanesBase pl{src + off, dst + off, (size_t)p.N, src + off};
 #if ELBM_ST >= 2 && ELBM_D == 2
         march2d_pair_segment<W, CAL, FIX>(p, pl, bx * W, y0, min(y0 + seg, p.ny), march_smem, acc, bad);
@@ -3059,27 +3059,27 @@ cudaError_t launch_fused_pf(const KParams& p, const void* src, void* dst, const 
 }
 
 template <bool CAL>
-cudaError_t launch_ensemble_march(const EnsembleArgs& a, const void* src, void* dst, int* status, int seg, int grid,
+cudaError_t launch_ensemble_march(const EnsembleArgs& a, const void* src, void* dst, int* status, int grid,
                                   cudaStream_t s) {
     auto kern = a.fixed ? ensemble_march2d_kernel<kW2, kNBM, CAL, true> : ensemble_march2d_kernel<kW2, kNBM, CAL, false>;
     constexpr size_t smem = march_smem_bytes<kW2, kNBM>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_dependent(kern, dim3(grid), march_threads<kW2, kNBM>, smem, s, a, (const P*)src, (P*)dst, seg, status);
-            if (e != cudaSuccess) return e;
+    e = launch_dependent(kern, dim3(grid), march_threads<kW2, kNBM>, smem, s, a, (const P*)src, (P*)dst, status);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 // Persistent ensemble step and `grid` CTAs: ty = 4, 8 or 16 runs one 32 x ty tile per work
 // unit; ty = kMarchSegs (32, 64 or 128) runs the row march over strips of kW2 nodes and
-// segments of ty rows.
+// segments of about ty rows.
 cudaError_t launch_ensemble(const EnsembleArgs& a, const void* src, void* dst, int* status, int ty, int grid,
                             cudaStream_t s, long long* launches) {
     if constexpr (kD == 2) {
         if (ty > 16) {
             ++*launches;
-            return a.caloric ? launch_ensemble_march<true>(a, src, dst, status, ty, grid, s)
-                             : launch_ensemble_march<false>(a, src, dst, status, ty, grid, s);
+            return a.caloric ? launch_ensemble_march<true>(a, src, dst, status, grid, s)
+                             : launch_ensemble_march<false>(a, src, dst, status, grid, s);
         }
         if (a.caloric) {
             if (ty == 4) launch_dependent(ensemble2d_kernel<4, true>, grid, dim3(TX, 4), 0, s, a, (const P*)src, (P*)dst, status);
