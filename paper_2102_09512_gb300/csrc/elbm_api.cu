@@ -89,7 +89,7 @@ const Ops* pick_ops(int D, int store) {
 constexpr int kMaxWidth = 12;   // widest partial vector: step totals 5, statistics kStatsSums
 static_assert(kStatsSums <= kMaxWidth, "finalize width");
 constexpr int kFinBlocks = 128;
-constexpr int kFinRows = 256;   // rows per CTA that are worth another CTA
+constexpr int kFinRows = 64;   // rows per CTA that are worth another CTA
 
 __device__ __forceinline__ void warp_dd_sum(double& s, double& c) {
 #pragma unroll

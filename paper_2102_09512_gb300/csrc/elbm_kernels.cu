@@ -372,21 +372,36 @@ __global__ void fields_kernel(const __grid_constant__ KParams p, const P* __rest
 // two additions per pair where a sum over each node's moments takes five or more, each of them
 // compensated.  FP32-arithmetic stores: the sums are three-float ones (Tri2) throughout, so no
 // FP64 instruction runs before a CTA's last warp; as an FP64 sum per node the FP64 pipe bounded
-// it (256^3, FP32: 6.08 ms, now 0.66).  FP64 store: plain sums of kTotRun pairs,
-// compensated from there on.  Each CTA writes five sums and their five corrections.
-constexpr int kTotRun = sizeof(R) == 8 ? 16 : 8;   // pairs in flight per thread
+// it (256^3, FP32: 6.08 ms, now 0.56, which is 6.5 TB/s).  FP64 store: sums of kTotRun pairs as
+// integers (FixedSum), compensated from there on (128^3: 0.65 ms, now 0.30; as FP64 sums 0.45).  Runs
+// of 16 pairs and a plane's bounds tested on its last unit alone: with runs of 8, a 64-bit
+// division a unit and five CTAs to an SM it waited for its own address arithmetic (256^3: FP32
+// 0.64 ms, FP16 0.70, now 0.53).  Each CTA writes five sums and their five corrections.
+constexpr int kTotRun = 16;   // pairs in flight per thread
 constexpr int kTotThreads = 256;
+constexpr int kTotCtas = sizeof(R) == 8 ? 1 : 3;   // per SM; FP64: what a thread does once takes the FP64 pipe
 struct TotalsF64 {
     double F = 0, Fc = 0, G = 0, Gc = 0, s[5] = {}, c[5] = {};
     __device__ __forceinline__ void pairs(const R* f, const R* g) {
-        double a = 0, b = 0;
+        dd_add(F, Fc, sum(f));
+        dd_add(G, Gc, sum(g));
+    }
+    static __device__ __forceinline__ double sum(const R* v) {
+        static_assert(kTotRun <= 27, "values that a sum of integers holds");
+        int top = 0;
 #pragma unroll
-        for (int k = 0; k < kTotRun; ++k) {
-            a += f[k];
-            b += g[k];
+        for (int k = 0; k < kTotRun; ++k) top = FixedSum::top_of(top, v[k]);
+        if (!FixedSum::usable(top)) {
+            double a = 0;
+#pragma unroll
+            for (int k = 0; k < kTotRun; ++k) a += v[k];
+            return a;
         }
-        dd_add(F, Fc, a);
-        dd_add(G, Gc, b);
+        top = (top >> 20) + 6;
+        long long a = kTotRun / 2;   // half a unit a value, as in fixed_sums
+#pragma unroll
+        for (int k = 0; k < kTotRun; ++k) a += FixedSum::fixed(v[k], top);
+        return FixedSum::value(a, top);
     }
     __device__ __forceinline__ void plane_end(int i) {
         const double cx = cx_of(i), cy = cy_of(i), cz = cz_of<kD>(i);
@@ -456,29 +471,35 @@ struct TotalsF32 {
         }
     }
 };
-__global__ void __launch_bounds__(kTotThreads, sizeof(R) == 8 ? 4 : 5)
+__global__ void __launch_bounds__(kTotThreads, kTotCtas)
 totals_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int units) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kTotThreads / 32;
     __shared__ double part[kWarps][10];
     std::conditional_t<sizeof(R) == 8, TotalsF64, TotalsF32> tot;
-    int last = -1;
-    for (long long u = blockIdx.x; u < (long long)Q * units; u += gridDim.x) {   // `units` per plane
-        const int i = (int)(u / units);
-        if (i != last && last >= 0) tot.plane_end(last);
-        last = i;
+    // unit `r` of direction i; the N nodes of a plane are at most 2^31
+    int i = 0, r = (int)blockIdx.x;
+    for (; r >= units && i < Q; ++i) r -= units;
+    while (i < Q) {
         // the plane that holds direction i (swapped in the even AA layout)
         const P* __restrict__ b = pop + (size_t)(p.aa == 1 ? Q - 1 - i : i) * (size_t)p.N;
-        const long long n = (u - (long long)i * units) * (kTotThreads * kTotRun) + threadIdx.x;
-        R f[kTotRun], g[kTotRun];
+        const unsigned N = (unsigned)p.N;
+        for (; r < units; r += (int)gridDim.x) {
+            const unsigned n = (unsigned)r * (kTotThreads * kTotRun) + threadIdx.x;
+            R f[kTotRun], g[kTotRun];
+            if (r < units - 1) {
 #pragma unroll
-        for (int k = 0; k < kTotRun; ++k) {
-            const long long m = n + (long long)k * kTotThreads;
-            Cd::dec(m < p.N ? b[m] : Cd::enc(R(0), R(0)), f[k], g[k]);
+                for (int k = 0; k < kTotRun; ++k) Cd::dec(b[n + k * kTotThreads], f[k], g[k]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < kTotRun; ++k)
+                    Cd::dec(n + k * kTotThreads < N ? b[n + k * kTotThreads] : Cd::enc(R(0), R(0)), f[k], g[k]);
+            }
+            tot.pairs(f, g);
         }
-        tot.pairs(f, g);
+        tot.plane_end(i);
+        for (; r >= units && i < Q; ++i) r -= units;
     }
-    if (last >= 0) tot.plane_end(last);
     tot.warp_total(lane, part[warp]);
     __syncthreads();
     if (threadIdx.x < 5) {
@@ -2674,7 +2695,7 @@ constexpr int kTY3 = ELBM_TY3;           // D3Q27 re-read and tensor-copy kernel
 #define ELBM_TYP_F32 8
 #endif
 constexpr int kTYP = (kST == ST_F32) ? ELBM_TYP_F32 : kTY3;
-constexpr int kTotalsBlocks = (sizeof(R) == 8 ? 4 : 5) * 152;   // totals_kernel grid (grid-stride)
+constexpr int kTotalsBlocks = kTotCtas * 152;   // totals_kernel grid (grid-stride)
 // Pipelined D3Q27 kernel per store: two plane buffers.  FP32 pairs make them 145 KB
 // (one CTA per SM, up to 255 registers; a third buffer would leave L1 almost no
 // room and measured 35 % slower); FP16/BF16 pairs are half the size (two CTAs per
