@@ -776,6 +776,7 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
 // thread of the second pass reads before it writes there.  Q~, which neighbours read, goes to
 // the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
 // moments 2.3 times (both with the arithmetic of their time); D2Q9 marches rows instead.
+constexpr int kSms = 152;   // SMs of the device the rules here are for
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
 __global__ void __launch_bounds__(kThreads1D)
@@ -859,12 +860,22 @@ collide64_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict_
     Relax<kD, R, DEV> rx;
     rx.init(rho, T, ux, uy, uz, dq, Dx, Dy, Dz, p);
     const unsigned nn = (unsigned)n;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        R f, g;
+    auto in = [&](int i, R& f, R& g) {
         Cd::dec(*src_ptr(p, src, r, i), f, g);
         if (kD == 2 && ((r.gmask >> i) & 1u)) fixed_pair(p, i, f, g);
-        (dst + (size_t)i * (size_t)N)[nn] = Cd::enc(rx.f(i, f, p), rx.g(i, g, p));
+    };
+    auto out = [&](int i, R f, R g) { (dst + (size_t)i * (size_t)N)[nn] = Cd::enc(f, g); };
+    // (a finite sum rho has finite terms, and T those of rho E).  With one CTA to an SM a warp has its FP64
+    // pipe to itself, and the chains of integers are longer: 24^3 24.5 us a step, in integers 26.3
+    if (gridDim.x > (unsigned)kSms && rx.usable() && finite64(rho) && finite64(T)) {
+        rx.all(in, out);
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            R f, g;
+            in(i, f, g);
+            out(i, rx.f(i, f, p), rx.g(i, g, p));
+        }
     }
 }
 #endif
@@ -2817,7 +2828,7 @@ int max_blocks(const KParams& p) {
 // reuse the first-level cache that this takes away, is slower with it: FP32 1024^2 28.0 -> 35.0;
 // the tiles and the D3Q27 kernel do not change.)  The function's attribute is set to the same value
 // every time: another thread's launch, or a graph captured before, may need more than this one.
-constexpr int kSms = 152, kSmShared = 228 * 1024;
+constexpr int kSmShared = 228 * 1024;
 template <class... Args>
 size_t spread_smem(void (*kern)(Args...), long long ctas, int stat) {
     const long long k = (ctas + kSms - 1) / kSms;

@@ -829,6 +829,48 @@ struct Relax {
     }
 };
 
+// Sums of products of FP64 values in integers: a product of significands of 62 and 63 bits, the upper
+// half of it (three multiplications of 32 bits, the lowest left out), up to four such terms shifted to
+// the exponent of the largest, added, and rounded once.  A term is off by less than 2^-57 of the
+// largest, where FP64 rounds every product and partial sum by up to 2^-53.  Zero counts as 2^-1023.
+// Terms must keep clear of infinity; results below the normal range are zero.
+struct FixedProd {
+    struct Sig { unsigned hi, lo, es; };              // significand; biased exponent, sign in bit 31
+    struct Term { unsigned long long r; unsigned es; };   // value r 2^-59 2^(e - 2046)
+    template <int S>   // 64 - S bits of significand: S = 1 and 2 multiply
+    static __device__ __forceinline__ Sig sig(double x) {
+        const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+        return {(__funnelshift_l(l, h, 11 - S) & ((0x80000000u >> S) - 1u)) | (0x80000000u >> S), l << (11 - S),
+                ((h >> 20) & 0x7ffu) | (h & 0x80000000u)};
+    }
+    static __device__ __forceinline__ Term mul(const Sig& a, const Sig& b) {   // sig<2> by sig<1>
+        const unsigned long long t = (unsigned long long)a.hi * b.lo + (unsigned long long)a.lo * b.hi;
+        return {(unsigned long long)a.hi * b.hi + (t >> 32), a.es + b.es};     // the signs add without carry
+    }
+    static __device__ __forceinline__ Term term(const Sig& b) {   // sig<1>, times one
+        return {(((unsigned long long)b.hi << 32) | b.lo) >> 3, b.es + 1023u};
+    }
+    template <int N>
+    static __device__ __forceinline__ double sum(const Term (&t)[N]) {
+        int top = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) top = max(top, (int)(t[k].es & 0x7fffffffu));
+        long long v = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            unsigned long long r;
+            asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(t[k].r), "r"(top - (int)(t[k].es & 0x7fffffffu)));   // 0 from 64 on
+            v += (long long)r ^ (long long)((int)t[k].es >> 31);
+        }
+        const unsigned long long m = (unsigned long long)(v ^ (v >> 63));
+        const int z = __clzll((long long)m), e = top - 1019 - z;
+        const unsigned long long b = (((m << z) >> 10) + 1ull) >> 1;
+        const unsigned long long bits = (b + ((unsigned long long)(unsigned)(e - 1) << 52)) |
+                                        ((unsigned long long)v & (1ull << 63));
+        return m == 0 || e < 1 ? 0.0 : __longlong_as_double((long long)bits);
+    }
+};
+
 // The same collision in FP64, arranged for the fewest FP64 instructions (the pipe takes one warp
 // instruction per 16 cycles and SM, so their number is the time: D2Q9 about 320 -> 190 a node,
 // D3Q27 about 860 -> 430 with the two passes below).
@@ -924,6 +966,73 @@ struct Relax<D, double, false, CAL> {
         ps[0] = s - o;
         ps[1] = fma(-2.0, s, u2);
         ps[2] = s + o;
+    }
+    // f and g of all directions with the products in integers (in(i, f, g) loads, out(i, f, g)
+    // stores); usable: every factor is finite and moderate.  A direction's f takes two FP64
+    // instructions or some 55 integer ones, g three or four or some 80: all in integers D2Q9 keeps the FP64
+    // pipe 80 % busy (1680 x 1440: 765 us a step all FP64, 644 with g, 580 with both), on D3Q27 a
+    // third of f stays FP64 (128^3: 1330; g 1122, a third of f too 1115, two thirds 1070, all 1129).
+    __device__ __forceinline__ bool usable() const {
+        int top = 0;
+        auto see = [&](double x) { top = max(top, __double2hiint(x) & 0x7fffffff); };
+        see(omw);
+        see(omw1);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            see(X[a]);
+            see(wY[a]);
+            see(gx[a]);
+            see(ax[a]);
+            see(A[a]);
+            see(B[a]);
+            see(hq[a]);
+            if (D == 3) {
+                see(Z[a]);
+                see(gz[a]);
+                see(sz[a]);
+            }
+        }
+        return top < (1023 + 200) << 20;
+    }
+    template <class In, class Out>
+    __device__ __forceinline__ void all(In in, Out out) const {
+        using FP = FixedProd;
+        const FP::Sig o = FP::sig<2>(omw), o1 = FP::sig<2>(omw1);
+        FP::Sig x[3], s[3], h[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            x[a] = FP::sig<2>(X[a]);
+            s[a] = FP::sig<2>(ax[a]);
+            h[a] = FP::sig<2>(gx[a]);
+        }
+#pragma unroll
+        for (int bc = 0; bc < (D == 3 ? 9 : 3); ++bc) {
+            const int b = bc % 3, c = bc / 3;
+            const double yzd = D == 3 ? wY[b] * Z[c] : wY[b];
+            const FP::Sig yz = FP::sig<1>(yzd), q1 = FP::sig<1>(D == 3 ? A[b] * gz[c] : A[b]),
+                          q2 = FP::sig<1>(D == 3 ? fma(A[b], sz[c], B[b] * gz[c]) : B[b]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int i = a + 3 * bc;
+                double f, g;
+                in(i, f, g);
+                const FP::Term tf[2] = {FP::mul(o, FP::sig<1>(f)), FP::mul(x[a], yz)};
+                const FP::Term g0 = FP::mul(o1, FP::sig<1>(g)), g1 = FP::mul(s[a], q1), g2 = FP::mul(h[a], q2);
+                f = (D == 2 || a != 1) ? FP::sum(tf) : fma(omw, f, X[a] * yzd);
+                const int cx = cx_of(i), cy = cy_of(i), cz = cz_of<D>(i);
+                if (cx * cx + cy * cy + cz * cz == 1) {
+                    FP::Sig q = FP::sig<1>(cx != 0 ? hq[0] : (cy != 0 ? hq[1] : hq[2]));
+                    if (cx + cy + cz > 0) q.es ^= 0x80000000u;
+                    if ((q.es & 0x7fffffffu) == 0u) q.es = 0u;   // no unit for the sign of a zero
+                    const FP::Term tg[4] = {g0, g1, g2, FP::term(q)};
+                    g = FP::sum(tg);
+                } else {
+                    const FP::Term tg[3] = {g0, g1, g2};
+                    g = FP::sum(tg);
+                }
+                out(i, f, g);
+            }
+        }
     }
     // i is a compile-time constant after unrolling; the row products are common subexpressions
     __device__ __forceinline__ double f(int i, double fi, const KParams&) const {
