@@ -410,12 +410,13 @@ def sod_measure(E, torch, steps=500, warmup=10, group=50):
 
 
 def aa_measure(E, torch, case, steps, warmup=3):
-    """The single-store (AA) layout on the bench workload: the two-pass schedule updating one
-    store in place (half the population memory), against the two-pass schedule on ping-pong
-    stores; GLUPS and the fraction of the measured HBM peak at the two-pass bytes per update
-    (the populations read twice and written once, plus the Q~ field)."""
+    """The single-store (AA) layout on the bench workload: one store updated in place (half the
+    population memory) by the fused march after a pass over the tiles' edges, against the
+    two-pass schedule on ping-pong stores; GLUPS and the fraction of the measured HBM peak at
+    the bytes per update (AA: the populations read and written once; two-pass: read twice and
+    written once, plus the Q~ field)."""
     peak, _ = _peak_hbm()
-    out = {"grid": [case.nx, case.ny, case.nz], "steps": steps, "schedule": "two-pass"}
+    out = {"grid": [case.nx, case.ny, case.nz], "steps": steps, "schedule": "aa: march in place, pingpong: two-pass"}
     for store in ("f32", "f16dev"):
         for name, layout in (("aa", 1), ("pingpong", 0)):
             try:
@@ -426,7 +427,9 @@ def aa_measure(E, torch, case, steps, warmup=3):
                 out[f"{store}_{name}"] = {"error": str(err)}
                 continue
             glups = case.N / (ms[0] * 1e-3) / 1e9
-            nbytes = 3 * BYTES_PER_UPDATE[store] // 2 + 3 * 4 * 2   # pairs read twice, written once; Q~ out and in
+            nbytes = BYTES_PER_UPDATE[store]
+            if not layout:
+                nbytes = 3 * nbytes // 2 + 3 * 4 * 2   # pairs read twice, written once; Q~ out and in
             out[f"{store}_{name}"] = {"glups": glups, "ms_per_step": ms[0], "hbm_frac": glups * nbytes / peak,
                                       "bytes_per_update": nbytes}
         torch.cuda.empty_cache()

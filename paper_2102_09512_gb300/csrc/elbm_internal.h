@@ -348,15 +348,15 @@ inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW
 // What the default schedule of a D2Q9 grid runs on a device of `sms` SMs, and the row segment of
 // the march.  Measured on 152 SMs, us a step (Sod parameters, zero-gradient x ends):
 //   FP32     strips  tiles  march        FP64   strips  tiles  two passes
-//   800x4      2.6    3.4    5.8         800x4     5.4   11.3      13.6
-//   180^2      3.3    3.8     -          800x20   13.0   17.9      14.4
-//   256^2      4.5    4.6    6.5         128^2    16.0   17.9      14.5
-//   384^2      7.4    5.8    7.8         160^2    18.1   17.9      18.3
-//   512^2     11.6   10.1    9.5         220^2      -    32.9      27.5
-//   724^2     20.6   17.6   14.6         256^2    46.6   33.0      33.0
-//   1024^2      -    37.2   29.3         384^2    94.4   63.2      60.8
-//                                        512^2    173    109       102
-//                                        1448^2     -    848       752   (march 880)
+//   800x4      2.6    3.4    5.8         800x4     5.1   10.3      14.0
+//   180^2      3.3    3.8     -          800x20   11.2   16.1      14.3
+//   256^2      4.5    4.6    6.5         128^2    16.0   16.1      14.3
+//   384^2      7.4    5.8    7.8         160^2    18.1   16.2      18.3
+//   512^2     11.6   10.1    9.5         220^2      -    28.0      24.0
+//   724^2     20.6   17.6   14.6         256^2      -    28.2      27.4
+//   1024^2      -    37.2   29.3         384^2      -    53.2      45.2
+//                                        512^2      -    91.5      72.5
+//                                        1448^2     -     698       495
 // (16-bit stores as FP32).  So: strips while there are at most eight to an SM, tiles while there
 // are at most four, else the march.  FP64: strips while there are at most four to an SM, each
 // of which keeps four warps busy; then the two passes, which the FP64 pipe bounds and no wave of

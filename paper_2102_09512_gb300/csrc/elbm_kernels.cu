@@ -5,16 +5,25 @@
 //   init_kernel          f = f^eq, g = g^eq of (rho, u, T)              (Eqs. 27eq, geq_i)
 //   fields_kernel        rho, u, T of the current populations           (Eqs. density..E)
 //   totals_kernel        FP64 totals of the current state (per-CTA partials)
+//   stats_kernel         turbulence statistics of the current state (per-CTA partials)
 //   moments_kernel       two-pass schedule, pass 1: Q~_aaa field        (Eq. anomalya)
 //   collide_kernel       two-pass schedule, pass 2: pull, collide, store (Eqs. fLBGK, gLBGK)
+//   moments64_kernel, collide64_kernel  the two passes in FP64 (the default of D3Q27 FP64, and of
+//                        D2Q9 FP64 grids beyond the strips and tiles)
+//   fused2d_row_kernel, fused2d_split_kernel  D2Q9 step of a small grid: strips of 30 nodes (FP64:
+//                        four warps share a strip's arithmetic)
 //   fused2d_kernel       D2Q9 one-kernel step: tile + halo moments in shared memory
+//   march2d_kernel, march2d_pair_kernel  D2Q9 row march (the latter: 16-bit stores, two nodes a thread)
+//   ensemble2d_kernel, ensemble_march2d_kernel  persistent steps of an ensemble
 //   fused3d_kernel       D3Q27 one-kernel step: xy tile + halo marching along z, the pulled
 //                        populations of each plane prefetched into shared memory with
-//                        cp.async one plane ahead
-//   moments64_kernel, collide64_kernel  the two passes in FP64 (the default of D3Q27 FP64)
+//                        cp.async one plane ahead; on the single store in place, after
+//                        aa_edges_kernel
+//   fused3d_tma_kernel   the same with tensor copies
 //   fused3d_reread_kernel  D3Q27 one-kernel step without the shared-memory plane buffers:
 //                        the populations of a plane are gathered twice (moments of the
 //                        next plane, then the collision), the second time from L2
+//   aa_moments_kernel, aa_collide_kernel  two passes on the single store
 //
 // Layout: element [i * N + n] holds the pair (f_i, g_i) of direction i at node n.
 // Streaming is "pull": the pair of direction i at node x is read from x - c_i of the
@@ -775,7 +784,8 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
 // the node's own pairs of the first planes of the destination store, which the same node's
 // thread of the second pass reads before it writes there.  Q~, which neighbours read, goes to
 // the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
-// moments 2.3 times (both with the arithmetic of their time); D2Q9 marches rows instead.
+// moments 2.3 times (both with the arithmetic of their time; with the sums and products in
+// integers, FixedSum and FixedProd, 1.07 now, of which the store's traffic takes a third).
 constexpr int kSms = 152;   // SMs of the device the rules here are for
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
