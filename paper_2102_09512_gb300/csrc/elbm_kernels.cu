@@ -785,7 +785,7 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
 // thread of the second pass reads before it writes there.  Q~, which neighbours read, goes to
 // the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
 // moments 2.3 times (both with the arithmetic of their time; with the sums and products in
-// integers, FixedSum and FixedProd, 1.07 now, of which the store's traffic takes a third).
+// integers, FixedSum and FixedProd, 1.07 now, of which the traffic takes 0.46).
 constexpr int kSms = 152;   // SMs of the device the rules here are for
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
