@@ -1666,7 +1666,8 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
         } else {
             Moments<R> hm;
             slot_moments(0, NT + tid, hm, Lite());
-            put_halo(0, anomaly(hm.rho, haxis == 1 ? hm.uy : hm.ux, hm.T));
+            if (haxis == 1) QY(0, hsy, hsx) = anomaly(hm.rho, hm.uy, hm.T);
+            else QX(0, hsy, hsx) = anomaly(hm.rho, hm.ux, hm.T);
         }
     }
 
@@ -1711,7 +1712,8 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
             } else {
                 Moments<R> hm;
                 slot_moments(sn, NT + tid, hm, Lite());
-                put_halo(bq ^ 1, anomaly(hm.rho, haxis == 1 ? hm.uy : hm.ux, hm.T));
+                if (haxis == 1) QY(bq ^ 1, hsy, hsx) = anomaly(hm.rho, hm.uy, hm.T);
+                else QX(bq ^ 1, hsy, hsx) = anomaly(hm.rho, hm.ux, hm.T);
             }
         }
 
@@ -1732,25 +1734,18 @@ fused3d_kernel(const __grid_constant__ KParams p, const __grid_constant__ DirPla
             node_totals(m_cur, m_cur.rE, v);
             acc.add(v);
             // collide and store pair by pair, decoding each just before its update
+            Relax<kD, R, DEV, CAL> rx;
+            rx.init(m_cur, Dx, Dy, Dz, p);
             const unsigned n = (unsigned)node_index(p, x, y, z);
             PullRows w;   // AA from L0: the new pairs go to where opposite directions are pulled from
             if constexpr (AA == 1) pull_rows(p, x, y, z, w);
             auto out = [&](int i) { return AA == 0 ? pl.dst[i] + n : AA == 2 ? pl.dst[opp(i)] + n : aa_slot(pl, w, i, opp(i)); };
-            if constexpr (DEV) {
-                RelaxDev<CAL> rx;
-                rx.init(m_cur, Dx, Dy, Dz, p);
-                rx.apply([&](int i, R& f, R& g) { Cd::dec(pk[i], f, g); },
-                         [&](int i, R f, R g) { store_pair(out(i), Cd::enc(f, g)); });
-            } else {
-                Relax<kD, R, DEV, CAL> rx;
-                rx.init(m_cur, Dx, Dy, Dz, p);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    R f, g;
-                    Cd::dec(pk[i], f, g);
-                    const float2 o = rx.fg(i, make_float2(f, g), p);
-                    store_pair(out(i), Cd::enc(o.x, o.y));
-                }
+            for (int i = 0; i < Q; ++i) {
+                R f, g;
+                Cd::dec(pk[i], f, g);
+                const float2 o = rx.fg(i, make_float2(f, g), p);
+                store_pair(out(i), Cd::enc(o.x, o.y));
             }
         }
         m_cur = m_next;
@@ -2036,22 +2031,15 @@ fused3d_tma_kernel(const __grid_constant__ KParams p, const __grid_constant__ Di
             R v[5];
             node_totals(m_cur, m_cur.rE, v);
             acc.add(v);
+            Relax<kD, R, DEV, CAL> rx;
+            rx.init(m_cur, Dx, Dy, Dz, p);
             const unsigned n = (unsigned)node_index(p, x, y, z);
-            if constexpr (DEV) {
-                RelaxDev<CAL> rx;
-                rx.init(m_cur, Dx, Dy, Dz, p);
-                rx.apply([&](int i, R& f, R& g) { Cd::dec(pk[i], f, g); },
-                         [&](int i, R f, R g) { store_pair(pl.dst[i] + n, Cd::enc(f, g)); });
-            } else {
-                Relax<kD, R, DEV, CAL> rx;
-                rx.init(m_cur, Dx, Dy, Dz, p);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    R f, g;
-                    Cd::dec(pk[i], f, g);
-                    const float2 o = rx.fg(i, make_float2(f, g), p);
-                    store_pair(pl.dst[i] + n, Cd::enc(o.x, o.y));
-                }
+            for (int i = 0; i < Q; ++i) {
+                R f, g;
+                Cd::dec(pk[i], f, g);
+                const float2 o = rx.fg(i, make_float2(f, g), p);
+                store_pair(pl.dst[i] + n, Cd::enc(o.x, o.y));
             }
         }
         m_cur = m_next;
@@ -2377,6 +2365,12 @@ template <int W, bool CAL, bool FIX, class PL>
 __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL& pl, int x0, int y0, int ye,
                                                      unsigned char* smem, float2 acc[4], bool& bad) {
     using MC = MarchPair<W>;
+    // Which of two products each sum of products rounds by itself (ALT) is that of the one-node march, bit
+    // for bit: it differed between the lattice alone without fixed faces and the others, and
+    // between a segment's first row and the rest (first).
+    constexpr bool kAlone = !FIX && std::is_same<PL, PlanesParam>::value;
+    using First = std::true_type;
+    using Later = std::false_type;
     constexpr int NS = MC::NS, QW = MC::QW;
     P* buf = reinterpret_cast<P*>(smem);                            // [2][Q][NS]
     float* qxs = reinterpret_cast<float*>(smem + MC::buf_bytes);    // [2][QW]
@@ -2420,24 +2414,28 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
         }
         cp_async_commit();
     };
-    // stored pairs of one node with the fixed state's in place of those marked in gm
-    auto node_fixed = [&](const P* v, int stride, unsigned gm, Moments<float>& m) {
+    // one node's stored pairs, with the fixed state's in place of those marked in gm
+    auto node_fixed = [&](const P* v, unsigned gm, Moments<float>& m) {
+        if (!gm) {
+            node_moments_stored<kD, kST, true, CAL>([&](int i) { return v[i * NS]; }, p, m);
+            return;
+        }
         float f[Q], g[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            Cd::dec(v[i * stride], f[i], g[i]);
+            Cd::dec(v[i * NS], f[i], g[i]);
             if ((gm >> i) & 1u) fixed_pair(p, i, f[i], g[i]);
         }
         node_moments<kD, float, true, true, CAL>(f, g, p, m);
     };
-    auto pair_moments = [&](int sb, int y, MomentsPair& m) {
+    auto pair_moments = [&](int sb, int y, MomentsPair& m, auto first) {
         const P* bb = buf + (size_t)sb * Q * NS + 2 * t;
         if (FIX) {
             const unsigned g0 = fixed_mask<FIX>(p, x, y), g1 = fixed_mask<FIX>(p, x + 1, y);
             if (g0 | g1) {
                 Moments<float> a, b;
-                node_fixed(bb, NS, g0, a);
-                node_fixed(bb + 1, NS, g1, b);
+                node_fixed(bb, g0, a);
+                node_fixed(bb + 1, g1, b);
                 m.rho = make_float2(a.rho, b.rho);
                 m.ux = make_float2(a.ux, b.ux);
                 m.uy = make_float2(a.uy, b.uy);
@@ -2452,7 +2450,7 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
         uint2 raw[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) raw[i] = *reinterpret_cast<const uint2*>(bb + i * NS);
-        node_moments_pair<kD, kST, CAL>(
+        node_moments_pair<kST, CAL, kAlone && (CAL || !decltype(first)::value)>(
             [&](int i, int k) { return *reinterpret_cast<const P*>(k ? &raw[i].y : &raw[i].x); }, p, m);
     };
     auto halo_q = [&](int sb, int y) {
@@ -2460,21 +2458,21 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
         const P* bb = buf + (size_t)sb * Q * NS + W + t;
         Moments<float> m;
         const unsigned gm = fixed_mask<FIX>(p, hx, y);
-        if (FIX && gm) node_fixed(bb, NS, gm, m);
+        if (FIX && gm) node_fixed(bb, gm, m);
         else node_moments_stored<kD, kST, false, CAL>([&](int i) { return bb[i * NS]; }, p, m);
         return anomaly(m.rho, m.ux, m.T);
     };
     float* const my_qx = qxs + 2 + 2 * t;
     float* const halo_qx = qxs + (t == 0 ? 1 : xl + 3);
     // Q~ of this thread's nodes: xxx to shared memory row b, yyy returned
-    auto put_q = [&](int b, const MomentsPair& m, bool x_too) {
+    auto put_q = [&](int b, const MomentsPair& m, bool x_too, auto first) {
         const float2 c = anomaly_c(m.T);
         if (x_too) {
-            const float2 v = anomaly2(m.rho, m.ux, c);
+            const float2 v = anomaly2<kAlone && !decltype(first)::value>(m.rho, m.ux, c);
             if (act1) *reinterpret_cast<float2*>(my_qx + b * QW) = v;
             else my_qx[b * QW] = v.x;
         }
-        return anomaly2(m.rho, m.uy, c);
+        return anomaly2<kAlone && decltype(first)::value>(m.rho, m.uy, c);
     };
 
     float2 qy_prev = both(0.f), qy_cur = both(0.f), qy_next = both(0.f);
@@ -2493,8 +2491,8 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
     cp_async_wait_pending<1>();
     __syncthreads();
     if (act0) {
-        pair_moments(0, y0, m_cur);
-        qy_cur = put_q(0, m_cur, true);
+        pair_moments(0, y0, m_cur, First());
+        qy_cur = put_q(0, m_cur, true, First());
     }
     if (has_halo) halo_qx[0] = halo_q(0, y0);
 
@@ -2515,8 +2513,8 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
             if (fixed_faces && beyond_fixed(p, 1, y + 1, p.ny)) {
                 qy_next = both(fixed_Q(p, 1));   // the last row of the grid: nothing after it
             } else {
-                pair_moments(sn, yn, m_next);
-                qy_next = put_q(sn, m_next, !last);
+                pair_moments(sn, yn, m_next, Later());
+                qy_next = put_q(sn, m_next, !last, Later());
             }
         }
         if (!last && has_halo) halo_qx[sn * QW] = halo_q(sn, yn);
@@ -2534,8 +2532,8 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
             acc[1] = fma2(m_cur.rho, m_cur.ux, acc[1]);
             acc[2] = fma2(m_cur.rho, m_cur.uy, acc[2]);
             acc[3] = add2(acc[3], m_cur.rE);
-            RelaxPair<kD, CAL> rx;
-            rx.init(m_cur, Dx, Dy, both(0.f), p);
+            RelaxPair<CAL> rx;
+            rx.init(m_cur, Dx, Dy, p);
             const unsigned n = (unsigned)(x + p.nx * y);
             const unsigned g0 = fixed_mask<FIX>(p, x, y), g1 = fixed_mask<FIX>(p, x + 1, y);
 #pragma unroll
@@ -2545,8 +2543,8 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
                 Cd::dec(*reinterpret_cast<const P*>(&pk[i].y), f.y, g.y);
                 if ((g0 >> i) & 1u) fixed_pair(p, i, f.x, g.x);
                 if ((g1 >> i) & 1u) fixed_pair(p, i, f.y, g.y);
-                f = rx.f(i, f);
-                g = rx.g(i, g);
+                f = rx.f(i, f, p);
+                g = rx.g(i, g, p);
                 const P o0 = Cd::enc(f.x, g.x), o1 = Cd::enc(f.y, g.y);
                 P* d = pl.d(i) + n;
                 if (even) {
@@ -2568,8 +2566,8 @@ __device__ __forceinline__ void march2d_pair_segment(const KParams& p, const PL&
     __syncthreads();   // the shared buffers are reused by the next segment of a persistent CTA
 }
 // Sixteen warps of 128 registers per SM (uncapped 145 registers, twelve warps: 4096^2 272 us a
-// step, twenty warps: 598, it spills).  4096^2, FP16: 301 us with a node a thread, 249 with two;
-// strips of 128 nodes 269, 512 nodes 253.
+// step, twenty warps: 598, it spills; strips of 128 nodes 269, 512 nodes 253, 256 nodes 249, all with
+// an arithmetic that is not used any more, see elbm_pair.cuh).
 template <int W> constexpr int kPairCtas = 1024 / W;
 template <int W, bool CAL, bool FIX>
 __global__ void __launch_bounds__(W / 2, kPairCtas<W>)

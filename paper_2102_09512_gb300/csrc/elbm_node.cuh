@@ -801,6 +801,7 @@ struct Relax {
         const R A = w1r * gy[b] * gz[c];
         const R B = w1r * (sy[b] * gz[c] + gy[b] * sz[c]);
         float2 t = make_float2(X[a] * yz, fma(ax[a], A, gx[a] * B));
+        if constexpr (DEV) t = __ffma2_rn(make_float2(-w, -w1), p.rest2[i], t);
         float2 o = __ffma2_rn(make_float2(omw, omw1), v, t);
         const int cx = cx_of(i), cy = cy_of(i), cz = cz_of<D>(i);
         if (cx * cx + cy * cy + cz * cz == 1) {
@@ -1054,148 +1055,16 @@ struct Relax<D, double, false, CAL> {
     }
 };
 
-// The collision of the deviation stores on D3Q27, one node in two-lane FP32 instructions (the
-// kernel of these stores is bound by instruction issue; 256^3, FP16: 820 -> 790 us a step, BF16
-// 884 -> 807).  The D2Q9 kernels outside the march wait for memory and keep Relax.  Lanes are
-// opposite directions along z (c_z = -1, +1 for each c_x, c_y), then along y in the plane
-// c_z = 0: they share the factor of c_x, and their row products come as a pair.  The rest
-// state's term -w r_i depends on the number of zero components of c_i alone and is added where
-// the products are (three instructions a direction for f and g together, and one each for the
-// relaxation, both for two directions).  Factors and rates as in the FP64 form above.
-template <bool CAL>
-struct RelaxDev {
-    float2 omw, omw1, X[3], gx[3], ax[3];     // both lanes alike
-    float2 rf[4], rg[4];                      // -w and -w1 times the rest pair, by zero components
-    float wY[3], A[3], B[3];
-    float2 Ze, gze, sze;                      // factors of c_z = -1 and +1; Z1, gz1, sz1: of c_z = 0
-    float Z1, gz1, sz1;
-    float hq[3];
-
-    static __device__ __forceinline__ constexpr int zeros(int i) {
-        return (cx_of(i) == 0) + (cy_of(i) == 0) + (cz_of<3>(i) == 0);
-    }
-    __device__ __forceinline__ void init(const Moments<float>& m, float Dx, float Dy, float Dz, const KParams& p) {
-        const float rho = m.rho, T = m.T, ux = m.ux, uy = m.uy, uz = m.uz;
-        float mu = p.f_mu0;
-        if (p.powlaw) mu *= qpow(T * p.f_invT0, p.f_mu_exp);
-        const float P = rho * T, PrP = p.f_Pr * P;
-        const float t = qdiv(P, fmaf(2.f, mu, P)), t1 = qdiv(PrP, fmaf(2.f, mu, PrP));   // w/2, w1/2
-        const float k = qdiv(mu, rho * P);
-        omw = both(fmaf(-2.f, t, 1.f));
-        omw1 = both(fmaf(-2.f, t1, 1.f));
-#pragma unroll
-        for (int z = 0; z < 4; ++z) {
-            constexpr int rep[4] = {0, 1, 4, 13};   // a direction with z zero components
-            rf[z] = both(-2.f * t * p.rest2[rep[z]].x);
-            rg[z] = both(-2.f * t1 * p.rest2[rep[z]].y);
-        }
-        const float rs = 0.25f * rho, wr = t * rs, w1r = t1 * rs;
-        const float T25 = 2.5f * T, TT = T * T;
-        {   // c_x
-            const float u2 = ux * ux, Pa = T + u2, Pe = fmaf(k, Dx, Pa);
-            const float o = ux * fmaf(0.5f, u2, T), s = fmaf(u2, fmaf(0.5f, u2, T25), TT);
-            const float U = U_of_T<float, CAL>(T, p);
-            const float g3[3] = {Pa - ux, fmaf(-2.f, Pa, 2.f), Pa + ux};
-            const float x3[3] = {Pe - ux, fmaf(-2.f, Pe, 2.f), Pe + ux};
-            const float s3[3] = {s - o, fmaf(-2.f, s, u2), s + o};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                X[a] = both(x3[a]);
-                gx[a] = both(g3[a]);
-                ax[a] = both(fmaf(U, g3[a], s3[a]));
-            }
-        }
-        // c_y and, in the other lane, c_z
-        const float2 u = make_float2(uy, uz), u2 = mul2(u, u), Pa = add2(both(T), u2);
-        const float2 Pe = fma2(both(k), make_float2(Dy, Dz), Pa);
-        const float2 o = mul2(u, fma2(u2, both(0.5f), both(T)));
-        const float2 s = fma2(u2, fma2(u2, both(0.5f), both(T25)), both(TT));
-        const float2 F0 = sub2(Pe, u), F1 = fma2(Pe, both(-2.f), both(2.f)), F2 = add2(Pe, u);
-        const float2 g0 = sub2(Pa, u), g1 = fma2(Pa, both(-2.f), both(2.f)), g2 = add2(Pa, u);
-        const float2 s0 = sub2(s, o), s1 = fma2(s, both(-2.f), u2), s2 = add2(s, o);
-        wY[0] = wr * F0.x; wY[1] = wr * F1.x; wY[2] = wr * F2.x;
-        A[0] = w1r * g0.x; A[1] = w1r * g1.x; A[2] = w1r * g2.x;
-        B[0] = w1r * s0.x; B[1] = w1r * s1.x; B[2] = w1r * s2.x;
-        Ze = make_float2(F0.y, F2.y);
-        gze = make_float2(g0.y, g2.y);
-        sze = make_float2(s0.y, s2.y);
-        Z1 = F1.y;
-        gz1 = g1.y;
-        sz1 = s1.y;
-        // (omega - omega_1)/2 (q* - q^eq), q* - q^eq = u . (P - rho T I - rho u u + div Q~ / 2)
-        const float jx = rho * ux, jy = rho * uy, h = t - t1;
-        const float dxx = fmaf(-jx, ux, fmaf(0.5f, Dx, m.Pxx - P)), dyy = fmaf(-jy, uy, fmaf(0.5f, Dy, m.Pyy - P));
-        const float dxy = fmaf(-jx, uy, m.Pxy);
-        const float dxz = fmaf(-jx, uz, m.Pxz), dyz = fmaf(-jy, uz, m.Pyz);
-        const float dzz = fmaf(-(rho * uz), uz, fmaf(0.5f, Dz, m.Pzz - P));
-        hq[0] = h * fmaf(uz, dxz, fmaf(uy, dxy, ux * dxx));
-        hq[1] = h * fmaf(uz, dyz, fmaf(uy, dyy, ux * dxy));
-        hq[2] = h * fmaf(uz, dzz, fmaf(uy, dyz, ux * dxz));
-    }
-    // load(i, f, g) gives the raw stored values of direction i, store(i, f, g) takes the new ones
-    template <class Load, class Store>
-    __device__ __forceinline__ void apply(Load load, Store store) const {
-        auto two = [&](int i, int j, int a, float2 yz, float2 q1, float2 q2, bool unit, float corr) {
-            float2 f, g;
-            load(i, f.x, g.x);
-            load(j, f.y, g.y);
-            const int z = zeros(i);
-            f = fma2(omw, f, fma2(X[a], yz, rf[z]));
-            g = fma2(omw1, g, fma2(ax[a], q1, fma2(gx[a], q2, rg[z])));
-            if (unit) g = add2(g, make_float2(corr, -corr));   // +-1 along the lanes' axis
-            store(i, f.x, g.x);
-            store(j, f.y, g.y);
-        };
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const float2 yz = mul2(both(wY[b]), Ze), q1 = mul2(both(A[b]), gze);
-            const float2 q2 = fma2(both(A[b]), sze, mul2(both(B[b]), gze));
-#pragma unroll
-            for (int a = 0; a < 3; ++a) two(a + 3 * b, a + 3 * b + 18, a, yz, q1, q2, a == 1 && b == 1, hq[2]);
-        }
-        constexpr int mid = 9;   // c_z = 0
-        float yz[3], q1[3], q2[3];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            yz[b] = wY[b] * Z1;
-            q1[b] = A[b] * gz1;
-            q2[b] = fmaf(A[b], sz1, B[b] * gz1);
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            two(mid + a, mid + a + 6, a, make_float2(yz[0], yz[2]), make_float2(q1[0], q1[2]),
-                make_float2(q2[0], q2[2]), a == 1, hq[1]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const int i = mid + 3 + a, z = zeros(i);
-            float f, g;
-            load(i, f, g);
-            f = fmaf(omw.x, f, fmaf(X[a].x, yz[1], rf[z].x));
-            g = fmaf(omw1.x, g, fmaf(ax[a].x, q1[1], fmaf(gx[a].x, q2[1], rg[z].x)));
-            if (a == 0) g += hq[0];
-            if (a == 2) g -= hq[0];
-            store(i, f, g);
-        }
-    }
-};
-
 // One collision in place on the raw stored values f, g.
 template <int D, typename R, bool DEV, bool CAL = true>
 __device__ __forceinline__ void collide(R* f, R* g, const Moments<R>& m, R Dx, R Dy, R Dz,
                                         const KParams& p) {
-    if constexpr (DEV && D == 3) {
-        RelaxDev<CAL> r;
-        r.init(m, Dx, Dy, Dz, p);
-        r.apply([&](int i, float& a, float& b) { a = f[i]; b = g[i]; },
-                [&](int i, float a, float b) { f[i] = a; g[i] = b; });
-    } else {
-        Relax<D, R, DEV, CAL> r;
-        r.init(m, Dx, Dy, Dz, p);
+    Relax<D, R, DEV, CAL> r;
+    r.init(m, Dx, Dy, Dz, p);
 #pragma unroll
-        for (int i = 0; i < Lat<D>::Q; ++i) {
-            f[i] = r.f(i, f[i], p);
-            g[i] = r.g(i, g[i], p);
-        }
+    for (int i = 0; i < Lat<D>::Q; ++i) {
+        f[i] = r.f(i, f[i], p);
+        g[i] = r.g(i, g[i], p);
     }
 }
 
