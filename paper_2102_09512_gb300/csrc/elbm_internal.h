@@ -310,15 +310,16 @@ constexpr int kShortestSegment = 1;
 inline int choose_segment(double tiles, int nplanes, int sms, int per_sm, int fallback,
                           int shortest = kShortestSegment) {
     if (sms <= 0 || per_sm <= 0) return fallback < nplanes ? fallback : nplanes;
+    // One pass over the lengths, longest first: those that some number of equal segments gives.  Once
+    // the fullest wave could not lift a shorter length above the best, it stops: an allocation-free
+    // step plans on every call, and a loop over the segment counts took 0.46 ms at 65536 rows.
     const double slots = (double)sms * per_sm;
-    const int lo = nplanes < shortest ? nplanes : shortest, hi = 128;
+    const int lo = nplanes < shortest ? nplanes : shortest, hi = nplanes < 128 ? nplanes : 128;
     int best = fallback < nplanes ? fallback : nplanes;
     double best_score = -1.0;
-    for (int nseg = 1; nseg <= nplanes; ++nseg) {
-        const int tz = (nplanes + nseg - 1) / nseg;
-        if (tz > hi) continue;
-        if (tz < lo) break;
+    for (int tz = hi; tz >= lo && best_score + 1e-9 < tz / (tz + 2.0); --tz) {
         const int ns = (nplanes + tz - 1) / tz;
+        if ((nplanes + ns - 1) / ns != tz) continue;   // ns equal segments are shorter
         const double waves = tiles * ns / slots;
         const double fill = waves / std::ceil(waves);
         const double score = fill * tz / (tz + 2.0);
