@@ -544,13 +544,16 @@ totals_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doub
 constexpr int kStats = kStatsSums;
 template <int DD>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
-stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int tz) {
+stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int tz,
+             unsigned tiles_x, unsigned tiles_y) {
     constexpr int TX = 32, TY = 8, NT = TX * TY;
     __shared__ R us[2][DD][TY + 2][TX + 2];
     __shared__ double part[NT / 32][kStats];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int zb = blockIdx.z * tz, ze = min(zb + tz, p.nz);
+    // columns in one dimension of the grid: the other two hold 65535 CTAs, and grids may be taller
+    const unsigned row = blockIdx.x / tiles_x, seg = row / tiles_y;
+    const int x0 = (int)(blockIdx.x - row * tiles_x) * TX, y0 = (int)(row - seg * tiles_y) * TY;
+    const int zb = (int)seg * tz, ze = min(zb + tz, p.nz);
     const int x = x0 + tx, y = y0 + ty;
     const bool active = x < p.nx && y < p.ny;
     const int xl = min(x0 + TX, p.nx) - 1 - x0, yl = min(y0 + TY, p.ny) - 1 - y0;
@@ -703,7 +706,7 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
         for (int w = 0; w < NT / 32; ++w) v += part[w][k];
         if (quad) v *= 0.25;
         if (tid == 10) v *= kF64 || !p.powlaw ? p.mu0 : p.mu0 * pow(p.T0, -p.mu_exp);
-        partials[(size_t)kStats * (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) + tid] = v;
+        partials[(size_t)kStats * blockIdx.x + tid] = v;
     }
 }
 
@@ -3171,10 +3174,10 @@ cudaError_t launch_stats(const KParams& p, const void* pop, double* partials, in
     const long long most = blocks_1d_of(p.N) > kTotalsBlocks ? blocks_1d_of(p.N) : kTotalsBlocks;
     int tz = choose_segment((double)tx * ty, p.nz, 152, 2, 32);
     while (tz < p.nz && (long long)tx * ty * ((p.nz + tz - 1) / tz) > most) tz = tz < p.nz / 2 ? 2 * tz : p.nz;
-    const dim3 grid(tx, ty, (p.nz + tz - 1) / tz);
-    stats_kernel<kD><<<grid, dim3(32, 8), 0, s>>>(p, (const P*)pop, partials, tz);
+    const long long grid = (long long)tx * ty * ((p.nz + tz - 1) / tz);
+    stats_kernel<kD><<<(unsigned)grid, dim3(32, 8), 0, s>>>(p, (const P*)pop, partials, tz, (unsigned)tx, (unsigned)ty);
     ++*launches;
-    *nblocks = (int)(grid.x * grid.y * grid.z);
+    *nblocks = (int)grid;
     return cudaGetLastError();
 }
 
