@@ -340,6 +340,13 @@ inline int choose_rows(const KParams& k, int sms, int per_sm, int fallback, int 
     return choose_segment((double)((k.nx + width - 1) / width), k.ny, sms, per_sm, fallback);
 }
 
+// Launches hold at most 65535 CTAs in their second and third dimension: whether the marching kernels
+// (D3Q27: tiles of `ty` rows) take a grid.  The one-dimensional two passes take any.
+inline bool march_launches(const KParams& k, int D, int ty) {
+    const long long y = D == 3 ? ((long long)k.ny + ty - 1) / ty : ((long long)k.ny + k.tz - 1) / k.tz;
+    return y <= 65535 && (D == 2 || ((long long)k.nz + k.tz - 1) / k.tz <= 65535);
+}
+
 // D2Q9 small-grid kernels: a strip of kRowW nodes of a row per CTA, kRowMost strips at most
 // (one partial vector each).
 constexpr int kRowW = 30;

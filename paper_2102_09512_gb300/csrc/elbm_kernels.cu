@@ -2941,7 +2941,7 @@ cudaError_t launch_aa_march(const KParams& p, void* A, void* qfield, double* par
 cudaError_t launch_step_aa(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
                            cudaStream_t s, long long* launches, int from_l1, const CUtensorMap* pmap) {
     *launches += 2;
-    if (kD == 3 && kPipe && (double)p.N * Q * sizeof(P) > 64e6)
+    if (kD == 3 && kPipe && (double)p.N * Q * sizeof(P) > 64e6 && march_launches(p, kD, kTYP))
         return launch_aa_march<kD>(p, A, qfield, partials, nblocks, status, s, from_l1, pmap);
     const unsigned nb = blocks_1d(p.N);
     if (from_l1) {

@@ -149,7 +149,8 @@ extern "C" int elbm_step_noalloc(const elbm_params* prm, const void* src, void* 
         else k.tz = choose_tz(k, ops->fused_tile_y, sms, per_sm, k.tz);
         // the fused kernels' partials may run into the Q~ field, which they do not use
         const size_t room = (kNoallocScratchBytes - lay.partials) / (5 * sizeof(double));
-        if (k.sched != kSchedTwoPass && (size_t)ops->max_blocks(k) <= room) {
+        const bool fits = k.sched != kSchedMarch || march_launches(k, D, ops->fused_tile_y);
+        if (k.sched != kSchedTwoPass && fits && (size_t)ops->max_blocks(k) <= room) {
             const cudaError_t e = ops->step_fused(k, src, dst, (double*)(s + lay.partials), &nb, nullptr, st, &launches);
             return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA;
         }
