@@ -111,11 +111,11 @@ typedef enum {
  * step parity (after an even number of steps the pairs of a node sit at the node with each
  * direction in the opposite direction's plane; after an odd number, each pair sits at the
  * node it streams to next): the first kernel of a step writes Q~ (of every node; D3Q27 with
- * FP32 arithmetic and more than 64 MB of store: of the nodes at the faces of the second
- * one's tiles), the second reads and writes exactly the slots each node read, so no two
- * threads touch one slot.  Half the population memory (D3Q27 FP32 at 1024^3: 232 GB instead
- * of 464 GB), 1.5x the bytes per update of the fused schedule.  Periodic grids only (a zero-gradient or fixed
- * face makes two nodes read one slot that one of them writes). */
+ * FP32 arithmetic, where the store is larger than some 64 MB and fills the 32 x 8 tiles well
+ * enough: of the nodes at the faces of the second one's tiles), the second reads and writes
+ * exactly the slots each node read, so no two threads touch one slot.  Half the population
+ * memory (D3Q27 FP32 at 1024^3: 232 GB instead of 464 GB).  Periodic grids only (a
+ * zero-gradient or fixed face makes two nodes read one slot that one of them writes). */
 typedef enum { ELBM_LAYOUT_PINGPONG = 0, ELBM_LAYOUT_AA = 1 } elbm_layout;
 
 typedef struct {
@@ -232,7 +232,8 @@ int elbm_set_kernel(elbm_handle *h, int kernel);
  * planes of prologue); a tuning knob, results agree to rounding.  D2Q9 grids of up to
  * eight 30-node strips or four 32 x 8 tiles per SM, and FP64 ones, run the fused schedule
  * without the march (see elbm_kernel); setting a segment length here selects the march for
- * any D2Q9 grid.  No effect on the default schedule of D3Q27 FP64. */
+ * any D2Q9 grid, and for the AA store of a D3Q27 grid above 64 MB in FP32 arithmetic
+ * (see elbm_layout).  No effect on the default schedule of D3Q27 FP64. */
 int elbm_set_tile_z(elbm_handle *h, int tz);
 
 /* Raw copy of the current population store (pop_bytes) to or from host memory,
@@ -264,10 +265,11 @@ int elbm_velocity(int lattice, int i, int c[3]);
 
 /* One time step, src -> dst, for callers that cannot allocate device memory (for example
  * a solver embedded in an application that owns the whole device memory pool and lends
- * the library only the populations it updates).  Grids below 2^14 nodes run the two-pass
- * schedule, larger ones the default schedule of a handle (results agree to rounding).  No handle and no auxiliary buffer: the scratch this step needs (the Q~
- * field and the per-CTA partials) lives in a fixed static device
- * array of 16 MiB that every GPU loading the library holds until the process exits.
+ * the library only the populations it updates).  Grids below 2^14 nodes, and those that leave
+ * many threads of the marching kernels' tiles without a node, run the two-pass schedule, others
+ * the default schedule of a handle (results agree to rounding).  No handle and no auxiliary
+ * buffer: the scratch this step needs (the Q~ field and the per-CTA partials) lives in a
+ * fixed static device array of 16 MiB that every GPU loading the library holds until the process exits.
  * The paper has no counterpart; this is an interface choice of the library.
  *   params  problem statement, validated as by elbm_create;
  *   src     current population store (device, pop_bytes, 256-byte aligned, read);

@@ -626,6 +626,7 @@ int elbm_set_tile_z(elbm_handle* h, int tz) {
     const int planes = h->D == 3 ? h->prm.nz : h->prm.ny;   // the marched axis
     k.tz = tz < planes ? tz : planes;
     if (h->D == 2) k.sched = kSchedMarch;   // an explicit row segment selects the row march
+    else if (h->layout == ELBM_LAYOUT_AA) k.sched = kSchedSegment;   // and the single store's march above 64 MB
     if (h->ops->max_blocks(k) > h->aux.max_blocks) return ELBM_ERR_ARG;   // partials would not fit
     h->kp.tz = k.tz;
     h->kp.sched = k.sched;

@@ -347,6 +347,42 @@ inline bool march_launches(const KParams& k, int D, int ty) {
     return y <= 65535 && (D == 2 || ((long long)k.nz + k.tz - 1) / k.tz <= 65535);
 }
 
+// Share of the threads of tiles of t nodes that an axis of n nodes fills.
+inline double axis_fill(int n, int t) { return (double)n / ((double)((n + t - 1) / t) * t); }
+
+// Whether the march of the D3Q27 single store (a pass over the tiles' edges, then the march in place) beats
+// the two passes: a marched tile costs the same however few of its 32 x `ty` threads have nodes, and
+// below some 64 MB the two passes' second one finds the store in the cache.  us a step, march
+// and two passes, with the store and the share of the threads that have nodes:
+//   FP32  64^3  57 MB 1.00   32.6  31.2     FP16  64^3       28 MB 1.00   24.0  25.8
+//   64x64x80    71 MB 1.00   36.0  37.0           100x100x60 65 MB 0.75   53.4  53.7
+//   64x64x96    85 MB 1.00   43.0  48.0           96^3       96 MB 1.00   60.1  86.1
+//   72^3        81 MB 0.75   49.5  43.9           65x65x130  59 MB 0.61   52.3  50.7
+//   65x65x130  119 MB 0.61   77.1  81.3           100^3     108 MB 0.75   88.0  99.5
+//   100^3      216 MB 0.75    141   144           16x16x4000 111 MB 0.50   112   104
+//   16x16x4000 221 MB 0.50    167   146           33x33x600  71 MB 0.43   77.8  59.1
+//   8x8x10000  138 MB 0.25    195    95           8x8x10000  69 MB 0.25    139    57
+inline bool aa_march_pays(const KParams& k, int ty, double store_bytes) {
+    const double fill = axis_fill(k.nx, 32) * axis_fill(k.ny, ty);
+    return fill >= 0.6 && fill * store_bytes > 64e6;
+}
+
+// The same for the allocation-free step from kNoallocFused nodes on, whose two passes need no more
+// scratch than the march (elbm_noalloc.cu).  us a step, march and two passes:
+//   FP32  32^3        1.00   7.9   9.0     FP16   8.2   8.1      D2Q9  FP32  16 x 62500  0.13   91   46
+//   61x45x53          0.89  18.3  18.6           16.8  16.5            32 x 31250  0.25   47   46
+//   80^3              0.83  55.5  75.0           35.7  51.4            48 x 20833  0.38   41   47
+//   48^3              0.75  15.1  16.8           13.0  15.1           130 x 7692   0.51   41   48
+//   100^3             0.75   123   140           80.2   103           192 x 5208   0.75   32   47
+//   26^3              0.66   7.7   8.9            8.2   7.8      FP16  16 x 62500  0.06  157   41
+//   40^3              0.63  12.7  11.8           12.8  10.8            48 x 20833  0.19   57   40
+//   65^3              0.61  41.3  36.2           27.0  29.4            64 x 15625  0.25   42   41
+//   33x33x300         0.43  56.8  45.2           39.6  33.2            96 x 10416  0.38   34   40
+//   8x8x4000          0.25  66.0  31.8           52.6  26.3           260 x 3846   0.51   35   41
+inline bool noalloc_march_pays(const KParams& k, int D, int width, int ty) {
+    return D == 3 ? axis_fill(k.nx, 32) * axis_fill(k.ny, ty) >= 0.7 : axis_fill(k.nx, width) >= 0.3;
+}
+
 // D2Q9 small-grid kernels: a strip of kRowW nodes of a row per CTA, kRowMost strips at most
 // (one partial vector each).
 constexpr int kRowW = 30;
@@ -371,6 +407,7 @@ inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW
 // CTAs leaves idle; but tiles where one to an SM does and the passes need a second warp to a
 // quarter of an SM (more than 128 nodes to an SM).
 constexpr int kSchedMarch = 0, kSchedTile = 1, kSchedRow = 2, kSchedTwoPass = 3;
+constexpr int kSchedSegment = 4;   // single store: a segment length was set, which selects the march above 64 MB
 inline void plan_d2q9(KParams& k, int sms, int per_sm, int width, bool f64) {
     k.tz = choose_rows(k, sms, per_sm, k.tz, width);
     const long long strips = row_strips(k), tiles = (long long)((k.nx + 31) / 32) * ((k.ny + 7) / 8);

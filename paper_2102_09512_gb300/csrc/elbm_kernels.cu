@@ -2906,9 +2906,8 @@ cudaError_t launch_fields_nodes(const KParams& p, const void* pop, double* rho, 
 constexpr int kPref = ELBM_PREF;   // planes of L2 prefetch ahead of the cp.async copies (with a tensor map)
 
 // One AA step on the single store A: from layout L1 (node-local reads, swapped writes) or
-// from L0 (pulled reads, pushed writes).  Stores larger than the L2 cache, D3Q27, FP32
-// arithmetic: the edges' Q~, then the march in place; the store is read 1.5 times less than by the
-// two passes, which take smaller grids (whose second pass finds the store in the cache).
+// from L0 (pulled reads, pushed writes).  D3Q27 with FP32 arithmetic, where aa_march_pays or a segment
+// length was set: the edges' Q~, then the march in place; else the two passes.
 template <int DD>
 cudaError_t launch_aa_march(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
                             cudaStream_t s, int from_l1, const CUtensorMap* pmap) {
@@ -2941,7 +2940,9 @@ cudaError_t launch_aa_march(const KParams& p, void* A, void* qfield, double* par
 cudaError_t launch_step_aa(const KParams& p, void* A, void* qfield, double* partials, int* nblocks, int* status,
                            cudaStream_t s, long long* launches, int from_l1, const CUtensorMap* pmap) {
     *launches += 2;
-    if (kD == 3 && kPipe && (double)p.N * Q * sizeof(P) > 64e6 && march_launches(p, kD, kTYP))
+    const double bytes = (double)p.N * Q * sizeof(P);
+    if (kD == 3 && kPipe && march_launches(p, kD, kTYP) &&
+        (p.sched == kSchedSegment ? bytes > 64e6 : aa_march_pays(p, kTYP, bytes)))
         return launch_aa_march<kD>(p, A, qfield, partials, nblocks, status, s, from_l1, pmap);
     const unsigned nb = blocks_1d(p.N);
     if (from_l1) {

@@ -81,9 +81,11 @@ const Ops* ops_for(int D, int store) {
     return nullptr;
 }
 
-// Grids of at least this many nodes run the default schedule of a handle (FP64 D3Q27: the two
-// passes, which are its default), which needs no Q~ field: D3Q27 FP32 96^3 71 us a step where the
-// two passes take 125, 61 x 45 x 53 18.6 and 18.8.
+// Grids of at least this many nodes run the default schedule of a handle (FP64 D3Q27: the two passes,
+// which are its default) where it pays (noalloc_march_pays; strips and tiles of D2Q9 do at every
+// size: FP32, us a step, 128^2 3.7 against 6.4, 256 x 160 4.4 against 7.2, 300^2 5.7 against 8.9).  Below it
+// the two passes, with the results to the last bit of a handle's two passes, though strips would
+// be faster there too (128 x 64 3.5 against 6.4).
 constexpr long long kNoallocFused = 1LL << 14;
 
 // Resident CTAs per SM of the fused kernel a problem would run, looked up once per device (a
@@ -149,7 +151,8 @@ extern "C" int elbm_step_noalloc(const elbm_params* prm, const void* src, void* 
         else k.tz = choose_tz(k, ops->fused_tile_y, sms, per_sm, k.tz);
         // the fused kernels' partials may run into the Q~ field, which they do not use
         const size_t room = (kNoallocScratchBytes - lay.partials) / (5 * sizeof(double));
-        const bool fits = k.sched != kSchedMarch || march_launches(k, D, ops->fused_tile_y);
+        const bool fits = k.sched != kSchedMarch || (march_launches(k, D, ops->fused_tile_y) &&
+                                                     noalloc_march_pays(k, D, ops->march_width, ops->fused_tile_y));
         if (k.sched != kSchedTwoPass && fits && (size_t)ops->max_blocks(k) <= room) {
             const cudaError_t e = ops->step_fused(k, src, dst, (double*)(s + lay.partials), &nb, nullptr, st, &launches);
             return e == cudaSuccess ? ELBM_OK : ELBM_ERR_CUDA;

@@ -1,6 +1,7 @@
 """CPU checks of the segment planner (choose_segment in csrc/elbm_internal.h), which the
 allocation-free step runs on every call: the lengths against the rule evaluated for every number of
-segments, and the time a call takes on long grids."""
+segments, and the time a call takes on long grids; and of the rules that choose between a march and the
+two passes (march_launches, aa_march_pays, noalloc_march_pays)."""
 import os
 import shutil
 import subprocess
@@ -75,3 +76,48 @@ def test_planning_a_long_grid_takes_microseconds(planned):
     """At most 128 lengths are looked at, some ten nanoseconds each: below 20 us with a wide margin
     (a loop over the segment counts takes 400 us and more here)."""
     assert float(planned[2]) < 20.0
+
+
+RULES = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "elbm_internal.h"
+int main(int argc, char** argv) {
+    elbm::KParams k{};
+    const int D = atoi(argv[1]);
+    k.nx = atoi(argv[2]); k.ny = atoi(argv[3]); k.nz = atoi(argv[4]); k.tz = atoi(argv[5]);
+    const double bytes = 27.0 * 8 * k.nx * k.ny * k.nz;
+    std::printf("%d %d %d %d\n", elbm::march_launches(k, D, 8), elbm::aa_march_pays(k, 8, bytes),
+                elbm::noalloc_march_pays(k, D, 128, 8), elbm::noalloc_march_pays(k, D, 256, 8));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    d = tmp_path_factory.mktemp("rule")
+    src, exe = d / "r.cu", str(d / "r")
+    src.write_text(RULES)
+    subprocess.run([nvcc, "-std=c++17", "-I", CSRC, "-I", os.path.join(ROOT, "include"), str(src), "-o", exe], check=True)
+    return lambda *a: [v == "1" for v in subprocess.run([exe, *map(str, a)], check=True, capture_output=True, text=True).stdout.split()]
+
+
+def test_marches_whose_tiles_stay_empty_are_not_taken(rule):
+    """Grids on which the march was measured slower than the two passes by 5 % or more do not take
+    it, those on which it was faster by 10 % or more do (FP32; the single store's own rule by its size too)."""
+    for shape, single, free in (((8, 8, 10000), False, False), ((33, 9, 2200), False, False), ((33, 33, 600), False, False),
+                                ((16, 16, 4000), False, False), ((72, 72, 72), False, True), ((65, 65, 65), False, False),
+                                ((40, 40, 40), False, False), ((96, 96, 96), True, True), ((80, 80, 80), True, True),
+                                ((128, 128, 128), True, True), ((64, 64, 96), True, True), ((48, 48, 48), False, True)):
+        assert rule(3, *shape, 16)[1:3] == [single, free], shape
+    for nx, f32, f16 in ((16, False, False), (48, True, False), (96, True, True), (130, True, True), (260, True, True)):
+        assert rule(2, nx, 4000, 1, 16)[2:] == [f32, f16], nx
+
+
+def test_marches_fit_their_launch(rule):
+    assert rule(3, 1, 524280, 1, 1)[0] and not rule(3, 1, 524281, 1, 1)[0]
+    assert rule(3, 1, 1, 65535, 1)[0] and not rule(3, 1, 1, 65536, 1)[0] and rule(3, 1, 1, 65536, 2)[0]
+    assert rule(2, 1, 65535, 1, 1)[0] and not rule(2, 1, 65536, 1, 1)[0]
