@@ -230,9 +230,9 @@ int elbm_set_kernel(elbm_handle *h, int kernel);
  * D3Q27, rows (y) for D2Q9.  Chosen at elbm_create for the current device (the
  * length that best fills the last wave of CTAs, each segment costing about two
  * planes of prologue); a tuning knob, results agree to rounding.  D2Q9 grids of up to
- * eight 30-node strips or four 32 x 8 tiles per SM, and FP64 ones, run the fused schedule
- * without the march (see elbm_kernel); setting a segment length here selects the march for
- * any D2Q9 grid, and for the AA store of a D3Q27 grid above 64 MB in FP32 arithmetic
+ * eight 30-node strips or four 32 x 8 tiles (16 with fixed-state faces) per SM, and FP64
+ * ones, run the fused schedule without the march (see elbm_kernel); setting a segment length
+ * here selects the march for any D2Q9 grid, and for the AA store of a D3Q27 grid above 64 MB in FP32 arithmetic
  * (see elbm_layout).  No effect on the default schedule of D3Q27 FP64. */
 int elbm_set_tile_z(elbm_handle *h, int tz);
 

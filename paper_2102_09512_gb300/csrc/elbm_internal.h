@@ -401,8 +401,12 @@ inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW
 //   1024^2      -    37.2   29.3         384^2      -    53.2      45.2
 //                                        512^2      -    91.5      72.5
 //                                        1448^2     -     698       495
-// (16-bit stores as FP32).  So: strips while there are at most eight to an SM, tiles while there
-// are at most four, else the march.  FP64: strips while there are at most four to an SM, each
+// (16-bit stores as FP32).  With fixed-state faces the march is compiled with tests of them in every row,
+// the tiles lose little (tiles, march; FP32 and, last, FP16):
+//   300x500    8.5   9.7   8.9  13.4      724^2  18.7  20.4  19.3  20.8      860^2  26.9  25.8  25.2  27.7
+//   512^2     10.8  12.4  10.9  13.5      800^2  22.5  25.5  22.4  27.7     1024^2  38.1  35.4  34.5  31.3
+// So: strips while there are at most eight to an SM, tiles while there
+// are at most four (with fixed-state faces 16), else the march.  FP64: strips while there are at most four to an SM, each
 // of which keeps four warps busy; then the two passes, which the FP64 pipe bounds and no wave of
 // CTAs leaves idle; but tiles where one to an SM does and the passes need a second warp to a
 // quarter of an SM (more than 128 nodes to an SM).
@@ -412,7 +416,8 @@ inline void plan_d2q9(KParams& k, int sms, int per_sm, int width, bool f64) {
     k.tz = choose_rows(k, sms, per_sm, k.tz, width);
     const long long strips = row_strips(k), tiles = (long long)((k.nx + 31) / 32) * ((k.ny + 7) / 8);
     if (sms > 0 && strips <= (f64 ? 4LL : 8LL) * sms && strips <= kRowMost) k.sched = kSchedRow;
-    else if (sms > 0 && (f64 ? tiles <= sms && k.N > 128LL * sms : tiles <= 4LL * sms)) k.sched = kSchedTile;
+    else if (sms > 0 && (f64 ? tiles <= sms && k.N > 128LL * sms : tiles <= (k.has_fixed ? 16LL : 4LL) * sms))
+        k.sched = kSchedTile;
     else k.sched = f64 ? kSchedTwoPass : kSchedMarch;
 }
 

@@ -86,6 +86,12 @@ int main(int argc, char** argv) {
     elbm::KParams k{};
     const int D = atoi(argv[1]);
     k.nx = atoi(argv[2]); k.ny = atoi(argv[3]); k.nz = atoi(argv[4]); k.tz = atoi(argv[5]);
+    if (D < 0) {   // plan_d2q9: store width of the strips, 64 bits, fixed faces
+        k.N = (long long)k.nx * k.ny; k.tz = 32; k.has_fixed = atoi(argv[6]);
+        elbm::plan_d2q9(k, 152, 4, 256, atoi(argv[5]));
+        std::printf("%d\n", k.sched);
+        return 0;
+    }
     const double bytes = 27.0 * 8 * k.nx * k.ny * k.nz;
     std::printf("%d %d %d %d\n", elbm::march_launches(k, D, 8), elbm::aa_march_pays(k, 8, bytes),
                 elbm::noalloc_march_pays(k, D, 128, 8), elbm::noalloc_march_pays(k, D, 256, 8));
@@ -102,7 +108,7 @@ def rule(tmp_path_factory):
     src, exe = d / "r.cu", str(d / "r")
     src.write_text(RULES)
     subprocess.run([nvcc, "-std=c++17", "-I", CSRC, "-I", os.path.join(ROOT, "include"), str(src), "-o", exe], check=True)
-    return lambda *a: [v == "1" for v in subprocess.run([exe, *map(str, a)], check=True, capture_output=True, text=True).stdout.split()]
+    return lambda *a: [v == "1" if a[0] > 0 else int(v) for v in subprocess.run([exe, *map(str, a)], check=True, capture_output=True, text=True).stdout.split()]
 
 
 def test_marches_whose_tiles_stay_empty_are_not_taken(rule):
@@ -121,3 +127,12 @@ def test_marches_fit_their_launch(rule):
     assert rule(3, 1, 524280, 1, 1)[0] and not rule(3, 1, 524281, 1, 1)[0]
     assert rule(3, 1, 1, 65535, 1)[0] and not rule(3, 1, 1, 65536, 1)[0] and rule(3, 1, 1, 65536, 2)[0]
     assert rule(2, 1, 65535, 1, 1)[0] and not rule(2, 1, 65536, 1, 1)[0]
+
+
+def test_tiles_are_kept_for_fixed_faces(rule):
+    """16-bit and FP32 grids with fixed-state faces ran on tiles up to some 724^2 nodes, which is where
+    the march (with its tests of the faces) begins to win; without such faces it does from four tiles an SM on."""
+    march, tile = 0, 1
+    for shape, fixed, free in (((300, 500), tile, march), ((512, 512), tile, march), ((724, 724), tile, march),
+                               ((1024, 1024), march, march), ((500, 300), tile, tile)):
+        assert rule(-1, *shape, 1, 0, 1) == [fixed] and rule(-1, *shape, 1, 0, 0) == [free], shape
