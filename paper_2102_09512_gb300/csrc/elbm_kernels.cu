@@ -407,7 +407,7 @@ struct TotalsF64 {
             return a;
         }
         top = (top >> 20) + 6;
-        long long a = kTotRun / 2;   // half a unit a value, as in fixed_sums
+        long long a = 0;
 #pragma unroll
         for (int k = 0; k < kTotRun; ++k) a += FixedSum::fixed(v[k], top);
         return FixedSum::value(a, top);
@@ -788,7 +788,7 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
 // thread of the second pass reads before it writes there.  Q~, which neighbours read, goes to
 // the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
 // moments 2.3 times (both with the arithmetic of their time; with the sums and products in
-// integers, FixedSum and FixedProd, 1.07 now, of which the traffic takes 0.46).
+// integers, FixedSum and FixedProd, 1.20 now, of which the traffic takes 0.46).
 constexpr int kSms = 152;   // SMs of the device the rules here are for
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
@@ -831,8 +831,9 @@ moments64_kernel(const __grid_constant__ KParams p, const P* src, R* __restrict_
     block_sum5_warp(tot, partials + 5 * blockIdx.x);
 }
 constexpr int kThreads64 = 128;   // second pass: smaller CTAs, so that one's loads overlap another's arithmetic
+// (registers capped at 128, D2Q9 102: uncapped 138 and 108 take a CTA from every SM, 96^3 409 -> 497 us)
 template <bool PULL>
-__global__ void __launch_bounds__(kThreads64, 2)
+__global__ void __launch_bounds__(kThreads64, kD == 3 ? 4 : 5)
 collide64_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict__ dst, const R* qf) {
     wait_for_previous();
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;

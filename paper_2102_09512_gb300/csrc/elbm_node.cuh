@@ -544,14 +544,40 @@ __device__ __forceinline__ void node_moments_stored(Pair pair, const KParams& p,
     }
 }
 
+// Shifts that clamp: 0 from 64 on.
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned n) {
+    asm("shr.b64 %0, %1, %2;" : "=l"(v) : "l"(v), "r"(n));
+    return v;
+}
+__device__ __forceinline__ unsigned long long shl64(unsigned long long v, unsigned n) {
+    asm("shl.b64 %0, %1, %2;" : "=l"(v) : "l"(v), "r"(n));
+    return v;
+}
+// m 2^(e - 1086), sign bit of hi `sign`, for 0 < m < 2^63 within the normal range, rounded to nearest, ties
+// to even (EVEN) or up; z leading zeros of m.
+template <bool EVEN>
+__device__ __forceinline__ double round64(unsigned long long m, int z, int e, unsigned sign) {
+    unsigned long long b;   // 53 bits, or 2^53
+    if (EVEN) {
+        const unsigned long long s = m << (z - 1 & 63);   // first bit at 62
+        b = (s + (0x1ffu + (((unsigned)s >> 10) & 1u))) >> 10;
+    } else {
+        b = (((m << z) >> 10) + 1ull) >> 1;
+    }
+    return __hiloint2double((int)(((unsigned)(b >> 32) + ((unsigned)(e - z - 1) << 20)) | sign), (int)(unsigned)b);
+}
+
 // Sums of FP64 values in 64-bit integers.  An FP64 instruction holds a quarter of an SM for 64 cycles
 // and an integer one for one or two, so the moments, which only add and subtract populations, are
-// summed as integers: fixed(x, top) is floor(x / unit), the unit 2^-57 of the power of two of the
+// summed as integers: fixed(x, top) is x in units of 2^-57 of the power of two of the
 // largest |x| (biased exponent + 6: top); the sums are exact and 26 values fit.  The value at
-// rest, part of rho and rho E alone and 16 times the next, is added in FP64.  Each value is off by half
-// a unit on average either way, about 2^-55 of the largest in a sum of 26, where an FP64 tree
-// rounds each partial sum by up to 2^-53 of it.  D3Q27 moments 243 -> 121 us (96^3; 141 -> 50 FP64
-// instructions a warp), the step 699 -> 574; D2Q9 127 -> 83 (1024^2), 1680 x 1440 870 -> 765.
+// rest, part of rho and rho E alone and 16 times the next, is added in FP64.  A value that has bits
+// below the unit is rounded to the odd one of its neighbours (von Neumann's rounding), others are
+// exact, and the sum is rounded to nearest, ties to even: no step has a sign on the average, where a floor and
+// half a unit added moved the mass of a periodic sheet by 2e-14 in 10,000 steps.  Each value is off by less
+// than a unit, about 2^-55 of the largest in a sum of 26, where an FP64 tree
+// rounds each partial sum by up to 2^-53 of it.  D3Q27 moments 243 -> 123 us (96^3; 141 -> 50 FP64
+// instructions a warp), D2Q9 127 -> 83 (1024^2).
 struct FixedSum {
     static __device__ __forceinline__ int top_of(int top, double x) { return max(top, __double2hiint(x) & 0x7fffffff); }
     // exponents that keep clear of infinities, NaN and the subnormal range
@@ -560,17 +586,15 @@ struct FixedSum {
         const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
         const unsigned h = __funnelshift_l(lo, hi, 11) | 0x80000000u, l = lo << 11;   // the significand, first bit set
         const unsigned n = (unsigned)top - ((hi >> 20) & 0x7ffu);                      // top = exponent + 6
-        const unsigned long long v = n > 63u ? 0ull : (((unsigned long long)h << 32) | l) >> n;
+        const unsigned long long sig = ((unsigned long long)h << 32) | l;
+        unsigned long long v = shr64(sig, n);
+        if (__funnelshift_rc(0u, l, n) != 0u) v |= 1ull;   // the low word's bits below the unit
         const long long neg = (int)hi >> 31;
-        return (long long)v ^ neg;
+        return ((long long)v ^ neg) - neg;
     }
-    static __device__ __forceinline__ double value(long long v, int top) {   // rounded to nearest
+    static __device__ __forceinline__ double value(long long v, int top) {
         const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
-        const int z = __clzll((long long)m);
-        const unsigned long long b = (((m << z) >> 10) + 1ull) >> 1;   // 53 bits, or 2^53
-        const unsigned long long e = (unsigned long long)(unsigned)(top - z - 1) << 52;
-        const unsigned long long r = (b + e) | (v < 0 ? 1ull << 63 : 0ull);
-        return v == 0 ? 0.0 : __longlong_as_double((long long)r);
+        return v == 0 ? 0.0 : round64<true>(m, __clzll((long long)m), top, (unsigned)(v >> 32) & 0x80000000u);
     }
 };
 template <int D, bool FULL>
@@ -594,15 +618,14 @@ __device__ __forceinline__ bool fixed_sums(const double* f, const double* g, con
         if (i != REST) E += FixedSum::fixed(g[i], tg);
     }
     f_moments<D, long long, true, false>(s, p, n[0], n[1], n[2], n[3], P);
-    // half a unit for each value that floor took on average half a unit from
-    rho = f[REST] + FixedSum::value(n[0] + (Q - 1) / 2, tf);
-    rE = g[REST] + FixedSum::value(E + (Q - 1) / 2, tg);
+    rho = f[REST] + FixedSum::value(n[0], tf);
+    rE = g[REST] + FixedSum::value(E, tg);
     jx = FixedSum::value(n[1], tf);
     jy = FixedSum::value(n[2], tf);
     jz = D == 3 ? FixedSum::value(n[3], tf) : 0.0;
     if (FULL)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) P6[k] = D == 2 && (k == 2 || k > 3) ? 0.0 : FixedSum::value(P[k] + (k < 3 ? Q / 3 : 0), tf);
+        for (int k = 0; k < 6; ++k) P6[k] = D == 2 && (k == 2 || k > 3) ? 0.0 : FixedSum::value(P[k], tf);
     return true;
 }
 
@@ -831,9 +854,12 @@ struct Relax {
 };
 
 // Sums of products of FP64 values in integers: a product of significands of 62 and 63 bits, the upper
-// half of it (three multiplications of 32 bits, the lowest left out), up to four such terms shifted to
-// the exponent of the largest, added, and rounded once.  A term is off by less than 2^-57 of the
-// largest, where FP64 rounds every product and partial sum by up to 2^-53.  Zero counts as 2^-1023.
+// half of it (three multiplications of 32 bits), up to four such terms shifted to the exponent of the
+// largest, added, and rounded once.  Every product has some 45 bits below the unit, so a floor
+// takes half a unit from it on the average, and the product of the low words, which is left out, is a
+// quarter of the last place before the shift on the average: both are added.  Of three terms' one and a half units
+// the last half is what rounding ties up adds.  A term is off by less than 2^-57 of the largest, where FP64
+// rounds every product and partial sum by up to 2^-53.  Zero counts as 2^-1023.
 // Terms must keep clear of infinity; results below the normal range are zero.
 struct FixedProd {
     struct Sig { unsigned hi, lo, es; };              // significand; biased exponent, sign in bit 31
@@ -845,30 +871,28 @@ struct FixedProd {
                 ((h >> 20) & 0x7ffu) | (h & 0x80000000u)};
     }
     static __device__ __forceinline__ Term mul(const Sig& a, const Sig& b) {   // sig<2> by sig<1>
-        const unsigned long long t = (unsigned long long)a.hi * b.lo + (unsigned long long)a.lo * b.hi;
+        const unsigned long long t = (unsigned long long)a.hi * b.lo + 0x40000000ull + (unsigned long long)a.lo * b.hi;
         return {(unsigned long long)a.hi * b.hi + (t >> 32), a.es + b.es};     // the signs add without carry
     }
     static __device__ __forceinline__ Term term(const Sig& b) {   // sig<1>, times one
         return {(((unsigned long long)b.hi << 32) | b.lo) >> 3, b.es + 1023u};
     }
     template <int N>
-    static __device__ __forceinline__ double sum(const Term (&t)[N]) {
+    static __device__ __forceinline__ double sum(const Term (&t)[N], int terms = N) {   // terms: those that are not zero
         int top = 0;
 #pragma unroll
         for (int k = 0; k < N; ++k) top = max(top, (int)(t[k].es & 0x7fffffffu));
-        long long v = 0;
+        long long v = terms >> 1;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            unsigned long long r;
-            asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(t[k].r), "r"(top - (int)(t[k].es & 0x7fffffffu)));   // 0 from 64 on
+            const unsigned long long r = shr64(t[k].r, (unsigned)(top - (int)(t[k].es & 0x7fffffffu)));
             v += (long long)r ^ (long long)((int)t[k].es >> 31);
         }
-        const unsigned long long m = (unsigned long long)(v ^ (v >> 63));
-        const int z = __clzll((long long)m), e = top - 1019 - z;
-        const unsigned long long b = (((m << z) >> 10) + 1ull) >> 1;
-        const unsigned long long bits = (b + ((unsigned long long)(unsigned)(e - 1) << 52)) |
-                                        ((unsigned long long)v & (1ull << 63));
-        return m == 0 || e < 1 ? 0.0 : __longlong_as_double((long long)bits);
+        if (N == 4 && terms == 3) v |= 1;   // half a unit, and no ties
+        const long long neg = v >> 63;
+        const unsigned long long m = (unsigned long long)((v ^ neg) - neg);
+        const int z = __clzll((long long)m);
+        return top - 1019 - z < 1 || m == 0 ? 0.0 : round64<N != 3>(m, z, top - 1019, (unsigned)neg & 0x80000000u);
     }
 };
 
@@ -972,7 +996,8 @@ struct Relax<D, double, false, CAL> {
     // stores); usable: every factor is finite and moderate.  A direction's f takes two FP64
     // instructions or some 55 integer ones, g three or four or some 80: all in integers D2Q9 keeps the FP64
     // pipe 80 % busy (1680 x 1440: 765 us a step all FP64, 644 with g, 580 with both), on D3Q27 a
-    // third of f stays FP64 (128^3: 1330; g 1122, a third of f too 1115, two thirds 1070, all 1129).
+    // third of f stays FP64 (128^3: 1330; g 1122, a third of f too 1115, two thirds 1070, all 1129; that
+    // was with floors, whose sign the mass followed: with the present roundings 1680 x 1440 588, 128^3 1197).
     __device__ __forceinline__ bool usable() const {
         int top = 0;
         auto see = [&](double x) { top = max(top, __double2hiint(x) & 0x7fffffff); };
@@ -1026,7 +1051,7 @@ struct Relax<D, double, false, CAL> {
                     if (cx + cy + cz > 0) q.es ^= 0x80000000u;
                     if ((q.es & 0x7fffffffu) == 0u) q.es = 0u;   // no unit for the sign of a zero
                     const FP::Term tg[4] = {g0, g1, g2, FP::term(q)};
-                    g = FP::sum(tg);
+                    g = FP::sum(tg, q.es ? 4 : 3);
                 } else {
                     const FP::Term tg[3] = {g0, g1, g2};
                     g = FP::sum(tg);
