@@ -392,34 +392,39 @@ constexpr int kTotCtas = sizeof(R) == 8 ? 1 : 3;   // per SM; FP64: what a threa
 struct TotalsF64 {
     double F = 0, Fc = 0, G = 0, Gc = 0, s[5] = {}, c[5] = {};
     __device__ __forceinline__ void pairs(const R* f, const R* g) {
-        dd_add(F, Fc, sum(f));
-        dd_add(G, Gc, sum(g));
+        add(F, Fc, f);
+        add(G, Gc, g);
     }
-    static __device__ __forceinline__ double sum(const R* v) {
+    // s + c += the values of a run: their integer sum as its upper bits and its low 24, either exact
+    static __device__ __forceinline__ void add(double& s, double& c, const R* v) {
         static_assert(kTotRun <= 27, "values that a sum of integers holds");
         int top = 0;
 #pragma unroll
         for (int k = 0; k < kTotRun; ++k) top = FixedSum::top_of(top, v[k]);
         if (!FixedSum::usable(top)) {
-            double a = 0;
 #pragma unroll
-            for (int k = 0; k < kTotRun; ++k) a += v[k];
-            return a;
+            for (int k = 0; k < kTotRun; ++k) dd_add(s, c, v[k]);
+            return;
         }
         top = (top >> 20) + 6;
         long long a = 0;
 #pragma unroll
         for (int k = 0; k < kTotRun; ++k) a += FixedSum::fixed(v[k], top);
-        return FixedSum::value(a, top);
+        const long long low = a & 0xffffff;
+        dd_add(s, c, FixedSum::value(a - low, top));
+        c += FixedSum::value(low, top);
     }
     __device__ __forceinline__ void plane_end(int i) {
         const double cx = cx_of(i), cy = cy_of(i), cz = cz_of<kD>(i);
-        F += Fc;
-        dd_add(s[0], c[0], F);
-        if (cx != 0.0) dd_add(s[1], c[1], cx * F);
-        if (cy != 0.0) dd_add(s[2], c[2], cy * F);
-        if (cz != 0.0) dd_add(s[3], c[3], cz * F);
-        dd_add(s[4], c[4], G + Gc);
+        auto put = [&](int k, double x, double v, double vc) {
+            dd_add(s[k], c[k], x * v);
+            c[k] += x * vc;
+        };
+        put(0, 1.0, F, Fc);
+        if (cx != 0.0) put(1, cx, F, Fc);
+        if (cy != 0.0) put(2, cy, F, Fc);
+        if (cz != 0.0) put(3, cz, F, Fc);
+        put(4, 1.0, G, Gc);
         F = Fc = G = Gc = 0.0;
     }
     // this warp's sums and corrections, in its lane 0
