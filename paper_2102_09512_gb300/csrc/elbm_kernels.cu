@@ -190,42 +190,30 @@ __device__ __forceinline__ void node_totals(const Moments<R>& m, R rE, R v[5]) {
     v[4] = rE;
 }
 
-// Per-thread running sum of the node totals over the planes of a z segment: in FP64 a
-// Kahan-compensated sum of plain sums of four nodes (compensating every node would cost 20 of
-// the update's FP64 instructions); in FP32 a plain sum (at most p.tz terms of per-node
+// Per-thread running sum of the node totals over the planes of a z segment:
+// Kahan-compensated in FP64; in FP32 a plain sum (at most p.tz terms of per-node
 // values that are themselves FP32 results), which saves the registers of the
 // compensation terms.
 struct Acc5 {
-    R s[5], c[5], q[5];
-    int n;
+    R s[5], c[5];
     __device__ __forceinline__ void zero() {
-        n = 0;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) s[k] = c[k] = q[k] = R(0);
-    }
-    __device__ __forceinline__ void kahan() {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            const R y = q[k] - c[k];
-            const R t = s[k] + y;
-            c[k] = (t - s[k]) - y;
-            s[k] = t;
-        }
+        for (int k = 0; k < 5; ++k) s[k] = c[k] = R(0);
     }
     __device__ __forceinline__ void add(const R v[5]) {
-        if constexpr (sizeof(R) == 8) {
-            const bool first = (n & 3) == 0;
 #pragma unroll
-            for (int k = 0; k < 5; ++k) q[k] = first ? v[k] : q[k] + v[k];
-            if ((++n & 3) == 0) kahan();
-        } else {
-#pragma unroll
-            for (int k = 0; k < 5; ++k) s[k] += v[k];
+        for (int k = 0; k < 5; ++k) {
+            if constexpr (sizeof(R) == 8) {
+                const R y = v[k] - c[k];
+                const R t = s[k] + y;
+                c[k] = (t - s[k]) - y;
+                s[k] = t;
+            } else {
+                s[k] += v[k];
+            }
         }
     }
     __device__ __forceinline__ void total(R out[5]) {
-        if constexpr (sizeof(R) == 8)
-            if (n & 3) kahan();
 #pragma unroll
         for (int k = 0; k < 5; ++k) out[k] = s[k] - c[k];
     }
