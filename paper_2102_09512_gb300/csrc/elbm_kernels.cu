@@ -642,17 +642,19 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
                 }
                 Df theta = df_add(G[0][0], G[1][1]);
                 const Df wz = df_add(G[1][0], df_neg(G[0][1]));
-                Df w2 = df_sq(wz), uu = df_add(df_prod(cur.u[0], cur.u[0]), df_prod(cur.u[1], cur.u[1]));
+                float uu_rest = 0.f;
+                Df w2 = df_sq(wz), uu = df_add(df_prod(cur.u[0], cur.u[0]), df_prod(cur.u[1], cur.u[1]), uu_rest);
                 if (DD == 3) {
                     theta = df_add(theta, G[2][2]);
                     w2 = df_add(w2, df_sq(df_add(G[2][1], df_neg(G[1][2]))));
                     w2 = df_add(w2, df_sq(df_add(G[0][2], df_neg(G[2][0]))));
-                    uu = df_add(uu, df_prod(cur.u[2], cur.u[2]));
+                    uu = df_add(uu, df_prod(cur.u[2], cur.u[2]), uu_rest);
                 }
                 const Df r2 = df_prod(cur.rho, cur.rho), ruu = df_scale(uu, cur.rho), th2 = df_sq(theta);
                 const Df T2 = df_prod(cur.T, cur.T), gxx = df_sq(G[0][0]), ux2 = df_prod(cur.u[0], cur.u[0]);
                 t[0].add(make_float2(cur.rho, r2.h), make_float2(0.f, r2.l));
                 t[1].add(make_float2(ruu.h, uu.h), make_float2(ruu.l, uu.l));
+                t[1].e2 = add2(t[1].e2, make_float2(cur.rho * uu_rest, uu_rest));
                 t[2].add(make_float2(th2.h, cur.T), make_float2(th2.l, 0.f));
                 t[3].add(make_float2(T2.h, gxx.h), make_float2(T2.l, gxx.l));
                 t[4].add(make_float2(w2.h, ux2.h), make_float2(w2.l, ux2.l));

@@ -307,6 +307,16 @@ __device__ __forceinline__ Df df_add(Df a, Df b) {
     const float h = s + e;
     return {h, e - (h - s)};
 }
+// The same, adding what is rounded away to rest: a sum of squares needs it, whose low bits are not random (an
+// odd number's square ends in 001) and whose roundings have a sign.
+__device__ __forceinline__ Df df_add(Df a, Df b, float& rest) {
+    const float s = a.h + b.h, bb = s - a.h, e1 = (a.h - (s - bb)) + (b.h - bb);
+    const float q = a.l + b.l, qb = q - a.l, e2 = (a.l - (q - qb)) + (b.l - qb);
+    const float e = e1 + q, eb = e - e1;
+    rest += e2 + ((e1 - (e - eb)) + (q - eb));
+    const float h = s + e;
+    return {h, e - (h - s)};
+}
 __device__ __forceinline__ Df df_neg(Df a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ Df df_prod(float a, float b) {   // a b, exact
     const float p = __fmul_rn(a, b);
