@@ -269,7 +269,7 @@ struct Ops {
                                  int grid, cudaStream_t s, long long* launches);
     int (*ensemble_occupancy)(int ty);
     cudaError_t (*stats)(const KParams& p, const void* pop, double* partials, int* nblocks, cudaStream_t s,
-                         long long* launches);   // kStatsSums partial sums per CTA
+                         long long* launches, bool wide);   // kStatsSums partial sums per CTA; wide: terms in FP64
     int fused_tile_y;             // D3Q27: tile height of the fused kernels (tile width 32); D2Q9: 1 (row march)
     // resident CTAs per SM of the default fused kernel for the grid p (the D2Q9 march is
     // compiled with and without fixed-state faces; 0: unknown)

@@ -533,10 +533,12 @@ totals_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doub
 // evaluations, 256^3 FP32 6.1 ms).  For the FP32-arithmetic stores the sums and their terms
 // are unevaluated sums of floats: differences and products of FP32 values are exact as two
 // floats, the viscosity law comes from pow_pos_df and the sums are Tri2 ones.  (With the law in
-// FP64 that pipe bounded the kernel: 256^3 FP32 1.48 ms, without 0.79.)
+// FP64 that pipe bounded the kernel: 256^3 FP32 1.48 ms, without 0.79.)  Terms or sums that leave the range
+// of floats, or fall so low that their second one does, show in the sums; elbm_turbulence_stats then asks for
+// them in FP64 (WIDE, which FP64 stores always take).
 constexpr int kStats = kStatsSums;
-template <int DD>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
+template <int DD, bool WIDE>
+__global__ void __launch_bounds__(256, WIDE ? 1 : 2)
 stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, double* __restrict__ partials, int tz,
              unsigned tiles_x, unsigned tiles_y) {
     constexpr int TX = 32, TY = 8, NT = TX * TY;
@@ -579,13 +581,12 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
         for (int a = 0; a < DD; ++a) us[b][a][r][c] = n.u[a];
     };
 
-    constexpr bool kF64 = sizeof(R) == 8;
-    double acc[kF64 ? kStats : 1] = {};   // FP64 store
-    Tri2 t[6];                            // FP32 arithmetic: the sums in pairs
+    double acc[WIDE ? kStats : 1] = {};
+    Tri2 t[6];   // not WIDE: the sums in pairs
 #pragma unroll
     for (int k = 0; k < 6; ++k) t[k].zero();
     const float eh = (float)p.mu_exp;
-    const Df mu_exp = {eh, kF64 ? 0.f : (float)(p.mu_exp - (double)eh)};
+    const Df mu_exp = {eh, WIDE ? 0.f : (float)(p.mu_exp - (double)eh)};
 
     Node prev = {}, cur = {}, next = {};
     if (active) {
@@ -605,29 +606,30 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
         if (DD == 3 && halo && z + 1 < ze) put(b ^ 1, hr, hc, node(hx, hy, zn));
         if (active) {
             auto U = [&](int a, int r, int c) { return us[b][a][ty + 1 + r][tx + 1 + c]; };
-            if constexpr (kF64) {
+            if constexpr (WIDE) {
                 double G[3][3] = {};   // twice d u_a / d x_b
 #pragma unroll
                 for (int a = 0; a < DD; ++a) {
-                    G[a][0] = U(a, 0, 1) - U(a, 0, -1);
-                    G[a][1] = U(a, 1, 0) - U(a, -1, 0);
-                    if (DD == 3) G[a][2] = next.u[a] - prev.u[a];
+                    G[a][0] = (double)U(a, 0, 1) - U(a, 0, -1);
+                    G[a][1] = (double)U(a, 1, 0) - U(a, -1, 0);
+                    if (DD == 3) G[a][2] = (double)next.u[a] - prev.u[a];
                 }
                 const double theta = G[0][0] + G[1][1] + G[2][2];
                 const double wx = G[2][1] - G[1][2], wy = G[0][2] - G[2][0], wz = G[1][0] - G[0][1];
                 const double w2 = wx * wx + wy * wy + wz * wz;
-                const double uu = cur.u[0] * cur.u[0] + cur.u[1] * cur.u[1] + cur.u[2] * cur.u[2];
-                acc[0] += cur.rho;
-                acc[1] = fma(cur.rho, cur.rho, acc[1]);
-                acc[2] = fma(cur.rho, uu, acc[2]);
+                const double rho = cur.rho, T = cur.T, ux = cur.u[0], uy = cur.u[1], uz = cur.u[2];
+                const double uu = ux * ux + uy * uy + uz * uz;
+                acc[0] += rho;
+                acc[1] = fma(rho, rho, acc[1]);
+                acc[2] = fma(rho, uu, acc[2]);
                 acc[3] += uu;
                 acc[4] = fma(theta, theta, acc[4]);
-                acc[5] += cur.T;
-                acc[6] = fma(cur.T, cur.T, acc[6]);
+                acc[5] += T;
+                acc[6] = fma(T, T, acc[6]);
                 acc[7] = fma(G[0][0], G[0][0], acc[7]);
                 acc[8] += w2;
-                acc[9] = fma(cur.u[0], cur.u[0], acc[9]);
-                if (p.powlaw) acc[10] = fma(pow_pos(cur.T * p.d_invT0, p.mu_exp), w2, acc[10]);
+                acc[9] = fma(ux, ux, acc[9]);
+                if (p.powlaw) acc[10] = fma(pow_pos(T * p.d_invT0, p.mu_exp), w2, acc[10]);
             } else {
                 Df G[3][3];
 #pragma unroll
@@ -660,11 +662,7 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
                 t[4].add(make_float2(w2.h, ux2.h), make_float2(w2.l, ux2.l));
                 if (p.powlaw) {   // T^mu_exp |omega|^2; mu0 T0^-mu_exp comes at the end
                     Df y;
-                    if (!pow_pos_df(cur.T, mu_exp, y)) {
-                        const double v = pow((double)cur.T, p.mu_exp);
-                        y.h = (float)v;
-                        y.l = (float)(v - (double)y.h);
-                    }
+                    if (!pow_pos_df(cur.T, mu_exp, y)) y.h = y.l = __int_as_float(0x7fffffff);   // NaN: FP64 wanted
                     y = df_mul(y, w2);
                     t[5].add(make_float2(y.h, 0.f), make_float2(y.l, 0.f));
                 }
@@ -674,7 +672,7 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
         cur = next;
     }
     const int lane = tid & 31, warp = tid >> 5;
-    if constexpr (kF64) {
+    if constexpr (WIDE) {
 #pragma unroll
         for (int k = 0; k < kStats; ++k) {
 #pragma unroll
@@ -693,14 +691,14 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
     }
     __syncthreads();
     if (tid < kStats) {
-        // theta, omega and d u_x / d x were summed as twice their values; the last sum lacks mu0 (FP32
-        // arithmetic: mu0 T0^-mu_exp)
+        // theta, omega and d u_x / d x were summed as twice their values; the last sum lacks mu0 (not
+        // WIDE: mu0 T0^-mu_exp)
         const bool quad = tid == 4 || tid == 7 || tid == 8 || tid == 10;
         const int k = tid == 10 && !p.powlaw ? 8 : tid;
         double v = 0.0;
         for (int w = 0; w < NT / 32; ++w) v += part[w][k];
         if (quad) v *= 0.25;
-        if (tid == 10) v *= kF64 || !p.powlaw ? p.mu0 : p.mu0 * pow(p.T0, -p.mu_exp);
+        if (tid == 10) v *= WIDE || !p.powlaw ? p.mu0 : p.mu0 * pow(p.T0, -p.mu_exp);
         partials[(size_t)kStats * blockIdx.x + tid] = v;
     }
 }
@@ -3166,13 +3164,14 @@ int ensemble_occupancy(int ty) {
 // Columns of 32 x 8 nodes over segments chosen like those of the fused kernels; a grid has at
 // most as many CTAs as the one-dimensional launches, or one per column (max_blocks bounds both).
 cudaError_t launch_stats(const KParams& p, const void* pop, double* partials, int* nblocks, cudaStream_t s,
-                         long long* launches) {
+                         long long* launches, bool wide) {
     const int tx = (p.nx + 31) / 32, ty = (p.ny + 7) / 8;
     const long long most = blocks_1d_of(p.N) > kTotalsBlocks ? blocks_1d_of(p.N) : kTotalsBlocks;
     int tz = choose_segment((double)tx * ty, p.nz, 152, 2, 32);
     while (tz < p.nz && (long long)tx * ty * ((p.nz + tz - 1) / tz) > most) tz = tz < p.nz / 2 ? 2 * tz : p.nz;
     const long long grid = (long long)tx * ty * ((p.nz + tz - 1) / tz);
-    stats_kernel<kD><<<(unsigned)grid, dim3(32, 8), 0, s>>>(p, (const P*)pop, partials, tz, (unsigned)tx, (unsigned)ty);
+    auto kern = wide ? stats_kernel<kD, true> : stats_kernel<kD, sizeof(R) == 8>;
+    kern<<<(unsigned)grid, dim3(32, 8), 0, s>>>(p, (const P*)pop, partials, tz, (unsigned)tx, (unsigned)ty);
     ++*launches;
     *nblocks = (int)grid;
     return cudaGetLastError();

@@ -32,3 +32,41 @@ def test_energy_sums_have_no_bias(E, store, seed):
     K, u_rms = 0.5 * (rho.ravel() * uu).sum() / uu.size, np.sqrt(uu.sum() / uu.size / 3)
     assert abs(dev["K"] / K - 1) <= 3 * 2.0 ** -53
     assert abs(dev["u_rms"] / u_rms - 1) <= 3 * 2.0 ** -53
+
+
+def host_stats(c, D, rho, u, T):
+    """The statistics' means in extended precision from node values on a periodic grid."""
+    sh = (c.nz, c.ny, c.nx)
+    rho, T, u = rho.astype(LD).reshape(sh), T.astype(LD).reshape(sh), u.astype(LD).reshape((D,) + sh)
+    G = [[(np.roll(u[a], -1, 2 - b) - np.roll(u[a], 1, 2 - b)) / 2 for b in range(D)] for a in range(D)]
+    theta = sum(G[a][a] for a in range(D))
+    w2 = (G[1][0] - G[0][1]) ** 2
+    if D == 3:
+        w2 = w2 + (G[2][1] - G[1][2]) ** 2 + (G[0][2] - G[2][0]) ** 2
+    uu = (u ** 2).sum(0)
+    mu = LD(c.mu0) * (T / LD(c.T0)) ** LD(c.mu_exp)
+    return dict(K=0.5 * (rho * uu).mean(), u_rms=np.sqrt(uu.mean() / D), theta_rms=np.sqrt((theta ** 2).mean()),
+                dudx2=(G[0][0] ** 2).mean(), omega_rms=np.sqrt(w2.mean()), enstrophy=0.5 * w2.mean(),
+                dissipation=(mu * w2).mean())
+
+
+# Exponents whose T^mu_exp (T = 0.15) is below, and above, what FP32 holds, and whose lower bits are; deviations from rest so
+# small that the squares of the velocities, or of their differences alone, are; and one state
+# that a float holds.  Bound 2^-46: the law takes T/T0, off by 2^-53, to the 60th power (2^-47); the sums are FP64.
+@pytest.mark.parametrize("D,shape", [(3, (33, 9, 7)), (2, (65, 17, 1))])
+@pytest.mark.parametrize("store,scale,mu_exp", [("f32", 0, 60.0), ("f32", 0, -60.0), ("f32", 0, 40.0), ("f32", 0, 0.76),
+                                                ("bf16dev", 2.0 ** -60, 0.76), ("bf16dev", 2.0 ** -80, 0.76),
+                                                ("bf16dev", 2.0 ** -40, 0.0)])
+def test_terms_outside_the_range_of_floats(E, store, scale, mu_exp, D, shape):
+    c = C.random_smooth(D, *shape, seed=9, mu0=0.01, du=0.05, u0=(0.09, -0.07, 0.06)[:D] + (0.0,) * (3 - D), mu_exp=mu_exp)
+    g = E.Solver.from_case(c, store=store)
+    if scale:   # populations rest + scale x (what the case has), exact: multiplied by a power of two
+        raw = g.get_populations().view(np.uint16)
+        v = (raw.astype(np.uint32) << 16).view(np.float32) * np.float32(scale)
+        g.set_populations((v.view(np.uint32) >> 16).astype(np.uint16).view(np.uint8))
+    dev = g.turbulence_stats()
+    ref = host_stats(c, D, *g.fields())
+    g.close()
+    for k, v in ref.items():
+        assert v > 0
+        assert abs(LD(dev[k]) / v - 1) <= 2.0 ** -46, k
