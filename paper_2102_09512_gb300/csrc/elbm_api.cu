@@ -563,7 +563,7 @@ int elbm_conservation(elbm_handle* h, double out[5]) {
 // 2^-149 and there are a few roundings like that to a term: below 2^-57 of a mean that is at least
 // 2^-88 (velocities or their differences of 6e-14).  Sums of zero are asked for again too: their terms may all have
 // underflowed.  One that is not finite shows a term beyond the range of floats or of pow_pos_df.
-// Both passes: 256^3 FP32 4.0 ms (mu_exp 60), the one in floats 0.82 (mu_exp 0.76).
+// Both passes: 256^3 FP32 4.0 ms, the one in floats 0.83.
 static bool stats_within_floats(const double sums[kStatsSums], double N, double mu0) {
     for (int k = 0; k < kStatsSums; ++k) {
         const double mean = sums[k] / N / (k == 10 ? mu0 : 1.0);

@@ -587,6 +587,8 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
     for (int k = 0; k < 6; ++k) t[k].zero();
     const float eh = (float)p.mu_exp;
     const Df mu_exp = {eh, WIDE ? 0.f : (float)(p.mu_exp - (double)eh)};
+    // log2 T0 to a multiple of 2^-8, which the law's logarithms are taken from
+    const float base = WIDE ? 0.f : rintf(log2f((float)p.T0) * 256.f) * 0x1p-8f;
 
     Node prev = {}, cur = {}, next = {};
     if (active) {
@@ -660,9 +662,9 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
                 t[2].add(make_float2(th2.h, cur.T), make_float2(th2.l, 0.f));
                 t[3].add(make_float2(T2.h, gxx.h), make_float2(T2.l, gxx.l));
                 t[4].add(make_float2(w2.h, ux2.h), make_float2(w2.l, ux2.l));
-                if (p.powlaw) {   // T^mu_exp |omega|^2; mu0 T0^-mu_exp comes at the end
+                if (p.powlaw) {   // (T 2^-base)^mu_exp |omega|^2
                     Df y;
-                    if (!pow_pos_df(cur.T, mu_exp, y)) y.h = y.l = __int_as_float(0x7fffffff);   // NaN: FP64 wanted
+                    if (!pow_pos_df(cur.T, mu_exp, y, base)) y.h = y.l = __int_as_float(0x7fffffff);   // NaN: FP64 wanted
                     y = df_mul(y, w2);
                     t[5].add(make_float2(y.h, 0.f), make_float2(y.l, 0.f));
                 }
@@ -691,14 +693,15 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
     }
     __syncthreads();
     if (tid < kStats) {
-        // theta, omega and d u_x / d x were summed as twice their values; the last sum lacks mu0 (not
-        // WIDE: mu0 T0^-mu_exp)
+        // theta, omega and d u_x / d x were summed as twice their values; the last sum lacks mu0, and (not
+        // WIDE) has base for log2 T0, at the exponent in two floats
         const bool quad = tid == 4 || tid == 7 || tid == 8 || tid == 10;
         const int k = tid == 10 && !p.powlaw ? 8 : tid;
         double v = 0.0;
         for (int w = 0; w < NT / 32; ++w) v += part[w][k];
         if (quad) v *= 0.25;
-        if (tid == 10) v *= WIDE || !p.powlaw ? p.mu0 : p.mu0 * pow(p.T0, -p.mu_exp);
+        if (tid == 10) v *= p.mu0;
+        if (tid == 10 && !WIDE && p.powlaw) v *= exp2(((double)mu_exp.h + mu_exp.l) * (base - log2(p.T0)));
         partials[(size_t)kStats * blockIdx.x + tid] = v;
     }
 }

@@ -335,10 +335,12 @@ __device__ __forceinline__ Df df_scale(Df a, float b) {
     return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
 }
 
-// pow_pos of an FP32 x as a sum of two floats (relative error about 2^-44): the same steps in
-// pairs of floats, about 90 FP32 instructions where one FP64 instruction keeps the SM as busy
-// as 64.  False (and no value) for an x or an exponent of 2 that pow_pos leaves to pow().
-__device__ __forceinline__ bool pow_pos_df(float x, Df e, Df& y) {
+// pow_pos of an FP32 x over 2^base, base a multiple of 2^-8, as a sum of two floats: the same steps in
+// pairs of floats, about 100 FP32 instructions where one FP64 instruction keeps the SM as busy
+// as 64.  Relative error about 2^-44, or 2^-47 |e (log2 x - base)| and 2^-49 where that is less; what many
+// x share (the tables' and the exponent's third floats) is carried beside, so that sums have
+// no more error than FP64 ones.  False (and no value) for an x or an exponent of 2 that pow_pos leaves to pow().
+__device__ __forceinline__ bool pow_pos_df(float x, Df e, Df& y, float base = 0.f) {
     const int b = __float_as_int(x);
     if ((unsigned)(b - 0x0d800000) >= 0x64000000u) return false;   // 2^-100 <= x < 2^100
     const int k = (b >> 23) - 127;
@@ -353,19 +355,22 @@ __device__ __forceinline__ bool pow_pos_df(float x, Df e, Df& y) {
     q = fmaf(r.h, q, 0x1.ec709ep-2f);
     const Df c1 = {0x1.715476p+0f, 0x1.4ae0c0p-26f}, c2 = {-0x1.715476p-1f, -0x1.4ae0c0p-27f};
     const Df s = df_mul(r, df_add(c1, df_mul(r, df_add(c2, df_prod(r.h, q)))));
-    const Df L = df_add(df_add({(float)k, 0.f}, {tab.y, tab.z}), s);
+    float rest = tab.w;
+    const Df L = df_add(df_add({(float)k - base, 0.f}, {tab.y, tab.z}, rest), s, rest);
     const Df t = df_mul(e, L);
     if (!(fabsf(t.h) < 60.f)) return false;
     const float n = rintf(t.h * 128.f);
     const float f0 = fmaf(n, -0x1p-7f, t.h), fh = f0 + t.l;
-    const Df f = {fh, t.l - (fh - f0)};
+    const Df f = {fh, fmaf(e.h, rest, t.l - (fh - f0))};
     // 2^f - 1 = f (d1 + f (d2 + f (d3 + f d4)))
     const Df d1 = {0x1.62e430p-1f, -0x1.05c610p-29f}, d2 = {0x1.ebfbe0p-3f, -0x1.f4e9c6p-33f};
     const float d = fmaf(f.h, 0x1.3b2ab6p-7f, 0x1.c6b08ep-5f);
     const Df w = df_mul(f, df_add(d1, df_mul(f, df_add(d2, df_prod(f.h, d)))));
     const int ni = (int)n;
     const float2 c = kExpTabF[ni & 127];
-    const Df z = df_add({c.x, c.y}, df_mul({c.x, c.y}, w));
+    Df cw = df_mul({c.x, c.y}, w);
+    cw.l += kExpTabL[ni & 127];
+    const Df z = df_add({c.x, c.y}, cw);
     const float two = __int_as_float(((ni >> 7) + 127) << 23);
     y = {z.h * two, z.l * two};
     return true;

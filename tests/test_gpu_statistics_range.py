@@ -50,15 +50,18 @@ def host_stats(c, D, rho, u, T):
                 dissipation=(mu * w2).mean())
 
 
-# Exponents whose T^mu_exp (T = 0.15) is below, and above, what FP32 holds, and whose lower bits are; deviations from rest so
-# small that the squares of the velocities, or of their differences alone, are; and one state
-# that a float holds.  Bound 2^-46: the law takes T/T0, off by 2^-53, to the 60th power (2^-47); the sums are FP64.
+# Exponents whose T^mu_exp (T = 0.15) is below, and above, what FP32 holds, and whose lower bits are, and whose
+# (T/T0)^mu_exp is (T0 = 15); deviations from rest so small that the squares of the velocities, or of
+# their differences alone, are; and one state that floats hold.
+# Bound 2^-46: the law takes T/T0, off by 2^-53, to the 60th power (2^-47); the sums are FP64.
 @pytest.mark.parametrize("D,shape", [(3, (33, 9, 7)), (2, (65, 17, 1))])
-@pytest.mark.parametrize("store,scale,mu_exp", [("f32", 0, 60.0), ("f32", 0, -60.0), ("f32", 0, 40.0), ("f32", 0, 0.76),
-                                                ("bf16dev", 2.0 ** -60, 0.76), ("bf16dev", 2.0 ** -80, 0.76),
-                                                ("bf16dev", 2.0 ** -40, 0.0)])
-def test_terms_outside_the_range_of_floats(E, store, scale, mu_exp, D, shape):
+@pytest.mark.parametrize("store,scale,mu_exp,T0", [("f32", 0, 60.0, 0.15), ("f32", 0, -60.0, 0.15), ("f32", 0, 40.0, 0.15),
+                                                   ("f32", 0, 60.0, 15.0), ("f32", 0, 0.76, 0.15),
+                                                   ("bf16dev", 2.0 ** -60, 0.76, 0.15), ("bf16dev", 2.0 ** -80, 0.76, 0.15),
+                                                   ("bf16dev", 2.0 ** -40, 0.0, 0.15)])
+def test_terms_outside_the_range_of_floats(E, store, scale, mu_exp, T0, D, shape):
     c = C.random_smooth(D, *shape, seed=9, mu0=0.01, du=0.05, u0=(0.09, -0.07, 0.06)[:D] + (0.0,) * (3 - D), mu_exp=mu_exp)
+    c.T0 = T0
     g = E.Solver.from_case(c, store=store)
     if scale:   # populations rest + scale x (what the case has), exact: multiplied by a power of two
         raw = g.get_populations().view(np.uint16)
@@ -70,3 +73,19 @@ def test_terms_outside_the_range_of_floats(E, store, scale, mu_exp, D, shape):
     for k, v in ref.items():
         assert v > 0
         assert abs(LD(dev[k]) / v - 1) <= 2.0 ** -46, k
+
+
+@pytest.mark.parametrize("store", ["f32", "f16dev"])
+def test_dissipation_has_no_bias(E, store):
+    """A state's dissipation is rounded some six times at the end (the factor of the law, mu0, the sums, the
+    division), 2^-53 each to either side, so that the mean error of eight states is below 2^-52 unless the
+    terms have one in common."""
+    err = []
+    for seed in range(8):
+        c = C.random_smooth(3, 40, 41, 42, seed=seed, T0=0.13 + 0.01 * seed, mu0=0.01 + 0.003 * seed, du=0.05,
+                            u0=(0.09, -0.07, 0.06), mu_exp=0.76)
+        g = E.Solver.from_case(c, store=store)
+        dev = g.turbulence_stats()
+        err.append(float(LD(dev["dissipation"]) / host_stats(c, 3, *g.fields())["dissipation"] - 1))
+        g.close()
+    assert abs(np.mean(err)) <= 2.0 ** -52, err
