@@ -325,8 +325,10 @@ int elbm_ensemble_bind(elbm_ensemble* e, void* pop_a, void* pop_b, void* aux, vo
     e->bound = true;
     // the one-launch-per-instance mode runs each instance as a single lattice would on this device
     const int sms = sm_count();
-    for (KParams& k : e->kp) plan_d2q9(k, sms, e->ops->fused_occupancy(k), e->ops->march_width,
-                                           e->store == ELBM_F64);
+    for (KParams& k : e->kp) {
+        k.sms = sms;
+        plan_d2q9(k, sms, e->ops->fused_occupancy(k), e->ops->march_width, e->store == ELBM_F64);
+    }
     cudaError_t c = cudaMemsetAsync(e->status(), 0, sizeof(int), e->stream);
     if (c == cudaSuccess)
         c = cudaMemcpyAsync(e->aux + e->a_params, e->kp.data(), e->kp.size() * sizeof(KParams),

@@ -43,6 +43,8 @@ inline void host_equilibria_d2q9(double rho, const double u[3], double T, double
         }
 }
 
+constexpr int kSms = 152;   // SMs of a GB300, for where the device is not asked
+
 // Validates a problem statement and fills the kernel parameters (host only, no CUDA
 // call, no allocation).  Returns ELBM_OK, ELBM_ERR_ARG or ELBM_ERR_UNSUPPORTED; *D_out is 2 or 3.
 inline int fill_kparams(const elbm_params& p, KParams& k, int* D_out) {
@@ -93,6 +95,7 @@ inline int fill_kparams(const elbm_params& p, KParams& k, int* D_out) {
     k.mu_exp = p.mu_exp;
     k.deriv = p.deriv;
     k.powlaw = p.mu_exp != 0.0;
+    k.sms = kSms;
     k.d_Cv = 1.0 / (p.gamma - 1.0);
     k.eos = p.eos == ELBM_EOS_CV_POLY;
     for (int j = 0; j < 4; ++j) {
@@ -383,10 +386,18 @@ inline bool noalloc_march_pays(const KParams& k, int D, int width, int ty) {
     return D == 3 ? axis_fill(k.nx, 32) * axis_fill(k.ny, ty) >= 0.7 : axis_fill(k.nx, width) >= 0.3;
 }
 
+// Dynamic shared memory that makes an SM hold ceil(ctas / sms) CTAs of `stat` bytes of their own and
+// no more (an SM has 228 KB, 1 KB of which goes with each CTA); none from nine on.  Figures: elbm_kernels.cu.
+constexpr int kSmShared = 228 * 1024;
+inline size_t spread_share(long long ctas, int sms, int stat) {
+    const long long k = (ctas + sms - 1) / sms;
+    return k > 8 ? 0 : (size_t)(kSmShared / (k + 1) - stat);
+}
+
 // D2Q9 small-grid kernels: a strip of kRowW nodes of a row per CTA, kRowMost strips at most
 // (one partial vector each).
 constexpr int kRowW = 30;
-constexpr int kRowMost = 8 * 152;
+constexpr int kRowMost = 8 * kSms;
 inline long long row_strips(const KParams& k) { return (long long)((k.nx + kRowW - 1) / kRowW) * k.ny; }
 
 // What the default schedule of a D2Q9 grid runs on a device of `sms` SMs, and the row segment of

@@ -785,7 +785,6 @@ __global__ void collide_kernel(const __grid_constant__ KParams p, const P* src,
 // the Q~ field.  D3Q27 128^3: 3.39 -> 1.74 ms a step, from the re-read kernel, which computes the
 // moments 2.3 times (both with the arithmetic of their time; with the sums and products in
 // integers, FixedSum and FixedProd, 1.20 now, of which the traffic takes 0.46).
-constexpr int kSms = 152;   // SMs of the device the rules here are for
 #if ELBM_ST == 0   // ST_F64
 template <bool PULL>
 __global__ void __launch_bounds__(kThreads1D)
@@ -877,7 +876,7 @@ collide64_kernel(const __grid_constant__ KParams p, const P* src, P* __restrict_
     auto out = [&](int i, R f, R g) { (dst + (size_t)i * (size_t)N)[nn] = Cd::enc(f, g); };
     // (a finite sum rho has finite terms, and T those of rho E).  With one CTA to an SM a warp has its FP64
     // pipe to itself, and the chains of integers are longer: 24^3 24.5 us a step, in integers 26.3
-    if (gridDim.x > (unsigned)kSms && rx.usable() && finite64(rho) && finite64(T)) {
+    if (gridDim.x > (unsigned)p.sms && rx.usable() && finite64(rho) && finite64(T)) {
         rx.all(in, out);
     } else {
 #pragma unroll
@@ -2714,7 +2713,7 @@ constexpr int kTY3 = ELBM_TY3;           // D3Q27 re-read and tensor-copy kernel
 #define ELBM_TYP_F32 8
 #endif
 constexpr int kTYP = (kST == ST_F32) ? ELBM_TYP_F32 : kTY3;
-constexpr int kTotalsBlocks = kTotCtas * 152;   // totals_kernel grid (grid-stride)
+constexpr int kTotalsBlocks = kTotCtas * kSms;   // totals_kernel grid (grid-stride)
 // Pipelined D3Q27 kernel per store: two plane buffers.  FP32 pairs make them 145 KB
 // (one CTA per SM, up to 255 registers; a third buffer would leave L1 almost no
 // room and measured 35 % slower); FP16/BF16 pairs are half the size (two CTAs per
@@ -2823,8 +2822,7 @@ int max_blocks(const KParams& p) {
     return (int)m;
 }
 
-// Dynamic shared memory that makes an SM hold ceil(ctas / 152) CTAs of `stat` bytes of their own
-// and no more (an SM has 228 KB, 1 KB of which goes with each CTA).  The next kernel's CTAs are set
+// Dynamic shared memory of spread_share, set as the kernel's limit.  The next kernel's CTAs are set
 // up while this one's still run: counted against the same limits, they went two and three to
 // an SM while others had none, and in FP64 such CTAs share one pipe.  us a step, zero-gradient
 // 2D grids and periodic boxes, without this limit and with it:
@@ -2836,30 +2834,31 @@ int max_blocks(const KParams& p) {
 // reuse the first-level cache that this takes away, is slower with it: FP32 1024^2 28.0 -> 35.0;
 // the tiles and the D3Q27 kernel do not change.)  The function's attribute is set to the same value
 // every time: another thread's launch, or a graph captured before, may need more than this one.
-constexpr int kSmShared = 228 * 1024;
 template <class... Args>
-size_t spread_smem(void (*kern)(Args...), long long ctas, int stat) {
-    const long long k = (ctas + kSms - 1) / kSms;
-    if (k > 8) return 0;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmShared / 2);
-    return (size_t)(kSmShared / (k + 1) - stat);
+cudaError_t spread_smem(void (*kern)(Args...), long long ctas, int sms, int stat, size_t* share) {
+    *share = spread_share(ctas, sms, stat);
+    return *share == 0 ? cudaSuccess
+                       : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmShared / 2);
 }
 
 template <bool PULL>
-void launch_two_passes(const KParams& p, const void* src, void* dst, void* qfield, double* partials, int* status,
-                       cudaStream_t s) {
+cudaError_t launch_two_passes(const KParams& p, const void* src, void* dst, void* qfield, double* partials,
+                              int* status, cudaStream_t s) {
     const unsigned nb = blocks_1d(p.N);
 #if ELBM_ST == 0
     const unsigned nc = (unsigned)((p.N + kThreads64 - 1) / kThreads64);
     constexpr int stat = 5 * kThreads1D * (int)sizeof(double);   // of the totals
-    const size_t sm = nc > 8 * kSms ? 0 : spread_smem(moments64_kernel<PULL>, nb, stat);
-    const size_t sc = spread_smem(collide64_kernel<PULL>, nc, 0);
+    size_t sm = 0, sc = 0;
+    cudaError_t e = spread_smem(collide64_kernel<PULL>, nc, p.sms, 0, &sc);
+    if (e == cudaSuccess && nc <= 8u * (unsigned)p.sms) e = spread_smem(moments64_kernel<PULL>, nb, p.sms, stat, &sm);
+    if (e != cudaSuccess) return e;
     launch_dependent(moments64_kernel<PULL>, nb, kThreads, sm, s, p, (const P*)src, (R*)qfield, (P*)dst, partials, status);
     launch_dependent(collide64_kernel<PULL>, nc, kThreads64, sc, s, p, (const P*)src, (P*)dst, (const R*)qfield);
 #else
     launch_dependent(moments_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (R*)qfield);
     launch_dependent(collide_kernel<PULL>, nb, kThreads, 0, s, p, (const P*)src, (P*)dst, (const R*)qfield, partials, status);
 #endif
+    return cudaGetLastError();
 }
 
 cudaError_t launch_init(const KParams& p, const double* rho, const double* u, const double* T, void* pop,
@@ -2873,9 +2872,8 @@ cudaError_t launch_init(const KParams& p, const double* rho, const double* u, co
     // extraction and totals read each node's own values.
     const unsigned nb = blocks_1d(p.N);
     init_kernel<<<nb, kThreads, 0, s>>>(p, rho, u, T, (P*)spare, status, 0, p.N);
-    launch_two_passes<false>(p, spare, pop, qfield, partials, status, s);
     *launches += 3;
-    return cudaGetLastError();
+    return launch_two_passes<false>(p, spare, pop, qfield, partials, status, s);
 }
 
 // f^eq, g^eq of nodes n0 .. n0 + cnt - 1 written in place into pop (fields of those nodes
@@ -2963,10 +2961,9 @@ cudaError_t launch_fields(const KParams& p, const void* pop, double* rho, double
 cudaError_t launch_twopass(const KParams& p, const void* src, void* dst, void* qfield, double* partials,
                            int* nblocks, int* status, cudaStream_t s, long long* launches) {
     const unsigned nb = blocks_1d(p.N);
-    launch_two_passes<true>(p, src, dst, qfield, partials, status, s);
     *launches += 2;
     *nblocks = (int)nb;
-    return cudaGetLastError();
+    return launch_two_passes<true>(p, src, dst, qfield, partials, status, s);
 }
 
 // A template so that the branch of the other lattice is never instantiated; CAL as in
@@ -2996,7 +2993,9 @@ cudaError_t launch_fused_cal(const KParams& p, const void* src, void* dst, doubl
             constexpr int threads = 32, stat = kRowSmem;
 #endif
             const long long strips = row_strips(p);
-            const size_t share = spread_smem(kern, strips, stat);
+            size_t share = 0;
+            const cudaError_t e = spread_smem(kern, strips, p.sms, stat, &share);
+            if (e != cudaSuccess) return e;
             return launch_dependent(kern, dim3((unsigned)strips), dim3(threads), share, s, p, (const P*)src, (P*)dst,
                                     (p.nx + kRowW - 1) / kRowW, partials, status);
         } else if (reread || p.sched == kSchedTile) {   // the tile kernel: one 32 x kTY2 tile per CTA, no march
@@ -3170,7 +3169,7 @@ cudaError_t launch_stats(const KParams& p, const void* pop, double* partials, in
                          long long* launches, bool wide) {
     const int tx = (p.nx + 31) / 32, ty = (p.ny + 7) / 8;
     const long long most = blocks_1d_of(p.N) > kTotalsBlocks ? blocks_1d_of(p.N) : kTotalsBlocks;
-    int tz = choose_segment((double)tx * ty, p.nz, 152, 2, 32);
+    int tz = choose_segment((double)tx * ty, p.nz, p.sms, 2, 32);
     while (tz < p.nz && (long long)tx * ty * ((p.nz + tz - 1) / tz) > most) tz = tz < p.nz / 2 ? 2 * tz : p.nz;
     const long long grid = (long long)tx * ty * ((p.nz + tz - 1) / tz);
     auto kern = wide ? stats_kernel<kD, true> : stats_kernel<kD, sizeof(R) == 8>;

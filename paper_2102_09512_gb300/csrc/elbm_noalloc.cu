@@ -140,11 +140,12 @@ extern "C" int elbm_step_noalloc(const elbm_params* prm, const void* src, void* 
     // No status word: nothing reads it here, and clearing it would part one step's kernels from the next's.
     int nb = 0;
     long long launches = 0;
+    int dev = -1, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return ELBM_ERR_CUDA;
+    k.sms = sms;
     if (k.N >= kNoallocFused) {
-        int dev = -1, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return ELBM_ERR_CUDA;
         const int per_sm = fused_per_sm(ops, k, D, p.store, dev);
         if (D == 2) plan_d2q9(k, sms, per_sm, ops->march_width, p.store == ELBM_F64);
         else if (p.store == ELBM_F64) k.sched = kSchedTwoPass;

@@ -35,6 +35,7 @@ struct KParams {
     int tz;                      // segment length of the fused kernels (D3Q27: z planes, D2Q9: rows)
     int sched;                   // what the default fused schedule runs: 0 the marching kernel, 1 (D2Q9) one
                                  // tile per CTA, 2 (D2Q9) one strip per CTA, 3 the two passes
+    int sms;                     // SMs of the device that the rules of the launches go by
     int aa;                      // layout of the store read by the diagnostics: 0 in place; AA single
                                  // store: 1 swapped at the node, 2 pushed to the neighbour
     float2 rest2[27];            // rest-state pair (f_i, g_i) of every direction, deviation stores

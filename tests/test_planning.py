@@ -86,6 +86,11 @@ int main(int argc, char** argv) {
     elbm::KParams k{};
     const int D = atoi(argv[1]);
     k.nx = atoi(argv[2]); k.ny = atoi(argv[3]); k.nz = atoi(argv[4]); k.tz = atoi(argv[5]);
+    if (D == -9) {   // CTAs of `stat` bytes that an SM holds with the share for k.nx CTAs on k.ny SMs (228 KB, 1 KB of it a CTA's)
+        const size_t share = elbm::spread_share(k.nx, k.ny, k.nz);
+        std::printf("%d\n", share ? (int)((228 * 1024) / (share + k.nz + 1024)) : 0);
+        return 0;
+    }
     if (D < 0) {   // plan_d2q9: store width of the strips, 64 bits, fixed faces
         k.N = (long long)k.nx * k.ny; k.tz = 32; k.has_fixed = atoi(argv[6]);
         elbm::plan_d2q9(k, 152, 4, 256, atoi(argv[5]));
@@ -136,3 +141,12 @@ def test_tiles_are_kept_for_fixed_faces(rule):
     for shape, fixed, free in (((300, 500), tile, march), ((512, 512), tile, march), ((724, 724), tile, march),
                                ((1024, 1024), march, march), ((500, 300), tile, tile)):
         assert rule(-1, *shape, 1, 0, 1) == [fixed] and rule(-1, *shape, 1, 0, 0) == [free], shape
+
+
+def test_small_launches_spread_over_the_sms_of_the_device(rule):
+    """As many CTAs to an SM as all SMs need, whatever the device's number of them."""
+    for sms in (76, 132, 148, 152, 160):
+        for ctas in (1, sms, sms + 1, 2 * sms, 5 * sms - 1, 8 * sms, 8 * sms + 1):
+            for stat in (0, 10240):
+                k = -(-ctas // sms)
+                assert rule(-9, ctas, sms, stat, 0) == [k if k <= 8 else 0], (sms, ctas, stat)
