@@ -322,7 +322,8 @@ int elbm_ensemble_set_mode(elbm_ensemble *e, int mode, int use_graph);
  * the SM count, capped by the unit count).  tile_y = 4, 8 or 16: one tile of 32 x tile_y
  * nodes per unit; tile_y = 32, 64 or 128: a strip of 128 nodes of an instance marched
  * along y over a segment of about tile_y rows: equal segments within an instance, their number
- * such that the CTAs get about the same rows (next rows prefetched into shared memory). */
+ * such that CTAs get about the same rows where as many to an SM run as it holds of the constant-gamma form
+ * without fixed faces (next rows prefetched into shared memory). */
 int elbm_ensemble_set_schedule(elbm_ensemble *e, int tile_y, int ctas_per_sm);
 int elbm_ensemble_get_schedule(const elbm_ensemble *e, int *tile_y, int *ctas_per_sm, int *grid);
 /* Autotuner: times every (work unit, CTAs per SM) the hardware can hold over

@@ -144,6 +144,9 @@ int sm_count() {
 // the order of the instances, the longest sum of the 64 lattices of sides 256 to 1024 was 8 % above
 // the mean and a few lattices left most CTAs idle: 812 -> 773 us a step (FP32), ten lattices of
 // sides 150 to 535 48.6 -> 37.0 (FP16; the tuner took tiles before), 16 of 1024^2 426 -> 403.
+// `slots` is that of the constant-gamma form without fixed faces at as many CTAs as an SM holds; other
+// forms and schedules run the same units, so that results do not depend on the CTAs, and share them less
+// evenly.
 void list_units(elbm_ensemble* e, int t, int slots) {
     const int n = e->n, rows = kTYs[t], width = rows > 16 ? kMarchW2 : kTileX;
     auto strips = [&](int k) { return (e->kp[k].nx + width - 1) / width; };
