@@ -413,8 +413,8 @@ def aa_measure(E, torch, case, steps, warmup=3):
     """The single-store (AA) layout on the bench workload: one store updated in place (half the
     population memory) by the fused march after a pass over the tiles' edges, against the
     two-pass schedule on ping-pong stores; GLUPS and the fraction of the measured HBM peak at
-    the bytes per update (AA: the populations read and written once; two-pass: read twice and
-    written once, plus the Q~ field)."""
+    the bytes per update (AA: the populations read and written once, without what the pass over
+    the edges reads, about one store more; two-pass: read twice and written once, plus the Q~ field)."""
     peak, _ = _peak_hbm()
     out = {"grid": [case.nx, case.ny, case.nz], "steps": steps, "schedule": "aa: march in place, pingpong: two-pass"}
     for store in ("f32", "f16dev"):

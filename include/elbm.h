@@ -114,7 +114,8 @@ typedef enum {
  * FP32 arithmetic, where the store is larger than some 64 MB and fills the 32 x 8 tiles well
  * enough: of the nodes at the faces of the second one's tiles), the second reads and writes
  * exactly the slots each node read, so no two threads touch one slot.  Half the population
- * memory (D3Q27 FP32 at 1024^3: 232 GB instead of 464 GB).  Periodic grids only (a
+ * memory (D3Q27 FP32 at 1024^3: 232 GB instead of 464 GB) for 1.5 times the memory traffic of the
+ * fused schedule: the first kernel reads about the whole store too.  Periodic grids only (a
  * zero-gradient or fixed face makes two nodes read one slot that one of them writes). */
 typedef enum { ELBM_LAYOUT_PINGPONG = 0, ELBM_LAYOUT_AA = 1 } elbm_layout;
 
