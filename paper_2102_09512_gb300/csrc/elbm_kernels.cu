@@ -585,6 +585,9 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
     Tri2 t[6];   // not WIDE: the sums in pairs
 #pragma unroll
     for (int k = 0; k < 6; ++k) t[k].zero();
+    // bits of all that was squared: u_x, the other velocities, theta, d u_x / d x, omega
+    unsigned any[5] = {};
+    auto seen = [&](int k, float v) { any[k] |= __float_as_uint(v); };
     const float eh = (float)p.mu_exp;
     const Df mu_exp = {eh, WIDE ? 0.f : (float)(p.mu_exp - (double)eh)};
     // log2 T0 to a multiple of 2^-8, which the law's logarithms are taken from
@@ -646,14 +649,22 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
                 }
                 Df theta = df_add(G[0][0], G[1][1]);
                 const Df wz = df_add(G[1][0], df_neg(G[0][1]));
+                seen(0, cur.u[0]);
+                seen(1, cur.u[1]);
+                seen(3, G[0][0].h);
+                seen(4, wz.h);
                 float uu_rest = 0.f;
                 Df w2 = df_sq(wz), uu = df_add(df_prod(cur.u[0], cur.u[0]), df_prod(cur.u[1], cur.u[1]), uu_rest);
                 if (DD == 3) {
                     theta = df_add(theta, G[2][2]);
-                    w2 = df_add(w2, df_sq(df_add(G[2][1], df_neg(G[1][2]))));
-                    w2 = df_add(w2, df_sq(df_add(G[0][2], df_neg(G[2][0]))));
+                    const Df wx = df_add(G[2][1], df_neg(G[1][2])), wy = df_add(G[0][2], df_neg(G[2][0]));
+                    w2 = df_add(df_add(w2, df_sq(wx)), df_sq(wy));
+                    seen(1, cur.u[2]);
+                    seen(4, wx.h);
+                    seen(4, wy.h);
                     uu = df_add(uu, df_prod(cur.u[2], cur.u[2]), uu_rest);
                 }
+                seen(2, theta.h);
                 const Df r2 = df_prod(cur.rho, cur.rho), ruu = df_scale(uu, cur.rho), th2 = df_sq(theta);
                 const Df T2 = df_prod(cur.T, cur.T), gxx = df_sq(G[0][0]), ux2 = df_prod(cur.u[0], cur.u[0]);
                 t[0].add(make_float2(cur.rho, r2.h), make_float2(0.f, r2.l));
@@ -682,6 +693,18 @@ stats_kernel(const __grid_constant__ KParams p, const P* __restrict__ pop, doubl
             if (lane == 0) part[warp][k] = acc[k];
         }
     } else {
+        // a sum of zero whose terms were not: they underflowed, FP64 wanted
+        const float nan = __int_as_float(0x7fffffff);
+        auto lost = [&](float& s, unsigned bits) {
+            if (s == 0.f && (bits & 0x7fffffffu) != 0u) s = nan;
+        };
+        lost(t[1].s.x, any[0] | any[1]);
+        lost(t[1].s.y, any[0] | any[1]);
+        lost(t[2].s.x, any[2]);
+        lost(t[3].s.y, any[3]);
+        lost(t[4].s.x, any[4]);
+        lost(t[4].s.y, any[0]);
+        if (p.powlaw) lost(t[5].s.x, any[4]);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             t[k].warp_sum();

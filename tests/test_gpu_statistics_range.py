@@ -89,3 +89,18 @@ def test_dissipation_has_no_bias(E, store):
         err.append(float(LD(dev["dissipation"]) / host_stats(c, 3, *g.fields())["dissipation"] - 1))
         g.close()
     assert abs(np.mean(err)) <= 2.0 ** -52, err
+
+
+def test_zeros_are_sums_of_zeros(E):
+    """A flow that does not depend on x has no dilatation and no d u_x / d x, one at rest no velocity: their sums
+    are exactly zero, and known to be from the one pass over the store (two launches, as for any state)."""
+    for D, shape, u0 in ((3, (33, 9, 7), 0.05), (2, (65, 17, 1), 0.05), (2, (40, 8, 1), 0.0)):
+        c = C.random_smooth(D, *shape, seed=9, mu0=0.01, mu_exp=0.76)
+        c.rho[:], c.T[:], c.u[:] = 1.0, 0.15, 0.0
+        c.u[0] = u0 * np.sin(2 * np.pi * np.arange(c.ny) / c.ny)[None, :, None]
+        g = E.Solver.from_case(c, store="f32")
+        before = g.launches
+        s = g.turbulence_stats()
+        assert g.launches - before == 2
+        assert s["theta_rms"] == s["dudx2"] == 0.0 and (s["omega_rms"] > 0) == (s["dissipation"] > 0) == (s["K"] > 0) == (u0 > 0)
+        g.close()
